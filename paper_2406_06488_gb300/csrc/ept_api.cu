@@ -935,7 +935,8 @@ int draw_mode_for(const ept_ctx *c, const Plan &P) {
 // The device work of one run, enqueued on s (and the side stream).  With `timed`,
 // events mark the phases (not used while capturing a graph).
 // The run's input copies on the copy stream (after `after`'s prior work), then ev_in:
-// the relabeling draws, which do not read the inputs, start while the copies run.
+// the relabeling draws, which do not read the inputs, start while the copies run
+// (caller relabelings in host memory are inputs: their kernel waits for ev_in too).
 ept_status enqueue_inputs(ept_ctx *c, cudaStream_t after) {
     CK(cudaEventRecord(c->ev_user, after));
     CK(cudaStreamWaitEvent(c->copy, c->ev_user, 0));
@@ -987,6 +988,8 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
     // relabelings on the side stream, beside the block build
     cudaStream_t s2 = c->side;
     CK(cudaStreamWaitEvent(s2, c->ev[1], 0));
+    if (P.user_masks && P.host_in)   // caller relabelings arrive with the inputs
+        CK(cudaStreamWaitEvent(s2, c->ev_in, with_inputs ? cudaEventWaitDefault : cudaEventWaitExternal));
     if (timed) CK(cudaEventRecord(c->ev_side[1], s2));
     launch_masks(b, c->num_sms, draw_mode_for(c, P), s2);
     CK(cudaGetLastError());
@@ -1893,6 +1896,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     CK(cudaEventRecord(c->ev[1], s));
     // relabeling draws on the side stream, beside the first pass
     CK(cudaStreamWaitEvent(c->side, c->ev[1], 0));
+    if (P.user_masks && P.host_in) CK(cudaStreamWaitEvent(c->side, c->ev_in, 0));   // they arrive with the inputs
     CK(cudaEventRecord(c->ev_side[1], c->side));
     launch_masks(bf, c->num_sms, draw_mode_for(c, P), c->side);
     CK(cudaGetLastError());
@@ -2045,6 +2049,7 @@ ept_status run_pooled(ept_ctx *c, const std::vector<TestSpec> &specs, bool on_de
     // the relabelings (Algorithm 5's SampleWithoutReplacement, the library's stream)
     // on the side stream, beside the matrix
     CK(cudaStreamWaitEvent(c->side, c->ev[1], 0));
+    if (P.user_masks && P.host_in) CK(cudaStreamWaitEvent(c->side, c->ev_in, 0));   // they arrive with the inputs
     CK(cudaEventRecord(c->ev_side[1], c->side));
     launch_masks(b, c->num_sms, draw_mode_for(c, P), c->side);
     CK(cudaGetLastError());
