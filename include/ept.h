@@ -286,12 +286,11 @@ ept_status ept_test_batch(ept_ctx *ctx, const ept_test_desc *tests, int64_t n_te
    flagged statistics, keeps the fastest for the shape (ept_result.tuning,
    .tune_candidates) and uses it from then on; every candidate computes the same
    statistics except for the accumulation order.
-   EPT_OPT_DRAW_MODE (default 0): relabeling-draw kernel, 0 = automatic (a thread
-   per column when the batch has at least 1024 columns per SM, else a warp per
-   column), 1 = a warp per column, 2 = a thread per column, 3 = groups of 32
-   columns, eight warps computing the slots' ranks and one warp the sequential
-   decisions; the draws are identical in every mode (caller relabelings always
-   take 1).
+   EPT_OPT_DRAW_MODE (default 0): relabeling-draw kernel, 0 = automatic (by columns per
+   SM: a warp per column below 36, groups of 16 columns below 400, a lane per column
+   from there), 1 = a warp per column, 2 = a lane per column, 3 = groups of 16 columns,
+   a lane per column and two words, whose words a ring of four warps takes in turn;
+   the draws are identical in every mode (caller relabelings always take 1).
    EPT_OPT_FAULT_INJECT_ALLOC (test hook, default 0): the next `value` acquisitions
    of device scratch (a run's arena, a serving batch's pool allocation) fail with
    EPT_ENOMEM on the host, without touching the GPU, to exercise error paths.

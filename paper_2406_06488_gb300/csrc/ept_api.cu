@@ -71,7 +71,7 @@ struct TestSpec {
 };
 
 // The tunable parameters of a run: contraction unit length in K-blocks, the
-// relabeling-draw kernel (0 automatic, DRAW_WARPS, DRAW_LANES, DRAW_SCAN) and the order of the
+// relabeling-draw kernel (0 automatic, DRAW_WARPS, DRAW_LANES, DRAW_RING) and the order of the
 // contraction schedule's units (0 automatic, 1 by length, 2 by first K-block, then
 // length).  Every choice computes the same statistics bit for bit except the unit
 // length, which changes the FP32 accumulation order (every length offered keeps the
@@ -608,7 +608,7 @@ struct ept_ctx {
     bool autotune = true;
     bool graphs = true;                 // replay captured graphs of repeated batches
     bool debug = false;                 // guard bands around scratch regions, plan invariants checked
-    int draw_mode = 0;                  // relabeling draws: 0 automatic, DRAW_WARPS, DRAW_LANES, DRAW_SCAN
+    int draw_mode = 0;                  // relabeling draws: 0 automatic, DRAW_WARPS, DRAW_LANES, DRAW_RING
     int64_t stream_blocks = 0;          // streaming mode: 0 automatic, k > 0 windows of <= k blocks, -1 never
     unsigned long long wait_ns = 0;     // limit of the kernels' bounded waits (0: their default, 2 s)
     int max_chunk = 32;                 // longest contraction unit the autotuner may pick
@@ -920,15 +920,11 @@ Batch device_view(ept_ctx *c, const Plan &P) {
     return b;
 }
 
-// relabeling-draw kernel of a run: the context's choice, else a thread per column
-// when there are at least 1024 columns per SM and a warp per column otherwise (the
-// producer / scanner kernel is an option: slower beside the block build, whose SMs
-// have no room left for its 32 KB of shared memory); caller relabelings always take
-// the warp kernel (it validates them)
+// relabeling-draw kernel of a run: the context's choice, else by the number of columns
+// (draw_mode_auto); caller relabelings always take the warp kernel (it validates them)
 int draw_mode_for(const ept_ctx *c, const Plan &P) {
     int mode = P.draw_mode ? P.draw_mode : c->draw_mode;
-    if (mode == 0)
-        mode = P.ncols_pad >= DRAW_LANES_MIN_COLS_PER_SM * (int64_t)c->num_sms ? DRAW_LANES : DRAW_WARPS;
+    if (mode == 0) mode = draw_mode_auto(P.ncols_pad, c->num_sms);
     return P.user_masks ? DRAW_WARPS : mode;
 }
 
@@ -1521,11 +1517,11 @@ ept_status run_tuned(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, b
         big_masks |= nw * Bp * 4 > MASKS_IN_L2_BYTES;
         user_masks |= sp.user_masks != nullptr;
     }
-    const int auto_draw = cols >= DRAW_LANES_MIN_COLS_PER_SM * (int64_t)c->num_sms ? DRAW_LANES : DRAW_WARPS;
+    const int auto_draw = draw_mode_auto(cols, c->num_sms);
     std::vector<Tuning> cand(1, def);
     if (!user_masks && c->draw_mode == 0) {
         Tuning t = def;
-        t.draw_mode = auto_draw == DRAW_LANES ? DRAW_WARPS : DRAW_LANES;
+        t.draw_mode = auto_draw == DRAW_RING ? DRAW_WARPS : DRAW_RING;   // the next best by columns
         cand.push_back(t);
     }
     {

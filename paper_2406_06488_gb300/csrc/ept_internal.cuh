@@ -368,12 +368,22 @@ void launch_median_select(const Batch &b, cudaStream_t s);   // exact radix sele
 void launch_rowsum_reduce(const Batch &b, cudaStream_t s);
 void launch_center(const Batch &b, cudaStream_t s);
 void launch_pack(const Batch &b, bool split, cudaStream_t s);   // split: FP16 hi/lo (tensor-core path)
-// draw kernels: a warp per relabeling column (caller relabelings, or few columns),
-// a thread per column (many columns: 32 warps per SM or more), or (an option) groups
-// of 32 columns whose ranks eight producer warps compute and one scanner warp turns
-// into decisions
-enum { DRAW_WARPS = 1, DRAW_LANES = 2, DRAW_SCAN = 3 };
-constexpr int64_t DRAW_LANES_MIN_COLS_PER_SM = 32 * 32;
+// draw kernels: a warp per relabeling column (caller relabelings, or few columns), a
+// lane per column with groups of 16 columns to a ring of four warps, and a lane per
+// column with every warp on its own (many columns)
+enum { DRAW_WARPS = 1, DRAW_LANES = 2, DRAW_RING = 3 };
+// The automatic choice, by relabeling columns per SM (measured, us: warps / ring / lanes):
+// n = 2000: 2500 columns 21 / 29 / 77, 5000 33 / 33 / 78, 10000 56 / 41 / 79, 40000 196 /
+// 133 / 138, 80000 383 / 242 / 223; n = 5000: 5000 69 / 72 / 182, 10000 119 / 92 / 182,
+// 20000 221 / 176 / 237.  The ring needs groups of 16 on every SM, three of them to
+// win (36 columns per SM), the lanes three CTAs of 128 columns (400).
+constexpr int64_t DRAW_RING_MIN_COLS_PER_SM = 36;
+constexpr int64_t DRAW_LANES_MIN_COLS_PER_SM = 400;
+inline int draw_mode_auto(int64_t cols, int num_sms) {
+    return cols >= DRAW_LANES_MIN_COLS_PER_SM * num_sms  ? DRAW_LANES
+           : cols >= DRAW_RING_MIN_COLS_PER_SM * num_sms ? DRAW_RING
+                                                         : DRAW_WARPS;
+}
 void launch_masks(const Batch &b, int num_sms, int mode, cudaStream_t s);   // draws or caller masks
 void launch_contract_simt(const Batch &b, cudaStream_t s);
 void launch_combine(const Batch &b, cudaStream_t s);                     // statistics, flags, counts, outputs

@@ -31,48 +31,141 @@ __device__ __forceinline__ uint32_t valid_bits(int w, int n) {
     return (1u << (n - lo)) - 1u;
 }
 
-// Philox4x32-10 of counter (c0, 0, blo, bhi) under the precomputed round keys: each
-// round multiplies counter words 0 and 2 by the two Philox multipliers (one wide
-// multiply gives both halves) and mixes the high halves with words 1 and 3 and the
-// round key.  Returns the two 64-bit output words (word 0 = (x1:x0), word 1 = (x3:x2)).
-__device__ __forceinline__ void philox_words(uint32_t c0, uint32_t blo, uint32_t bhi, const uint32_t *kx,
-                                             const uint32_t *ky, uint64_t &w0, uint64_t &w1) {
-    uint32_t x0 = c0, x1 = 0u, x2 = blo, x3 = bhi;
+// The column's part of Philox4x32-10: the round keys of the test's seed and the
+// products of the first two rounds that depend on the draw alone (counter (c0, 0, blo,
+// bhi): round 1 multiplies blo and c0, round 2 the two results, and the one that comes
+// from blo does not change from slot to slot).
+struct DrawKey {
+    uint32_t kx[10], ky[10];
+    uint32_t bhi, a1, qhi, qlo;
+    __device__ __forceinline__ DrawKey(uint64_t seed, uint64_t b) {
+        kx[0] = (uint32_t)seed;
+        ky[0] = (uint32_t)(seed >> 32);
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint64_t p0 = (uint64_t)0xD2511F53u * (uint64_t)x0;
-        const uint64_t p1 = (uint64_t)0xCD9E8D57u * (uint64_t)x2;
-        const uint32_t y0 = (uint32_t)(p1 >> 32) ^ x1 ^ kx[r];
-        const uint32_t y2 = (uint32_t)(p0 >> 32) ^ x3 ^ ky[r];
-        x1 = (uint32_t)p1;
-        x3 = (uint32_t)p0;
-        x0 = y0;
-        x2 = y2;
+        for (int r = 1; r < 10; ++r) {
+            kx[r] = kx[r - 1] + 0x9E3779B9u;
+            ky[r] = ky[r - 1] + 0xBB67AE85u;
+        }
+        bhi = (uint32_t)(b >> 32);
+        const uint64_t a = (uint64_t)0xCD9E8D57u * (uint32_t)b;
+        a1 = (uint32_t)a;
+        const uint64_t q = (uint64_t)0xD2511F53u * ((uint32_t)(a >> 32) ^ kx[0]);
+        qhi = (uint32_t)(q >> 32);
+        qlo = (uint32_t)q;
     }
-    w0 = ((uint64_t)x1 << 32) | x0;
-    w1 = ((uint64_t)x3 << 32) | x2;
+    // What rounds 1 and 2 of counter c0 give whatever the draw's low word: round 1's
+    // product of c0 and round 2's of its high half (columns of one high word share it).
+    struct Slot { uint32_t p, sh, sl; };
+    __device__ __forceinline__ Slot slot(uint32_t c0) const {
+        const uint64_t p = (uint64_t)0xD2511F53u * c0;
+        const uint64_t s = (uint64_t)0xCD9E8D57u * ((uint32_t)(p >> 32) ^ bhi ^ ky[0]);
+        return Slot{(uint32_t)p ^ ky[1], (uint32_t)(s >> 32) ^ kx[1], (uint32_t)s};
+    }
+    // rounds 3..9; the last round needs x0 and x2 (and the low halves of its products, no key)
+    __device__ __forceinline__ void nine(const Slot &s, uint32_t &x0, uint32_t &x1, uint32_t &x2, uint32_t &x3) const {
+        x0 = s.sh ^ a1;
+        x1 = s.sl;
+        x2 = s.p ^ qhi;
+        x3 = qlo;
+#pragma unroll
+        for (int r = 2; r < 9; ++r) {
+            const uint64_t p0 = (uint64_t)0xD2511F53u * x0;
+            const uint64_t p1 = (uint64_t)0xCD9E8D57u * x2;
+            x0 = (uint32_t)(p1 >> 32) ^ x1 ^ kx[r];
+            x2 = (uint32_t)(p0 >> 32) ^ x3 ^ ky[r];
+            x1 = (uint32_t)p1;
+            x3 = (uint32_t)p0;
+        }
+    }
+    // high halves of the two 64-bit words of counter c0 (the low halves of the last
+    // round's products: no wide multiplication, no key)
+    __device__ __forceinline__ void high(const Slot &s, uint32_t &h0, uint32_t &h1) const {
+        uint32_t x0, x1, x2, x3;
+        nine(s, x0, x1, x2, x3);
+        h0 = 0xCD9E8D57u * x2;
+        h1 = 0xD2511F53u * x0;
+    }
+    // the two whole words of counter c0
+    __device__ __forceinline__ void words(uint32_t c0, uint64_t &w0, uint64_t &w1) const {
+        uint32_t x0, x1, x2, x3;
+        nine(slot(c0), x0, x1, x2, x3);
+        const uint64_t p0 = (uint64_t)0xD2511F53u * x0;
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * x2;
+        w0 = (p1 << 32) | ((uint32_t)(p1 >> 32) ^ x1 ^ kx[9]);
+        w1 = (p0 << 32) | ((uint32_t)(p0 >> 32) ^ x3 ^ ky[9]);
+    }
+};
+
+// Rank of a slot, floor(u m / 2^64) with m = n - t slots left, from the high half uh of
+// u alone: v = uh m; u m = v 2^32 + ul m, so the rank is v >> 32, plus one when the low
+// half's ul m / 2^32 < m carries out of v's low word.  That takes a low word above
+// 2^32 - m, which one slot in 2^32 / m has: `frac` collects the largest low word, and a
+// group of slots that reaches 2^32 - n is decided again from whole words
+// (DRAW_SLOW_FRAC).  Past the end (m <= 0) the rank is larger than any count.
+constexpr uint32_t NO_RANK = 0x7FFFFFFFu;
+__device__ __forceinline__ uint32_t rank_high(uint32_t uh, uint32_t m, uint32_t &frac) {
+    const uint64_t v = (uint64_t)uh * m;
+    frac = max(frac, (uint32_t)v);
+    return (uint32_t)(v >> 32);
+}
+__device__ __forceinline__ bool draw_slow(uint32_t frac, int n) { return frac >= 0u - (uint32_t)n; }
+
+// rank of slot t from whole words
+__device__ __forceinline__ uint32_t rank_exact(uint64_t u, int t, int n) {
+    return t < n ? (uint32_t)mulhi_64x32(u, (uint32_t)(n - t)) : NO_RANK;
 }
 
-// Decisions of one 64-slot window: lane l holds the ranks r0 (slot base+l) and r1
-// (slot base+32+l); returns the two ballots (kept slots) and lowers `need`.  The
-// sequential dependence through `need` is resolved by a fixed-point iteration over
-// ballots: with every earlier decision known a slot's decision is determined, so
-// iterating "decide from the previous guesses" reaches the unique sequential
-// solution in at most 65 rounds (almost always 1 or 2).
-__device__ __forceinline__ void decide_window(int r0, int r1, unsigned lt, int &need, unsigned &m0, unsigned &m1) {
-    m0 = __ballot_sync(0xFFFFFFFFu, r0 < need);
-    m1 = __ballot_sync(0xFFFFFFFFu, r1 < need);
+// Word w of a column decided slot by slot from whole words (the rare case above).
+__device__ __forceinline__ uint32_t draw_word_exact(const DrawKey &key, int n, int w, int need) {
+    uint32_t bits = 0;
+#pragma unroll 1
+    for (int j = 0; j < 16; ++j) {
+        const int t = 32 * w + 2 * j;
+        uint64_t u0, u1;
+        key.words((uint32_t)(t >> 1), u0, u1);
+        if ((int)rank_exact(u0, t, n) < need) { bits |= 1u << (2 * j); --need; }
+        if ((int)rank_exact(u1, t + 1, n) < need) { bits |= 2u << (2 * j); --need; }
+    }
+    return bits;
+}
+
+// Decisions of one 64-slot window: lane l holds the ranks e and o of its slots 2 l and
+// 2 l + 1; returns the ballots of the kept even and odd slots and lowers `need`.  A slot is kept
+// iff its rank is below need less the slots kept before it in the window; those are at
+// most all `cnt` ranks below need, so when the ballots against need - cnt are the same
+// they are the decisions (about six windows in seven at n = 5000).  Otherwise the
+// sequential dependence is resolved by a fixed-point iteration over ballots: with
+// every earlier decision known a slot's decision is determined, so iterating "decide
+// from the previous guesses" reaches the unique sequential solution in at most 65
+// rounds (almost always 2).
+__device__ __forceinline__ void decide_window(uint32_t e, uint32_t o, unsigned lt, int &need, unsigned &me,
+                                              unsigned &mo) {
+    me = __ballot_sync(0xFFFFFFFFu, (int)e < need);
+    mo = __ballot_sync(0xFFFFFFFFu, (int)o < need);
+    const int low = need - (__popc(me) + __popc(mo));
+    if (__ballot_sync(0xFFFFFFFFu, (int)e < low) == me && __ballot_sync(0xFFFFFFFFu, (int)o < low) == mo) {
+        need = low;
+        return;
+    }
     for (int it = 0; it < 70; ++it) {
-        const int before0 = __popc(m0 & lt);
-        const int before1 = __popc(m0) + __popc(m1 & lt);
-        const unsigned nm0 = __ballot_sync(0xFFFFFFFFu, r0 < need - before0);
-        const unsigned nm1 = __ballot_sync(0xFFFFFFFFu, r1 < need - before1);
-        const bool same = (nm0 == m0) && (nm1 == m1);
-        m0 = nm0;
-        m1 = nm1;
+        const int be = __popc(me & lt) + __popc(mo & lt);             // kept before slot 2 l
+        const int bo = be + (int)((me >> (threadIdx.x & 31)) & 1u);   // and before slot 2 l + 1
+        const unsigned ne = __ballot_sync(0xFFFFFFFFu, (int)e < need - be);
+        const unsigned no = __ballot_sync(0xFFFFFFFFu, (int)o < need - bo);
+        const bool same = (ne == me) && (no == mo);
+        me = ne;
+        mo = no;
         if (same) break;
     }
-    need -= __popc(m0) + __popc(m1);
+    need -= __popc(me) + __popc(mo);
+}
+
+// the 16 low bits of v at the even positions
+__device__ __forceinline__ uint32_t spread16(uint32_t v) {
+    v = (v | (v << 8)) & 0x00FF00FFu;
+    v = (v | (v << 4)) & 0x0F0F0F0Fu;
+    v = (v | (v << 2)) & 0x33333333u;
+    return (v | (v << 1)) & 0x55555555u;
 }
 
 // One warp writes one relabeling column (words w = 0..nw-1 at col[w * stride]; nw is
@@ -80,12 +173,15 @@ __device__ __forceinline__ void decide_window(int r0, int r1, unsigned lt, int &
 // selection sampling (Algorithm S) over the n pooled slots, slot t kept iff
 // floor(u_t (n - t) / 2^64) < need, with u_t the 64-bit word (t mod 2) of
 // Philox4x32-10(counter = (t/2, 0, b lo, b hi), key = (seed lo, seed hi)).  The warp
-// takes 128 consecutive slots per step: lane l runs the Philox calls of slots
-// base+2l, base+2l+1 and base+64+2l, base+64+2l+1 (two independent chains, so that
-// few warps per SM keep the integer pipes busy) and forms their floor(u (n - t) /
-// 2^64) values; shuffles then place slot base+l on lane l (first word) and slot
-// base+32+l on lane l (second word) of each 64-slot window, so one ballot is one
-// output word.  comp: store the complement (the y* members).
+// takes 256 consecutive slots per step, in four windows of 64: lane l runs the Philox
+// call of slots 2 l and 2 l + 1 of each window (four independent chains), ballots
+// decide the even and the odd slots, and the first eight lanes interleave them into
+// the step's eight output words.  comp: store the complement (the y* members).
+// Bound by the multiplier (a wide multiplication holds its pipe for four cycles, busy 62 %)
+// and the logic pipe (53 %): per two slots 16 wide multiplications and 17 three-input
+// XORs, with ranks and decisions on top.  n = 5000, 10^4 columns: 119 us (137 us with
+// the last round's wide products, ranks from whole words and shuffled slots);
+// 5000 columns 69 us (79).
 __device__ void draw_column(uint64_t seed, int nx, int n, int64_t b, int nw, bool comp, uint32_t *col,
                             int64_t stride) {
     const int lane = threadIdx.x & 31;
@@ -96,50 +192,49 @@ __device__ void draw_column(uint64_t seed, int nx, int n, int64_t b, int nw, boo
         }
         return;
     }
-    uint32_t kx[10], ky[10];
-    kx[0] = (uint32_t)seed;
-    ky[0] = (uint32_t)(seed >> 32);
-#pragma unroll
-    for (int r = 1; r < 10; ++r) {
-        kx[r] = kx[r - 1] + 0x9E3779B9u;
-        ky[r] = ky[r - 1] + 0xBB67AE85u;
-    }
-    const uint32_t blo = (uint32_t)(uint64_t)b, bhi = (uint32_t)((uint64_t)b >> 32);
+    const DrawKey key(seed, (uint64_t)b);
     const unsigned lt = (1u << lane) - 1u;
-    const int src = lane >> 1;
-    const bool odd = lane & 1;
     int need = nx;
-    for (int base = 0; base < nw * 32; base += 128) {
-        // ranks of this lane's four slots ("never kept" past the end or once need is 0)
-        uint32_t ra = 0xFFFFFFFFu, rb = 0xFFFFFFFFu, rc = 0xFFFFFFFFu, rd = 0xFFFFFFFFu;
-        if (need > 0) {
-            const int tp = base + 2 * lane, tq = tp + 64;
-            uint64_t u0, u1, u2, u3;
-            philox_words((uint32_t)(tp >> 1), blo, bhi, kx, ky, u0, u1);
-            philox_words((uint32_t)(tq >> 1), blo, bhi, kx, ky, u2, u3);
-            if (tp < n) ra = (uint32_t)mulhi_64x32(u0, (uint32_t)(n - tp));
-            if (tp + 1 < n) rb = (uint32_t)mulhi_64x32(u1, (uint32_t)(n - tp - 1));
-            if (tq < n) rc = (uint32_t)mulhi_64x32(u2, (uint32_t)(n - tq));
-            if (tq + 1 < n) rd = (uint32_t)mulhi_64x32(u3, (uint32_t)(n - tq - 1));
+    for (int base = 0; base < nw * 32; base += 256) {
+        unsigned me[4] = {0u, 0u, 0u, 0u}, mo[4] = {0u, 0u, 0u, 0u};
+        if (need > 0 && base < n) {
+            uint32_t e[4], o[4], frac = 0;
+            const int left = n - base - 2 * lane;   // slots left at this lane's first slot
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t h0, h1;
+                key.high(key.slot((uint32_t)((base >> 1) + 32 * q + lane)), h0, h1);
+                const int m = left - 64 * q;
+                e[q] = rank_high(h0, (uint32_t)m, frac);
+                o[q] = rank_high(h1, (uint32_t)(m - 1), frac);
+            }
+            if (base + 256 > n) {   // the last step: slots past the end are never kept
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (left - 64 * q <= 0) e[q] = NO_RANK;
+                    if (left - 64 * q <= 1) o[q] = NO_RANK;
+                }
+            }
+            if (__any_sync(0xFFFFFFFFu, draw_slow(frac, n))) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int t = base + 64 * q + 2 * lane;
+                    uint64_t u0, u1;
+                    key.words((uint32_t)(t >> 1), u0, u1);
+                    e[q] = rank_exact(u0, t, n);
+                    o[q] = rank_exact(u1, t + 1, n);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) decide_window(e[q], o[q], lt, need, me[q], mo[q]);
         }
-        unsigned m[4];
-        {
-            const uint32_t a0 = __shfl_sync(0xFFFFFFFFu, ra, src), b0 = __shfl_sync(0xFFFFFFFFu, rb, src);
-            const uint32_t a1 = __shfl_sync(0xFFFFFFFFu, ra, src + 16), b1 = __shfl_sync(0xFFFFFFFFu, rb, src + 16);
-            const int r0 = (int)min(odd ? b0 : a0, 0x7FFFFFFFu);
-            const int r1 = (int)min(odd ? b1 : a1, 0x7FFFFFFFu);
-            decide_window(r0, r1, lt, need, m[0], m[1]);
-        }
-        {
-            const uint32_t a0 = __shfl_sync(0xFFFFFFFFu, rc, src), b0 = __shfl_sync(0xFFFFFFFFu, rd, src);
-            const uint32_t a1 = __shfl_sync(0xFFFFFFFFu, rc, src + 16), b1 = __shfl_sync(0xFFFFFFFFu, rd, src + 16);
-            const int r0 = (int)min(odd ? b0 : a0, 0x7FFFFFFFu);
-            const int r1 = (int)min(odd ? b1 : a1, 0x7FFFFFFFu);
-            decide_window(r0, r1, lt, need, m[2], m[3]);
-        }
-        if (lane < 4) {
+        // word 2 q + h of the step: lanes 16 h .. 16 h + 15 of window q
+        const int q = (lane >> 1) & 3, sh = (lane & 1) * 16;
+        const uint32_t ve = q == 0 ? me[0] : q == 1 ? me[1] : q == 2 ? me[2] : me[3];
+        const uint32_t vo = q == 0 ? mo[0] : q == 1 ? mo[1] : q == 2 ? mo[2] : mo[3];
+        uint32_t v = spread16((ve >> sh) & 0xFFFFu) | (spread16((vo >> sh) & 0xFFFFu) << 1);
+        if (lane < 8) {
             const int w = (base >> 5) + lane;
-            uint32_t v = lane == 0 ? m[0] : lane == 1 ? m[1] : lane == 2 ? m[2] : m[3];
             if (comp) v = ~v & valid_bits(w, n);
             col[(int64_t)w * stride] = v;
         }
@@ -189,165 +284,158 @@ __global__ void __launch_bounds__(128) k_masks(const Batch bt) {
     }
 }
 
-// One thread per relabeling column (used when the batch has enough columns to fill
-// the GPU this way, and no caller relabelings): the thread runs Algorithm S over
-// its column's slots one at a time, from the same Philox words as draw_column, so
-// the two kernels write identical bits.  Without the warp's ballots, shuffles and
-// fixed-point rounds a slot costs about half the instructions, and the 32 lanes of
-// a warp write 32 neighbouring columns of a word with one coalesced store.
-__global__ void __launch_bounds__(256) k_masks_lanes(const Batch bt) {
-    const int64_t gc = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gc >= bt.ncols_total) return;
-    const int t = find_test(bt.pre.cols, bt.n_tests, gc);
-    const TestDesc &d = bt.desc[t];
-    const int64_t c = gc - bt.pre.cols[t];
-    const int n = (int)d.n, nw = (int)d.nw, nx = (int)d.nx;
-    const int64_t Bp = d.Bp;
-    const bool comp = d.comp != 0;
-    uint32_t *col = bt.maskT + d.mask0 + c;
-    if (c >= d.ncols) {
-        for (int w = 0; w < nw; ++w) col[(int64_t)w * Bp] = 0u;
-        return;
-    }
-    if (c == 0) {
-        for (int w = 0; w < nw; ++w) {
-            const uint32_t v = valid_bits(w, nx);
-            col[(int64_t)w * Bp] = comp ? (~v & valid_bits(w, n)) : v;
-        }
-        return;
-    }
-    const uint64_t seed = d.seed;
-    uint32_t kx[10], ky[10];
-    kx[0] = (uint32_t)seed;
-    ky[0] = (uint32_t)(seed >> 32);
-#pragma unroll
-    for (int r = 1; r < 10; ++r) {
-        kx[r] = kx[r - 1] + 0x9E3779B9u;
-        ky[r] = ky[r - 1] + 0xBB67AE85u;
-    }
-    const uint64_t bdraw = (uint64_t)(d.b0 + c - 1);   // column c >= 1 holds draw b0 + c - 1
-    const uint32_t blo = (uint32_t)bdraw, bhi = (uint32_t)(bdraw >> 32);
-    int need = nx;
-    for (int w = 0; w < nw; ++w) {
-        uint32_t bits = 0;
-        const int t0 = w * 32;
-        if (need > 0 && t0 < n) {
-            // two Philox calls per step (slots tp .. tp + 3): independent chains for the
-            // scheduler to interleave
-#pragma unroll 2
-            for (int j = 0; j < 16; j += 2) {
-                const int tp = t0 + 2 * j;
-                uint64_t u0, u1, u2, u3;
-                philox_words((uint32_t)(tp >> 1), blo, bhi, kx, ky, u0, u1);
-                philox_words((uint32_t)(tp >> 1) + 1u, blo, bhi, kx, ky, u2, u3);
-                const uint64_t uu[4] = {u0, u1, u2, u3};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int ts = tp + q;
-                    if (ts < n && (int)mulhi_64x32(uu[q], (uint32_t)(n - ts)) < need) {
-                        bits |= 1u << (2 * j + q);
-                        --need;
-                    }
-                }
-            }
-        }
-        col[(int64_t)w * Bp] = comp ? (~bits & valid_bits(w, n)) : bits;
-    }
+// The float rank of a slot: X m with X = floor(uh / 2^9) / 2^23 (a funnel shift puts the
+// 23 bits behind the exponent of 1.0), rounded once.  The slot's u m / 2^64 lies within
+// m 2^-23 above X m, and the rounding moves it by at most m 2^-24, so it is below the
+// integer `need` exactly when the float is, unless the two are closer than n 2^-22: one
+// slot in 2^21, whose word is decided again from whole words.  Costs a shift and an FMA
+// where the integer rank takes another wide multiplication.
+__device__ __forceinline__ float rank_float(uint32_t uh, float m) {
+    return fmaf(__uint_as_float(__funnelshift_r(uh, 0x7Fu, 9)), m, -m);
 }
 
-// Relabeling columns in groups of 32 per CTA, with Algorithm S split into its two
-// parts: a slot's rank r_t = floor(u_t (n - t) / 2^64) depends only on the stream
-// (the same Philox words as draw_column), and only the decisions "keep slot t iff
-// r_t < need" depend on each other.  Eight producer warps compute the ranks of the
-// next 128 slots of all 32 columns into shared memory (two buffers) while one
-// scanner warp, a lane per column, runs the sequential decisions over the previous
-// 128 (a compare and a subtraction per slot) and writes each 32-slot word, the 32
-// lanes storing neighbouring columns of a word together.  No ballots, shuffles or
-// fixed-point rounds: about half the instructions per slot of the warp kernel, with
-// the columns' Philox work spread over eight times as many threads as the thread
-// kernel.  The identity (column 0) and padding columns are written by the scanner
-// lane; caller relabelings take the warp kernel.  A group never straddles two tests
-// (every test's column count Bp is a multiple of 32).
-constexpr int SCAN_SLOTS = 128;                    // slots per chunk
-constexpr int SCAN_PRODUCERS = 256;                // eight producer warps
-constexpr int SCAN_THREADS = SCAN_PRODUCERS + 32;  // and the scanner warp
-static_assert(COL_PAD % 32 == 0, "column groups of 32 stay inside one test");
+// The sequential decisions of one word: slot e kept iff r[e] < need.  The sign of
+// r - need is shifted into the word and taken off need (-2^40 (r - need) saturated to
+// [0, 1] is 1 when it is negative: a non-zero difference is at least 2^-24, and r = need
+// = 0 gives 0).  near: the smallest |r - need|.  (Deciding against need - r less the
+// count so far, an eight-cycle chain instead of twelve, measured 5 % faster with few
+// columns and 4 % slower with many.)
+__device__ __forceinline__ uint32_t word_decide(const float (&r)[32], float &need, float &near) {
+    uint32_t bits = 0;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+        const float d = r[e] - need;
+        bits = __funnelshift_l(__float_as_uint(d), bits, 1);
+        near = fminf(near, fabsf(d));
+        need -= __saturatef(d * -1099511627776.f);
+    }
+    return __brev(bits);
+}
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_masks_scan(const Batch bt) {
-    __shared__ uint32_t rank[2][SCAN_SLOTS][32];   // [buffer][slot in chunk][column in group]
-    const int64_t gc0 = (int64_t)blockIdx.x * 32;  // first batch column of the group
-    if (gc0 >= bt.ncols_total) return;             // uniform over the CTA, before any barrier
+// Relabeling columns, a lane per column, words taken in turn by a ring of warps.  A slot's
+// rank depends only on the stream (the same Philox words as draw_column), and only
+// the decisions "keep slot t iff its rank is below need" depend on each other: a
+// warp computes the ranks of its words into registers while the other warps of its
+// group do theirs, then waits for its turn at `need` (one named barrier between
+// neighbours of the ring), decides its slots, passes `need` on and stores the words.
+// HALVES = 2: a group is 16 columns and a turn two words, the first on lanes 0..15 and
+// the second on lanes 16..31 (decided after the first; the ranks of both are computed
+// at once): twice as many groups, whose number per SM then rounds up to less.
+// WARPS = 1, HALVES = 1: 32 columns to a warp and no turns to wait for.  Both write the
+// bits of draw_column; caller relabelings take the warp kernel.  A CTA's columns never
+// straddle two tests (every test's column count is a multiple of 256).
+// Bound by the multiplier's pipe: 14 wide multiplications per two slots are left (what
+// rounds 1 and 2 owe to the slot alone is computed once per warp and read from shared
+// memory, the last round needs low halves only), 42 cycles per slot and warp, that
+// pipe busy 78 %.  n = 1000, 1.24e6 columns (WARPS = 1): 1.33 ms, 2.1 ms before with whole
+// words; n = 5000, 10^4 columns (WARPS = 4): 92 us, against 119 us for the warp kernel and 182 us with one
+// warp per group.
+// Turns of a ring of four warps: warp k waits at named barrier 1 + k for the warp before it
+// (immediate numbers, so that the CTA reserves five barriers and not all sixteen).
+__device__ __forceinline__ void ring_wait(int k) {
+    if (k == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+    else if (k == 1) asm volatile("bar.sync 2, 64;" ::: "memory");
+    else if (k == 2) asm volatile("bar.sync 3, 64;" ::: "memory");
+    else asm volatile("bar.sync 4, 64;" ::: "memory");
+}
+__device__ __forceinline__ void ring_pass(int k) {
+    if (k == 0) asm volatile("bar.arrive 1, 64;" ::: "memory");
+    else if (k == 1) asm volatile("bar.arrive 2, 64;" ::: "memory");
+    else if (k == 2) asm volatile("bar.arrive 3, 64;" ::: "memory");
+    else asm volatile("bar.arrive 4, 64;" ::: "memory");
+}
+
+template <int WARPS, int HALVES>
+__global__ void __launch_bounds__(128, 5) k_masks_group(const Batch bt) {
+    static_assert((WARPS == 1 && HALVES == 1) || (WARPS == 4 && HALVES == 2), "a ring passes one turn per step");
+    constexpr int COLS = 32 / HALVES, GROUPS = 4 / WARPS;   // columns of a group, groups of a CTA
+    __shared__ float need_s[COLS];                          // WARPS > 1: the group's counts, handed from warp to warp
+    __shared__ uint4 slot_s[4][34];                         // per warp: the step's 32 slot pairs (halves 17 apart)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ring = warp % WARPS, half = HALVES == 2 ? lane >> 4 : 0;
+    const int64_t gc0 = (int64_t)blockIdx.x * (GROUPS * COLS);   // the CTA's first batch column
+    if (gc0 >= bt.ncols_total) return;                           // uniform over the CTA, before any barrier
     const int t = find_test(bt.pre.cols, bt.n_tests, gc0);
     const TestDesc &d = bt.desc[t];
-    const int64_t c0 = gc0 - bt.pre.cols[t];       // first column of the group within the test
+    const int64_t c0 = gc0 - bt.pre.cols[t] + (warp / WARPS) * COLS;   // the group's first column
+    const int64_t c = c0 + (lane & (COLS - 1));                        // this lane's column
     const int n = (int)d.n, nw = (int)d.nw;
-    const int nchunks = nw * 32 / SCAN_SLOTS;      // nw is a multiple of 8
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t c = c0 + lane;                   // this lane's column (producers and scanner)
-
-    // producer state: round keys and the draw of this thread's column
-    uint32_t kx[10], ky[10];
-    kx[0] = (uint32_t)d.seed;
-    ky[0] = (uint32_t)(d.seed >> 32);
-#pragma unroll
-    for (int r = 1; r < 10; ++r) {
-        kx[r] = kx[r - 1] + 0x9E3779B9u;
-        ky[r] = ky[r - 1] + 0xBB67AE85u;
-    }
-    const uint64_t bdraw = (uint64_t)(d.b0 + c - 1);   // column c >= 1 holds draw b0 + c - 1
-    const uint32_t blo = (uint32_t)bdraw, bhi = (uint32_t)(bdraw >> 32);
-    const bool drawn = c >= 1 && c < d.ncols;
-    // ranks of chunk k into buffer buf: this thread's column, slot pairs warp + 8 i
-    auto produce = [&](int k, int buf) {
-        if (!drawn) return;
-#pragma unroll 2
-        for (int i = 0; i < SCAN_SLOTS / 2 / 8; ++i) {
-            const int jp = warp + 8 * i;                 // slot pair within the chunk
-            const int ts = k * SCAN_SLOTS + 2 * jp;      // its first slot
-            uint64_t u0, u1;
-            philox_words((uint32_t)(ts >> 1), blo, bhi, kx, ky, u0, u1);
-            rank[buf][2 * jp][lane] = ts < n ? (uint32_t)mulhi_64x32(u0, (uint32_t)(n - ts)) : 0xFFFFFFFFu;
-            rank[buf][2 * jp + 1][lane] =
-                ts + 1 < n ? (uint32_t)mulhi_64x32(u1, (uint32_t)(n - ts - 1)) : 0xFFFFFFFFu;
-        }
-    };
-
-    // scanner state
-    uint32_t *col = bt.maskT + d.mask0 + c;
     const int64_t Bp = d.Bp;
     const bool comp = d.comp != 0;
-    uint32_t need = (uint32_t)d.nx;
-
-    if (warp < 8) produce(0, 0);
-    __syncthreads();
-    for (int k = 0; k < nchunks; ++k) {
-        if (warp == 8) {
-            const int buf = k & 1;
-#pragma unroll 1
-            for (int q = 0; q < SCAN_SLOTS / 32; ++q) {
-                const int w = k * (SCAN_SLOTS / 32) + q;   // output word
-                uint32_t bits;
-                if (drawn) {
-                    uint32_t r[32];
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) r[e] = rank[buf][q * 32 + e][lane];
-                    bits = 0;
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const uint32_t keep = r[e] < need ? 1u : 0u;
-                        bits |= keep << e;
-                        need -= keep;
-                    }
-                } else {
-                    bits = (c == 0) ? valid_bits(w, (int)d.nx) : 0u;   // identity, or padding
-                }
-                if (c < d.ncols) bits = comp ? (~bits & valid_bits(w, n)) : bits;
-                col[(int64_t)w * Bp] = bits;
-            }
-        } else if (k + 1 < nchunks) {
-            produce(k + 1, (k + 1) & 1);
+    const uint64_t draw = (uint64_t)(d.b0 + c - 1);   // column c >= 1 holds draw b0 + c - 1
+    const bool any = c0 < d.ncols;                    // a group past the test's columns has nothing to draw
+    // columns of one high word share the slot table; a group that straddles two is decided from whole words
+    const bool split = (uint32_t)((uint64_t)(d.b0 + c0 - 1) >> 32) != (uint32_t)((uint64_t)(d.b0 + c0 + COLS - 2) >> 32);
+    uint32_t *col = bt.maskT + d.mask0 + c;
+    const DrawKey key(d.seed, draw);
+    const float limit = split ? 3.0e38f : (float)n * 2.384185791015625e-7f;   // n 2^-22
+    uint4 *slots = slot_s[warp];
+    float need = (float)d.nx;
+    for (int w0 = 2 * ring; w0 < nw; w0 += 2 * WARPS) {   // nw is a multiple of 8
+        const bool some = any && 32 * w0 < n;             // uniform over the group
+        if (some) {
+            __syncwarp();
+            const DrawKey::Slot s = key.slot((uint32_t)(16 * w0 + lane));
+            slots[lane + (lane >> 4)] = make_uint4(s.p, s.sh, s.sl, 0u);
+            __syncwarp();
         }
-        __syncthreads();
+#pragma unroll 1
+        for (int k = 0; k < 2; k += HALVES) {
+            const int w = w0 + k + half;
+            const int left = n - 32 * w;
+            float r[32], near = 3.0e38f;
+            if (some) {
+                const float m = (float)left;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const uint4 sv = slots[17 * (k + half) + j];
+                    uint32_t h0, h1;
+                    key.high(DrawKey::Slot{sv.x, sv.y, sv.z}, h0, h1);
+                    r[2 * j] = rank_float(h0, m - (float)(2 * j));
+                    r[2 * j + 1] = rank_float(h1, m - (float)(2 * j + 1));
+                }
+                if (left < 32) {   // slots past the end are never kept
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        if (e >= left) r[e] = 1.0e30f;
+                }
+            }
+            if (WARPS > 1 && w0 > 0) {
+                __syncwarp();
+                ring_wait(ring);
+                need = need_s[lane & (COLS - 1)];
+            }
+            uint32_t bits = 0;
+            if (some) {
+                float before = need;
+                bits = word_decide(r, need, near);
+                if (HALVES == 2) {
+                    if (half == 0 && near <= limit) {
+                        bits = draw_word_exact(key, n, w, (int)before);
+                        need = before - (float)__popc(bits);
+                    }
+                    // the second word starts where the first ended
+                    before = __shfl_sync(0xFFFFFFFFu, need, lane & 15);
+                    if (half == 1) {
+                        need = before;
+                        near = 3.0e38f;
+                        bits = word_decide(r, need, near);
+                    }
+                }
+                if (half == HALVES - 1 && near <= limit) {
+                    bits = draw_word_exact(key, n, w, (int)before);
+                    need = before - (float)__popc(bits);
+                }
+            }
+            if (WARPS > 1 && w0 + 2 < nw) {
+                if (half == HALVES - 1) need_s[lane & (COLS - 1)] = need;
+                __syncwarp();
+                ring_pass((ring + 1) & 3);
+            }
+            if (c == 0) bits = valid_bits(w, (int)d.nx);   // the identity
+            if (comp) bits = ~bits & valid_bits(w, n);
+            col[(int64_t)w * Bp] = c < d.ncols ? bits : 0u;
+        }
     }
 }
 
@@ -365,14 +453,12 @@ static int mask_blocks_per_sm() {
 
 void launch_masks(const Batch &b, int num_sms, int mode, cudaStream_t s) {
     if (b.ncols_total <= 0) return;
-    if (mode == DRAW_SCAN) {
-        k_masks_scan<<<(unsigned)((b.ncols_total + 31) / 32), SCAN_THREADS, 0, s>>>(b);
+    if (mode == DRAW_RING) {
+        k_masks_group<4, 2><<<(unsigned)(b.ncols_total / 16), 128, 0, s>>>(b);
         return;
     }
     if (mode == DRAW_LANES) {
-        // few columns: small blocks, so that they spread over the SMs beside the build
-        const int threads = (b.ncols_total >= 1024 * (int64_t)(num_sms > 0 ? num_sms : 1)) ? 256 : 64;
-        k_masks_lanes<<<(unsigned)((b.ncols_total + threads - 1) / threads), threads, 0, s>>>(b);
+        k_masks_group<1, 1><<<(unsigned)(b.ncols_total / 128), 128, 0, s>>>(b);
         return;
     }
     int64_t blocks = (b.ncols_total + 3) / 4;
