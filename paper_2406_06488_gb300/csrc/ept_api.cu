@@ -1486,6 +1486,8 @@ bool worth_tuning(const std::vector<TestSpec> &specs) {
     return n * n * (double)specs[0].B >= 2.5e10;
 }
 
+constexpr float TUNE_MARGIN = 0.97f;
+
 // Parameters for this batch shape (tensor-core path): from the cache, or (first call
 // of the shape) by timing whole device runs with each candidate on this very batch:
 // the defaults; the other relabeling-draw kernel; the other unit order; units of 4
@@ -1543,16 +1545,26 @@ ept_status run_tuned(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, b
             t.kernel = k;
             cand.push_back(t);
         }
-    Tuning best = def;
-    float best_ms = 1e30f;
+    // A candidate with another rounding order (unit length, contraction kernel) has to be
+    // 3 % faster than the best with the default's order, and again when both are timed a
+    // second time (the first candidate's run is a cold one): runs whose times differ by
+    // noise alone then return the same bits.
+    auto same_order = [&def](const Tuning &tn) { return tn.chunk_kb == def.chunk_kb && tn.kernel == def.kernel; };
+    Tuning best = def, other = def;
+    float best_ms = 1e30f, other_ms = 1e30f;
     for (const Tuning &tn : cand) {
         float ms = 0.f;
         ept_status st = run_once(c, specs, prec, on_device, tn, false, out, stream, &ms);
         if (st != EPT_OK) return st;
-        if (ms < best_ms) {
-            best_ms = ms;
-            best = tn;
-        }
+        if (same_order(tn) ? ms < best_ms : ms < other_ms) (same_order(tn) ? best : other) = tn;
+        (same_order(tn) ? best_ms : other_ms) = std::min(ms, same_order(tn) ? best_ms : other_ms);
+    }
+    if (other_ms < TUNE_MARGIN * best_ms) {
+        float ms = 0.f, ms2 = 0.f;
+        ept_status st = run_once(c, specs, prec, on_device, best, false, out, stream, &ms);
+        if (st == EPT_OK) st = run_once(c, specs, prec, on_device, other, false, out, stream, &ms2);
+        if (st != EPT_OK) return st;
+        if (std::min(ms2, other_ms) < TUNE_MARGIN * std::min(ms, best_ms)) best = other;
     }
     c->tuned[key] = best;
     save_tune_file(c);
