@@ -995,9 +995,9 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
     CK(cudaStreamWaitEvent(s, c->ev_in, with_inputs ? cudaEventWaitDefault : cudaEventWaitExternal));
     if (tc) {
         launch_split_rows(b, s);
-        alignas(64) CUtensorMap tm[4];
+        alignas(64) CUtensorMap tm[5];
         char emsg[160];
-        if (!encode_rows_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, emsg, sizeof(emsg)))
+        if (!encode_build_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, b.D, P.nblk, emsg, sizeof(emsg)))
             return fail(EPT_ECUDA, "%s", emsg);
         CK(launch_build_tc(b, tm, c->num_sms, s));
     } else {
@@ -1912,10 +1912,10 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     CK(cudaStreamWaitEvent(s, c->ev_in, 0));
     launch_split_rows(bf, s);
     CK(cudaGetLastError());
-    alignas(64) CUtensorMap tm[4];
+    alignas(64) CUtensorMap tm[5];
     alignas(64) CUtensorMap th, tl;
     char emsg[160];
-    if (!encode_rows_tmaps(tm, bf.Zh, bf.Zl, P.nrows, P.p_stride, emsg, sizeof(emsg)))
+    if (!encode_build_tmaps(tm, bf.Zh, bf.Zl, P.nrows, P.p_stride, bf.D, P.win_blk, emsg, sizeof(emsg)))
         return fail(EPT_ECUDA, "%s", emsg);
     if (!encode_block_tmaps(&th, &tl, bf.Chi, bf.Clo, P.win_blk, bf.c_stride, emsg, sizeof(emsg)))
         return fail(EPT_ECUDA, "%s", emsg);
@@ -2746,9 +2746,9 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     CK(cudaMemsetAsync(b.ctr, 0, sizeof(Counters), s));
     if (prec == EPT_PREC_SPLIT_BF16) {
         launch_split_rows(b, s);
-        alignas(64) CUtensorMap tm[4];
+        alignas(64) CUtensorMap tm[5];
         char emsg[160];
-        if (!encode_rows_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, emsg, sizeof(emsg))) return fail(EPT_ECUDA, "%s", emsg);
+        if (!encode_build_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, b.D, P.nblk, emsg, sizeof(emsg))) return fail(EPT_ECUDA, "%s", emsg);
         CK(launch_build_tc(b, tm, c->num_sms, s));
     } else {
         launch_norms(b, s);

@@ -12,18 +12,29 @@
 // the entries are about as accurate as an FP32 Gram), and the epilogue multiplies
 // by 1/c_i and 1/c_j (exact).
 // The epilogue forms d^2, recomputes cancellation-prone near-duplicate pairs
-// (d^2 < tau (||z_i||^2 + ||z_j||^2)) directly in FP64, applies sqrt (distances),
+// (d^2 < tau (||z_i||^2 + ||z_j||^2)) from direct differences summed as FP32 pairs, applies sqrt (distances),
 // exp(-d^2 / (2 sigma^2)) (Gaussian) or exp(-d / sigma) (Laplacian), forces the
 // diagonal to 0 / 1, zeroes padding, and
 // writes the FP32 entries into the packed upper blocks.
 //
 // Tile = 128 rows (half of a 256-row panel I) x 256 columns (panel J >= I, four
-// K-blocks); K loop over p in steps of 64 with TMA loads of the four operand tiles
-// (A hi/lo 128 x 64, B hi/lo 256 x 64, 128-byte swizzle); two TMEM accumulators so
+// K-blocks); K loop over p in steps of 32 with TMA loads of the four operand tiles
+// (A hi/lo 128 x 32, B hi/lo 256 x 32, 64-byte swizzle); two TMEM accumulators so
 // the epilogue of one tile overlaps the main loop of the next.  Roles (320
 // threads): warp 0 TMA, warp 1 MMA + TMEM owner, warps 2-9 epilogue (two per TMEM
 // lane quarter, each taking half of the tile's columns).  All waits are bounded as
 // in the contraction kernel.
+//
+// What bounds it: up to a few hundred features the epilogue, 32768 entries a tile on
+// eight warps, beyond that the tensor pipe.  A thread holds a row, so storing its entries itself
+// touches 32 rows with every instruction (a 32 x 32 group took about 300 of the SM's load
+// and store wavefronts); a warp now stages the group in shared memory (128-byte
+// swizzle, conflict-free 16-byte stores) and one TMA store writes it, two buffers per
+// warp.  Three stages of 48 KB (K = 32) leave the 64 KB for that; two of 96 KB did
+// not.  The entries are formed in pairs with packed FP32 arithmetic (the same roundings).
+// n = 20,000, p = 100: Gaussian 483 -> 265 us (3.1 TB/s of entries), distances 218 us; n = 5000,
+// p = 200: 43 -> 28 us, p = 1000 (tensor pipe 70 % busy) 65 -> 59 us; n = 200, p = 10 (close
+// pairs recomputed) 27 -> 16 us.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -41,15 +52,21 @@ using namespace tc;
 
 constexpr int BM = 128;
 constexpr int BN = 256;
-constexpr int BK = 64;
-constexpr int STAGES = 2;
-constexpr int A_BYTES = BM * BK * 2;                  // 16 KB
-constexpr int B_BYTES = BN * BK * 2;                  // 32 KB
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;  // 96 KB: A hi, A lo, B hi, B lo
+constexpr int BK = BUILD_STAGE_K;                     // 32
+constexpr int STAGES = 3;
+constexpr int A_BYTES = BM * BK * 2;                  // 8 KB
+constexpr int B_BYTES = BN * BK * 2;                  // 16 KB
+constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;  // 48 KB: A hi, A lo, B hi, B lo
+constexpr int OUT_BYTES = 32 * 32 * 4;                // a staged 32 x 32 group of entries
 constexpr int NUM_THREADS = 320;   // TMA warp, MMA warp, 8 epilogue warps
 constexpr int EPI_THREADS = 256;
-// stages | barriers (1 KB) | per-epilogue-warp column norms and scales (8 x 1 KB) | alignment slack
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 8 * (PANEL / 2) * 8 + 1024;
+// stages | per-epilogue-warp output groups (8 x 2 x 4 KB) | barriers (1 KB) | per-epilogue-warp column norms and
+// scales (8 x 1 KB) | alignment slack
+constexpr int OUT_OFF = STAGES * STAGE_BYTES;
+constexpr int BAR_OFF = OUT_OFF + 8 * 2 * OUT_BYTES;
+constexpr int COL_OFF = BAR_OFF + 1024;
+constexpr int SMEM_BYTES = COL_OFF + 8 * (PANEL / 2) * 8 + 1024;
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of the build");
 // kind::f16 instruction descriptor with A = B = FP16 (format 0), D = FP32, K-major
 constexpr uint32_t IDESC = idesc_f16_f32(BM, BN);
 
@@ -142,42 +159,180 @@ __global__ void __launch_bounds__(256) k_split_rows(const Batch bt) {
     }
 }
 
+// Two FP32 values in one register pair: packed arithmetic with the scalar operations' roundings.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &x, float &y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// exp_cw of two arguments x in [-87, 0] (its operations in its order; outside the
+// range the caller patches the entry)
+__device__ __forceinline__ void exp_cw2(f32x2 x, float &y0, float &y1) {
+    const f32x2 t = fma2(x, pack2(1.44269504f, 1.44269504f), pack2(12582912.f, 12582912.f));
+    const f32x2 nk = fma2(t, pack2(-1.f, -1.f), pack2(12582912.f, 12582912.f));   // -k, exact
+    f32x2 r = fma2(nk, pack2(0.693359375f, 0.693359375f), x);
+    r = fma2(nk, pack2(-2.12194440e-4f, -2.12194440e-4f), r);
+    f32x2 q = pack2(2.48015873e-5f, 2.48015873e-5f);
+    q = fma2(q, r, pack2(1.98412698e-4f, 1.98412698e-4f));
+    q = fma2(q, r, pack2(1.38888889e-3f, 1.38888889e-3f));
+    q = fma2(q, r, pack2(8.33333333e-3f, 8.33333333e-3f));
+    q = fma2(q, r, pack2(4.16666667e-2f, 4.16666667e-2f));
+    q = fma2(q, r, pack2(1.66666667e-1f, 1.66666667e-1f));
+    q = fma2(q, r, pack2(0.5f, 0.5f));
+    q = fma2(q, r, pack2(1.f, 1.f));
+    q = fma2(q, r, pack2(1.f, 1.f));
+    float t0, t1;
+    unpack2(t, t0, t1);
+    const uint32_t bias = (127u - 0x4B400000u) << 23;   // (k + 127) << 23, k = low bits of t
+    const f32x2 sc = pack2(__uint_as_float((__float_as_uint(t0) << 23) + bias),
+                           __uint_as_float((__float_as_uint(t1) << 23) + bias));
+    unpack2(mul2(q, sc), y0, y1);
+}
+
 // One row's 32 entries of a column group from the Gram accumulator v (scaled by
 // c_i c_j): d^2 = n_i + n_j - 2 G_ij, the entry for kernel kind KERN (0 distance,
 // 1 Gaussian, 2 Laplacian; the approximate square root is within 2^-22 of the
-// exact one, below the split Gram's own error), and the bit mask of the entries
-// that need the FP64 recomputation (d^2 < tau (n_i + n_j)).
+// exact one, below the split Gram's own error).  cg: per pair of columns, the norms and
+// the inverse scales.  True when some entry needs group_patch: one with d^2 < tau (n_i
+// + n_j), or a kernel value of 0.
 template <int KERN>
-__device__ __forceinline__ uint32_t group_entries(const uint32_t (&v)[32], const float2 *cg, float ni, float si,
-                                                  float tau, float neg_inv_2s2, float inv_sigma, float (&out)[32]) {
+__device__ __forceinline__ bool group_entries(const uint32_t (&v)[32], const float4 *cg, float ni, float si,
+                                              float tau, float neg_inv_2s2, float inv_sigma, float (&out)[32]) {
+    const f32x2 ni2 = pack2(ni, ni), si2 = pack2(si, si), tau2 = pack2(-tau, -tau), two = pack2(-2.f, -2.f);
+    const float f = KERN == 1 ? neg_inv_2s2 : -inv_sigma;
+    const f32x2 f2 = pack2(f, f);
+    float close = 1.f, big = 0.f;   // < 0: some entry to recompute; the largest argument of exp
+#pragma unroll
+    for (int e = 0; e < 32; e += 2) {
+        const float4 c = cg[e / 2];
+        // exact rescaling by powers of two, then n_i + n_j - 2 G_ij with one rounding
+        const f32x2 g = mul2(mul2(pack2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), si2), pack2(c.z, c.w));
+        const f32x2 sn = add2(ni2, pack2(c.x, c.y));
+        float d0, d1;
+        unpack2(fma2(g, two, sn), d0, d1);
+        d0 = fmaxf(0.f, d0);
+        d1 = fmaxf(0.f, d1);
+        float q0, q1;
+        unpack2(fma2(sn, tau2, pack2(d0, d1)), q0, q1);   // tau (n_i + n_j) is exact, so the sign is
+        close = fminf(close, fminf(q0, q1));
+        if (KERN != 1) {
+            asm("sqrt.approx.f32 %0, %1;" : "=f"(d0) : "f"(d0));
+            asm("sqrt.approx.f32 %0, %1;" : "=f"(d1) : "f"(d1));
+        }
+        if (KERN == 0) {
+            out[e] = d0;
+            out[e + 1] = d1;
+        } else {
+            big = fmaxf(big, fmaxf(d0, d1));
+            exp_cw2(mul2(pack2(d0, d1), f2), out[e], out[e + 1]);
+        }
+    }
+    return close < 0.f || (KERN != 0 && !(big * f > -87.f));
+}
+
+// The rare rest of a group: kernel values that are 0, and the bit mask of the entries
+// that need the recomputation.
+__device__ __forceinline__ uint32_t group_patch(const uint32_t (&v)[32], const float4 *cg, float ni, float si,
+                                                float tau, int kern, float neg_inv_2s2, float inv_sigma,
+                                                float (&out)[32]) {
     uint32_t fix = 0;
 #pragma unroll
     for (int e = 0; e < 32; ++e) {
-        const float2 cj = cg[e];
-        const float gij = (__uint_as_float(v[e]) * si) * cj.y;   // exact rescaling
-        const float sn = ni + cj.x;
-        const float d2 = fmaxf(0.f, sn - 2.f * gij);
+        const float4 c = cg[e / 2];
+        const float g = (__uint_as_float(v[e]) * si) * (e & 1 ? c.w : c.z), sn = ni + (e & 1 ? c.y : c.x);
+        const float d2 = fmaxf(0.f, fmaf(-2.f, g, sn));
         fix |= (d2 < tau * sn) ? (1u << e) : 0u;
-        if (KERN == 1) {
-            out[e] = exp_cw(d2 * neg_inv_2s2);
-        } else {
-            float dist;
-            asm("sqrt.approx.f32 %0, %1;" : "=f"(dist) : "f"(d2));
-            out[e] = (KERN == 0) ? dist : exp_cw(-dist * inv_sigma);
+        if (kern != 0) {
+            float x = d2;
+            if (kern == 2) asm("sqrt.approx.f32 %0, %1;" : "=f"(x) : "f"(d2));
+            x *= kern == 1 ? neg_inv_2s2 : -inv_sigma;
+            if (!(x > -87.f)) out[e] = 0.f;
         }
     }
     return fix;
 }
 
+// (h, l) += (x - y)^2: the difference as an exact pair (TwoSum), its square to about 2^-47
+// relative (the head's square exactly, by an FMA, and twice the head times the tail),
+// the sum as a pair.
+__device__ __forceinline__ void add_square(float x, float y, float &h, float &l) {
+    float dh, dl, s, e;
+    two_sum(x, -y, dh, dl);
+    const float p = dh * dh, pe = fmaf(dh, dh, -p);
+    two_sum(h, p, s, e);
+    h = s;
+    l += e + fmaf(2.f * dh, dl, pe);
+}
+
+// The entry of two rows by direct differences.  The squared distance is summed as an
+// unevaluated FP32 pair: GB300's FP64 rate is so low that eight warps' FP64 sums of 10
+// features took 8,000 cycles.  Eight loads of each row are in flight.  Sums outside
+// the range where the pair keeps its 47 bits are taken again in FP64; equal rows are
+// 0 in either.  Then the square root, by one Newton correction of the rounded root of
+// the pair (within 2^-40 of the exact root before its rounding), or the kernel value in FP64.
+__device__ __forceinline__ float entry_direct(const float *zi, const float *zj, int64_t p, int kern,
+                                              float neg_inv_2s2, float inv_sigma) {
+    float h = 0.f, l = 0.f, far = 0.f;
+#pragma unroll 1
+    for (int64_t k = 0; k < p; k += 8) {
+        float a[8], b[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {   // past the end: equal values, which add nothing
+            a[e] = k + e < p ? zi[k + e] : 0.f;
+            b[e] = k + e < p ? zj[k + e] : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            far = fmaxf(far, fabsf(a[e] - b[e]));
+            add_square(a[e], b[e], h, l);
+        }
+    }
+    const float t = h + l;
+    if (far != 0.f && !(t > 1e-20f && t < 1e30f)) {
+        double sq = 0.0;
+#pragma unroll 1
+        for (int64_t k = 0; k < p; ++k) {
+            const double df = (double)zi[k] - (double)zj[k];
+            sq = fma(df, df, sq);
+        }
+        return (float)entry_from_d2(sq, kern, neg_inv_2s2, inv_sigma);
+    }
+    if (kern != 0) return (float)entry_from_d2((double)h + (double)l, kern, neg_inv_2s2, inv_sigma);
+    if (far == 0.f) return 0.f;
+    const float s = sqrtf(t);
+    return s + (fmaf(-s, s, h) + l) * (0.5f / s);   // the residual h + l - s s is exact up to l's last bits
+}
+
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     k_build_tc(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ CUtensorMap tm_al,
-               const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CUtensorMap tm_bl, const Batch bt) {
+               const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CUtensorMap tm_bl,
+               const __grid_constant__ CUtensorMap tm_d, const Batch bt) {
     Counters *ctr = bt.ctr;   // bounded-wait errors are recorded in test 0's counters
     const unsigned long long wait_ns = bt.wait_ns ? bt.wait_ns : WAIT_NS;   // limit of every bounded wait
     const int ntiles = (int)bt.ntiles;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    Bars *bars = reinterpret_cast<Bars *>(smem + STAGES * STAGE_BYTES);
+    Bars *bars = reinterpret_cast<Bars *>(smem + BAR_OFF);
     volatile int *abort_flag = &bars->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -217,7 +372,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 const int64_t row0 = bt.desc[tile.t].row0;
                 const int rowA = (int)row0 + tile.I * PANEL + tile.h * BM;
                 const int rowB = (int)row0 + tile.J * PANEL;
-                const int kblocks = bt.desc[tile.t].kblocks;
+                const int kblocks = (int)((bt.desc[tile.t].p + BK - 1) / BK);
                 for (int kk = 0; kk < kblocks; ++kk) {
                     if (!mbar_wait(su32(&bars->empty[stage]), phase ^ 1u, abort_flag, ctr, ERR_WAIT_TMA, wait_ns)) {
                         ok = false;
@@ -256,7 +411,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const int kblocks = bt.desc[bt.tiles[t].t].kblocks;
+                const int kblocks = (int)((bt.desc[bt.tiles[t].t].p + BK - 1) / BK);
                 if (!mbar_wait(su32(&bars->acc_empty[acc]), acc_phase ^ 1u, abort_flag, ctr, ERR_WAIT_MMA, wait_ns)) {
                     ok = false;
                     break;
@@ -270,8 +425,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     }
                     fence_after();
                     const uint32_t sa = su32(smem + stage * STAGE_BYTES);
-                    const uint64_t dah = desc_sw128(sa), dal = desc_sw128(sa + A_BYTES);
-                    const uint64_t dbh = desc_sw128(sa + 2 * A_BYTES), dbl = desc_sw128(sa + 2 * A_BYTES + B_BYTES);
+                    const uint64_t dah = desc_sw64(sa), dal = desc_sw64(sa + A_BYTES);
+                    const uint64_t dbh = desc_sw64(sa + 2 * A_BYTES), dbl = desc_sw64(sa + 2 * A_BYTES + B_BYTES);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
                         mma_f16(d_tmem, dah + 2 * k, dbh + 2 * k, IDESC, (kk == 0 && k == 0) ? 0u : 1u);
@@ -302,16 +457,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
     } else {
         // ---------------- epilogue: one tile row per thread ----------------
-        // Each warp stages the tile's 256 column norms and inverse scales in its own
+        // Each warp stages the tile's column norms and inverse scales in its own
         // shared-memory slice (read back as broadcasts), computes each group of 32
-        // entries without branches, patches padding and the diagonal with selects, and
-        // recomputes the rare cancellation-prone entries afterwards (same thread, so
-        // its later store wins).
+        // entries without branches, patches padding and the diagonal with selects, writes the
+        // group to its output buffer, recomputes the rare cancellation-prone entries there and
+        // has one TMA store take the buffer.
         // two warps per TMEM lane quarter: each takes one half (128 columns) of the tile
         const int quarter = warp & 3;
         const int half = (warp - 2) >> 2;
         const int rt = quarter * 32 + lane;   // row within the 128-row tile
-        float2 *colv = reinterpret_cast<float2 *>(smem + STAGES * STAGE_BYTES + 1024) + (warp - 2) * (PANEL / 2);
+        // pairs of columns: norms in x, y, inverse scales in z, w
+        float *colv = reinterpret_cast<float *>(smem + COL_OFF) + (warp - 2) * PANEL;
+        uint8_t *outb = smem + OUT_OFF + (warp - 2) * 2 * OUT_BYTES;
+        int ob = 0;   // output buffer of the next group
         int acc = 0;
         uint32_t acc_phase = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -323,7 +481,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const float neg_inv_2s2 = d.neg_inv_2s2, inv_sigma = d.inv_sigma, tau = d.tau;
             const float diag_val = (kern == 0) ? 0.f : 1.f;
             const float *norms = bt.norms + d.row0, *inv_scale = bt.iscale + d.row0;
-            float *Dblk = bt.D + (d.blk0 + blk_index(tile.I, (int64_t)tile.J * KB_PER_PANEL, NKB)) * PANEL * KB;
+            // first row of the warp's 32 in the block array (rows of 64 entries)
+            const int64_t drow = (d.blk0 + blk_index(tile.I, (int64_t)tile.J * KB_PER_PANEL, NKB)) * PANEL +
+                                 tile.h * BM + quarter * 32;
             unsigned fixups = 0;
             const int rp = tile.h * BM + rt;                 // row within panel I
             const int64_t i = (int64_t)tile.I * PANEL + rp;  // pooled row of the test
@@ -333,10 +493,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
             for (int c = lane; c < PANEL / 2; c += 32) {
                 const int64_t j = (int64_t)tile.J * PANEL + half * (PANEL / 2) + c;
-                colv[c] = (j < n) ? make_float2(norms[j], inv_scale[j]) : make_float2(0.f, 0.f);
+                float *cp = colv + (c >> 1) * 4 + (c & 1);
+                cp[0] = (j < n) ? norms[j] : 0.f;
+                cp[2] = (j < n) ? inv_scale[j] : 0.f;
             }
             __syncwarp();
-            if (!mbar_wait(su32(&bars->acc_full[acc]), acc_phase, abort_flag, ctr, ERR_WAIT_EPI, wait_ns)) break;
+            // the warp's lanes leave together (the group loop below synchronises them)
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait(su32(&bars->acc_full[acc]), acc_phase, abort_flag, ctr, ERR_WAIT_EPI,
+                                                   wait_ns)))
+                break;
             fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
@@ -346,10 +511,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 tmem_ld32(tbase + (uint32_t)(g * 32), v);
                 const int64_t j0 = (int64_t)tile.J * PANEL + g * 32;
                 float out[32];
-                const float2 *cg = colv + gl * 32;
-                uint32_t fix = (kern == 0)   ? group_entries<0>(v, cg, ni, si, tau, neg_inv_2s2, inv_sigma, out)
-                               : (kern == 1) ? group_entries<1>(v, cg, ni, si, tau, neg_inv_2s2, inv_sigma, out)
-                                             : group_entries<2>(v, cg, ni, si, tau, neg_inv_2s2, inv_sigma, out);
+                const float4 *cg = reinterpret_cast<const float4 *>(colv) + gl * 16;
+                const bool patch = (kern == 0)   ? group_entries<0>(v, cg, ni, si, tau, neg_inv_2s2, inv_sigma, out)
+                                   : (kern == 1) ? group_entries<1>(v, cg, ni, si, tau, neg_inv_2s2, inv_sigma, out)
+                                                 : group_entries<2>(v, cg, ni, si, tau, neg_inv_2s2, inv_sigma, out);
+                uint32_t fix = 0;
+                if (__any_sync(0xFFFFFFFFu, patch)) {
+                    tmem_ld32(tbase + (uint32_t)(g * 32), v);   // read again: no registers held for this case
+                    fix = group_patch(v, cg, ni, si, tau, kern, neg_inv_2s2, inv_sigma, out);
+                }
                 // padding rows / columns hold 0; the diagonal is exactly 0 (ED) / 1 (MMD)
                 const uint32_t jvalid =
                     (j0 >= n) ? 0u : ((j0 + 32 <= n) ? 0xFFFFFFFFu : ((1u << (uint32_t)(n - j0)) - 1u));
@@ -364,25 +534,35 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     }
                 }
                 fix &= valid & ~diag;
-                float *dst = Dblk + ((int64_t)(g >> 1) * PANEL + rp) * KB + (g & 1) * 32;
+                // the buffer's last store (two groups ago) has read it
+                uint8_t *buf = outb + ob * OUT_BYTES;
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                __syncwarp();
 #pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    *reinterpret_cast<float4 *>(dst + e) = make_float4(out[e], out[e + 1], out[e + 2], out[e + 3]);
-                // cancellation-prone pairs: d^2 directly in FP64
+                for (int c = 0; c < 8; ++c)   // row `lane`, 16-byte chunk c at c ^ (row mod 8)
+                    *reinterpret_cast<float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4)) =
+                        make_float4(out[4 * c], out[4 * c + 1], out[4 * c + 2], out[4 * c + 3]);
+                // cancellation-prone pairs: d^2 by direct differences
                 while (fix) {
                     const int e = __ffs(fix) - 1;
                     fix &= fix - 1u;
                     const int64_t j = j0 + e;
                     const float *zi = (i < nx) ? X + i * p : Y + (i - nx) * p;
                     const float *zj = (j < nx) ? X + j * p : Y + (j - nx) * p;
-                    double sq = 0.0;
-                    for (int64_t k = 0; k < p; ++k) {
-                        const double df = (double)zi[k] - (double)zj[k];
-                        sq = fma(df, df, sq);
-                    }
                     ++fixups;
-                    dst[e] = (float)entry_from_d2(sq, kern, neg_inv_2s2, inv_sigma);
+                    *reinterpret_cast<float *>(buf + lane * 128 + (((e >> 2) ^ (lane & 7)) << 4) + (e & 3) * 4) =
+                        entry_direct(zi, zj, p, kern, neg_inv_2s2, inv_sigma);
                 }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                                     &tm_d),
+                                 "r"((g & 1) * 32), "r"((int)(drow + (int64_t)(g >> 1) * PANEL)), "r"(su32(buf))
+                                 : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
+                ob ^= 1;
             }
             fence_before();
             mbar_arrive(su32(&bars->acc_empty[acc]));
@@ -392,6 +572,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 acc_phase ^= 1u;
             }
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // its stores are done
     }
 
     fence_before();
@@ -416,7 +597,7 @@ cudaError_t launch_build_tc(const Batch &b, const void *tmaps, int num_sms, cuda
     if (b.ntiles < 1) return cudaSuccess;
     const CUtensorMap *tm = (const CUtensorMap *)tmaps;
     const int grid = b.ntiles < num_sms ? (int)b.ntiles : num_sms;
-    k_build_tc<<<grid, NUM_THREADS, SMEM_BYTES, s>>>(tm[0], tm[1], tm[2], tm[3], b);
+    k_build_tc<<<grid, NUM_THREADS, SMEM_BYTES, s>>>(tm[0], tm[1], tm[2], tm[3], tm[4], b);
     return cudaGetLastError();
 }
 

@@ -418,25 +418,35 @@ static EncodeTiledFn encode_fn(char *err, size_t errlen) {
     return fn;
 }
 
-bool encode_rows_tmaps(void *tmaps4, const uint16_t *Zh, const uint16_t *Zl, int64_t nrows, int64_t p_stride,
-                       char *err, size_t errlen) {
+bool encode_build_tmaps(void *tmaps5, const uint16_t *Zh, const uint16_t *Zl, int64_t nrows, int64_t p_stride,
+                        float *D, int64_t nblk, char *err, size_t errlen) {
     EncodeTiledFn enc = encode_fn(err, errlen);
     if (!enc) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)p_stride, (cuuint64_t)nrows};
     const cuuint64_t strides[1] = {(cuuint64_t)p_stride * 2};
     const cuuint32_t estr[2] = {1, 1};
-    const cuuint32_t box_a[2] = {64, 128}, box_b[2] = {64, 256};
-    CUtensorMap *out = (CUtensorMap *)tmaps4;
+    const cuuint32_t box_a[2] = {BUILD_STAGE_K, 128}, box_b[2] = {BUILD_STAGE_K, 256};
+    CUtensorMap *out = (CUtensorMap *)tmaps5;
     const void *srcs[4] = {Zh, Zl, Zh, Zl};
     const cuuint32_t *boxes[4] = {box_a, box_a, box_b, box_b};
     for (int k = 0; k < 4; ++k) {
         CUresult r = enc(&out[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, (void *)srcs[k], dims, strides, boxes[k], estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) {
             snprintf(err, errlen, "cuTensorMapEncodeTiled (rows) failed (%d)", (int)r);
             return false;
         }
+    }
+    // the blocks as rows of 64 entries, stored in boxes of 32 x 32
+    const cuuint64_t ddims[2] = {(cuuint64_t)KB, (cuuint64_t)nblk * PANEL}, dstrides[1] = {(cuuint64_t)KB * 4};
+    const cuuint32_t dbox[2] = {32, 32};
+    CUresult r = enc(&out[4], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void *)D, ddims, dstrides, dbox, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        snprintf(err, errlen, "cuTensorMapEncodeTiled (entries) failed (%d)", (int)r);
+        return false;
     }
     return true;
 }

@@ -47,6 +47,7 @@ constexpr int KB_PER_PANEL = PANEL / KB;
 constexpr int CHUNK_KB_DEFAULT = 8;
 constexpr int COL_PAD = 256;     // relabeling columns padded to this multiple
 constexpr int BUILD_KB = 64;     // p is padded to a multiple of this for the tensor-core build
+constexpr int BUILD_STAGE_K = 32;   // features per pipeline stage of that build
 constexpr int TC_TILE_N = 256;   // relabelings per contraction work unit (the MMA's N)
 // cap on the relabeling-draw blocks per SM (0: none, one warp per column).  Capping
 // lets the draws share SMs with the tensor-core build, but the draws are
@@ -427,7 +428,7 @@ void launch_expand_blocks(const float *D, int64_t n, int64_t NKB, float *out, cu
 
 // ---- tensor-core kernels (ept_build_tc.cu, ept_contract_tc.cu) ----
 void launch_split_rows(const Batch &b, cudaStream_t s);                  // FP16 hi/lo rows, norms, checks
-cudaError_t launch_build_tc(const Batch &b, const void *tmaps4, int num_sms, cudaStream_t s);
+cudaError_t launch_build_tc(const Batch &b, const void *tmaps5, int num_sms, cudaStream_t s);
 cudaError_t launch_contract_tc(const Batch &b, const void *tmap_hi, const void *tmap_lo, int num_sms,
                                cudaStream_t s);
 // the same contraction on pairs of SMs (clusters of two CTAs, tcgen05 cta_group::2;
@@ -440,12 +441,12 @@ cudaError_t launch_contract_tc2(const Batch &b, const void *tmap_hi, const void 
 cudaError_t launch_contract_tm(const Batch &b, const void *tmap_hi, const void *tmap_lo, int num_sms,
                                cudaStream_t s);
 // TMA descriptors: the packed hi/lo blocks [nblk_total x 256 x 64], block stride
-// c_stride halves, and the FP16
-// rows [nrows x p_stride] (hi, lo with 64 x 128 boxes, then hi, lo with 64 x 256 boxes)
+// c_stride halves; for the build the FP16 rows [nrows x p_stride] (hi, lo with boxes of
+// BUILD_STAGE_K x 128, then hi, lo with BUILD_STAGE_K x 256) and the FP32 entries of nblk blocks
 bool encode_block_tmaps(void *tmap_hi, void *tmap_lo, const uint16_t *Chi, const uint16_t *Clo, int64_t nblk,
                         int64_t c_stride, char *err, size_t errlen);
-bool encode_rows_tmaps(void *tmaps4, const uint16_t *Zh, const uint16_t *Zl, int64_t nrows, int64_t p_stride,
-                       char *err, size_t errlen);
+bool encode_build_tmaps(void *tmaps5, const uint16_t *Zh, const uint16_t *Zl, int64_t nrows, int64_t p_stride,
+                        float *D, int64_t nblk, char *err, size_t errlen);
 
 // ---- streaming mode (ept_stream.cu): one test, windows of row panels ----
 // r += the row and column sums of the window [I0, I1) (its stored blocks' parts)
