@@ -21,24 +21,37 @@
 //   64 multiply-adds (half of what the relabelings-as-M mapping needs), and three
 //   64 KB stages fit in shared memory.  Two accumulators (512 TMEM columns) let the
 //   epilogue of one unit overlap the main loop of the next.
-//   Epilogue: TMEM lane = row i; a warp reads 32 relabelings at a time, takes the
-//   mask bits of its 32 rows for them with a 32 x 32 bit transpose (shuffles), masks
-//   its values, and sums over its 32 rows with a butterfly transpose-reduce (lane e
-//   ends with relabeling e's sum).  The four warps' sums meet in shared memory and
-//   are added in a fixed order.
+//   Epilogue: TMEM lane = row i; a warp takes its 32 rows of 32 relabelings at a time,
+//   masks them and sums over the rows (masked_block_sum in ept_tc_common.cuh).  The four
+//   warps' sums meet in shared memory and are added in a fixed order.
 //
-// Roles (576 threads): warp 0 = TMA producer, warp 1 = MMA issuer (and TMEM
+// Roles (640 threads): warp 0 = TMA producer, warp 1 = MMA issuer (and TMEM
 // owner), warps 2-9 = epilogue (two warps per TMEM lane quarter, each taking half
-// of the relabelings), warps 10-17 = relabeling-tile producers (one B row each).
+// of the relabelings), warps 10-12, 14-16, 18, 19 = relabeling-tile producers (one B row
+// a thread); warps 13 and 17 leave at once.
 // Every role takes its units from the precomputed 64-byte records of the schedule
 // (UnitRec) and reads the next unit's record while it works on the current one, so
 // that no role waits on the schedule, test and chunk tables at a unit boundary.
-// Two epilogue and two producer warps per SM sub-partition hide each other's
-// shared-memory and L2 latencies.  Every wait on an mbarrier is bounded (2 s unless
+// Every wait on an mbarrier is bounded (2 s unless
 // the context sets another limit), and a waiting thread sleeps in the wait until its
 // phase completes; on expiry the kernel records an error code, raises a CTA-wide
 // abort flag, drains its own copies and MMAs (bounded again), frees its tensor
 // memory and returns.
+//
+// What bounds it: the MMAs (128 cycles each for 128 x 256 x 16: 221 us at the 1.96 GHz
+// it runs at for n = 5000, B = 10^4; 3.40 ms for n = 20,000), as far as their issuer keeps
+// them coming.  The tensor core queues little: whatever delays the issuer between two
+// stages is a gap, and its instructions compete for issue slots with the warps of its SM
+// sub-partition.  Hence: the whole warp runs the issuing loop (uniform operands, one
+// elected lane issues); a stage has one barrier for the copies and the relabeling tile;
+// no producer warp shares the sub-partition of warp 1 (two epilogue warps have to: a TMEM
+// lane quarter belongs to the sub-partition); the tile is expanded by arithmetic, not from a table in
+// shared memory, whose bandwidth the MMAs' operands take to three quarters; and
+// the epilogue needs few shuffles and selects.  Without any epilogue or producer work the
+// same launch takes 246 us.  n = 5000: 303 -> 256 us (step by step: expansion in registers
+// 297, epilogue 284, uniform issuer 280, sub-partitions 264, one barrier 256); n = 20,000: 4.44 -> 3.73 ms;
+// n = 9500, B = 5000: 524 -> 442 us; n = 2600: 53 -> 45 us.  Tried and slower: looking at the next stage's
+// barrier ahead of time, one arrival per producer warp, one polling lane per warp.
 #include <cuda.h>
 #include <cstdio>
 #include <cstring>
@@ -59,9 +72,9 @@ constexpr int A_BYTES = TC_M * KB * 2;            // 16 KB (hi or lo)
 constexpr int B_BYTES = TC_N * KB * 2;            // 32 KB
 constexpr int STAGE_BYTES = 2 * A_BYTES + B_BYTES;   // A hi | A lo | B
 constexpr int RED_BYTES = 2 * 4 * TC_N * 4;       // epilogue sums: 2 buffers x 4 warps x 256 floats
-constexpr int NUM_THREADS = 576;
+constexpr int NUM_THREADS = 640;
 constexpr int EPI_THREADS = 256;                  // warps 2-9
-constexpr int PROD_THREADS = 256;                 // warps 10-17
+constexpr int PROD_THREADS = 256;                 // warps 10-12, 14-16, 18, 19 (none beside the MMA issuer, warp 1)
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*barriers*/ + RED_BYTES + 1024 /*alignment*/;
 
 // error codes recorded in Counters::err_code
@@ -70,10 +83,10 @@ constexpr unsigned long long ERR_WAIT_TMA = 0x101, ERR_WAIT_MMA = 0x102, ERR_WAI
 
 constexpr uint32_t IDESC = idesc_f16_f32(TC_M, TC_N);
 
-// the barrier region (1 KB): Bars at its start, the 128-byte nibble table at byte 512
+// the barrier region (1 KB)
 struct Bars {
-    unsigned long long b_full[STAGES];   // 256 producer-thread arrivals (relabeling tile)
-    unsigned long long a_full[STAGES];   // 1 arrival + TMA transaction bytes (C half-block)
+    unsigned long long full[STAGES];     // 256 producer-thread arrivals (relabeling tile), 1 arrival + TMA
+                                         //   transaction bytes (C half-block)
     unsigned long long empty[STAGES];    // 1 arrival (tcgen05.commit)
     unsigned long long acc_full[2];      // 1 arrival (tcgen05.commit)
     unsigned long long acc_empty[2];     // 256 epilogue-thread arrivals
@@ -82,7 +95,7 @@ struct Bars {
     uint32_t tmem_base;
     int abort_flag;
 };
-static_assert(sizeof(Bars) <= 512, "barriers overlap the nibble table");
+static_assert(sizeof(Bars) <= 1024, "barrier region");
 
 // MMA N for a unit: the tile's existing relabeling columns, rounded up to 16
 __device__ __forceinline__ int mma_n(const UnitRec &x) { return x.left >= TC_N ? TC_N : (x.left + 15) / 16 * 16; }
@@ -106,17 +119,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int64_t k_step = bt.sched ? 1 : (int64_t)gridDim.x;
     auto record = [&bt, k_end](int64_t k) { return k < k_end ? unit_at_position(bt, k) : UnitRec{}; };
 
-    // nibble -> four FP16 values (1.0 where the bit is set), for the relabeling producers
-    uint2 *lut = reinterpret_cast<uint2 *>(smem + STAGES * STAGE_BYTES + 512);
-    if (threadIdx.x < 16) {
-        const uint32_t n = threadIdx.x;
-        lut[n] = make_uint2((n & 1u) * 0x3C00u + (n & 2u) * 0x1E000000u,
-                            ((n >> 2) & 1u) * 0x3C00u + ((n >> 2) & 2u) * 0x1E000000u);
-    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(su32(&bars->b_full[s]), PROD_THREADS);
-            mbar_init(su32(&bars->a_full[s]), 1);
+            mbar_init(su32(&bars->full[s]), PROD_THREADS + 1);
             mbar_init(su32(&bars->empty[s]), 1);
         }
         for (int a = 0; a < 2; ++a) {
@@ -157,12 +162,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         ok = false;
                         break;
                     }
-                    const uint32_t afull = su32(&bars->a_full[stage]);
-                    mbar_arrive_tx(afull, 2 * A_BYTES);
+                    const uint32_t full = su32(&bars->full[stage]);
+                    mbar_arrive_tx(full, 2 * A_BYTES);
                     const int blk = (int)(x.blk0 + blk_index(x.I, kb, x.NKB));
                     uint8_t *st = smem + stage * STAGE_BYTES;
-                    tma_load_3d(su32(st), &tmap_hi, 0, row, blk, afull);
-                    tma_load_3d(su32(st + A_BYTES), &tmap_lo, 0, row, blk, afull);
+                    tma_load_3d(su32(st), &tmap_hi, 0, row, blk, full);
+                    tma_load_3d(su32(st + A_BYTES), &tmap_lo, 0, row, blk, full);
                     armed[stage] = (int)phase;
                     if (++stage == STAGES) {
                         stage = 0;
@@ -171,12 +176,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 }
             }
             if (!ok) {
-                // drain: the copies armed last on each stage complete that phase of
-                // a_full; wait for it (bounded) before the CTA may exit
+                // drain: the copies armed last on each stage complete that phase of its
+                // barrier (the producers arrive on every stage when they give up); wait
+                // for it (bounded) before the CTA may exit
                 for (int s2 = 0; s2 < STAGES; ++s2) {
                     if (armed[s2] < 0) continue;
                     const unsigned long long t0 = gtimer();
-                    while (!mbar_try(su32(&bars->a_full[s2]), (uint32_t)armed[s2])) {
+                    while (!mbar_try(su32(&bars->full[s2]), (uint32_t)armed[s2])) {
                         if (gtimer() - t0 > wait_ns) {
                             atomicCAS(&ctr->err_code, 0ull, ERR_DRAIN);
                             break;
@@ -187,57 +193,65 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            int stage = 0, acc = 0;
-            uint32_t phase = 0, acc_phase = 0;
-            bool ok = true;
-            // failure-path test hook: wait (bounded) on a flag that nothing sets; the
-            // expiry takes the same abort path as any other expired wait
-            if (bt.inject_stall && !flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns)) ok = false;
-            UnitRec nx = record(k_first);
-            for (int64_t k = k_first; k < k_end && ok; k += k_step) {
-                const UnitRec x = nx;
-                nx = record(k + k_step);
-                const int ncols = mma_n(x);
-                const uint32_t idesc = (ncols == TC_N) ? IDESC : idesc_f16_f32(TC_M, ncols);
-                if (!mbar_wait(su32(&bars->acc_empty[acc]), acc_phase ^ 1u, abort_flag, ctr, ERR_WAIT_MMA, wait_ns)) {
+        // The whole warp runs the loop, so that its values are uniform (an MMA takes its
+        // operands from uniform registers; in a branch of one lane each had to be moved there
+        // first, by the warp whose delays the tensor pipe sees), and one elected lane issues.
+        int stage = 0, acc = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        bool ok = true;
+        // failure-path test hook: wait (bounded) on a flag that nothing sets; the
+        // expiry takes the same abort path as any other expired wait
+        if (bt.inject_stall) ok = __all_sync(0xFFFFFFFFu, flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns));
+        UnitRec nx = record(k_first);
+        for (int64_t k = k_first; k < k_end && ok; k += k_step) {
+            const UnitRec x = nx;
+            nx = record(k + k_step);
+            const int ncols = mma_n(x);
+            const uint32_t idesc = (ncols == TC_N) ? IDESC : idesc_f16_f32(TC_M, ncols);
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait(su32(&bars->acc_empty[acc]), acc_phase ^ 1u, abort_flag, ctr,
+                                                   ERR_WAIT_MMA, wait_ns))) {
+                ok = false;
+                break;
+            }
+            fence_after();
+            const uint32_t d_tmem = tmem_base + (uint32_t)(acc * TC_N);
+            uint32_t accumulate = 0;
+            for (int kb = x.kb0; kb < x.kb1; ++kb) {
+                if (!__all_sync(0xFFFFFFFFu,
+                                mbar_wait(su32(&bars->full[stage]), phase, abort_flag, ctr, ERR_WAIT_MMA, wait_ns))) {
                     ok = false;
                     break;
                 }
                 fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * TC_N);
-                bool first = true;
-                for (int kb = x.kb0; kb < x.kb1; ++kb) {
-                    if (!mbar_wait(su32(&bars->a_full[stage]), phase, abort_flag, ctr, ERR_WAIT_MMA, wait_ns) ||
-                        !mbar_wait(su32(&bars->b_full[stage]), phase, abort_flag, ctr, ERR_WAIT_MMA, wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    fence_after();
-                    const uint32_t sa = su32(smem + stage * STAGE_BYTES);
-                    const uint64_t dhi = desc_sw128(sa);
-                    const uint64_t dlo = desc_sw128(sa + A_BYTES);
-                    const uint64_t db = desc_sw128(sa + 2 * A_BYTES);
+                const uint32_t sa = su32(smem) + (uint32_t)(stage * STAGE_BYTES);
+                const uint64_t dhi = desc_sw128(sa);
+                const uint64_t dlo = desc_sw128(sa + A_BYTES);
+                const uint64_t db = desc_sw128(sa + 2 * A_BYTES);
+                if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < KB / 16; ++k)
-                        mma_f16(d_tmem, dhi + 2 * k, db + 2 * k, idesc, (first && k == 0) ? 0u : 1u);
+                        mma_f16(d_tmem, dhi + 2 * k, db + 2 * k, idesc, k == 0 ? accumulate : 1u);
 #pragma unroll
                     for (int k = 0; k < KB / 16; ++k) mma_f16(d_tmem, dlo + 2 * k, db + 2 * k, idesc, 1u);
                     mma_commit(su32(&bars->empty[stage]));
-                    first = false;
-                    if (++stage == STAGES) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
                 }
-                if (!ok) break;
-                mma_commit(su32(&bars->acc_full[acc]));
-                if (++acc == 2) {
-                    acc = 0;
-                    acc_phase ^= 1u;
+                __syncwarp();
+                accumulate = 1;
+                if (++stage == STAGES) {
+                    stage = 0;
+                    phase ^= 1u;
                 }
             }
-            // drain every MMA this thread issued before the CTA frees its tensor memory
+            if (!ok) break;
+            if (elect_one()) mma_commit(su32(&bars->acc_full[acc]));
+            __syncwarp();
+            if (++acc == 2) {
+                acc = 0;
+                acc_phase ^= 1u;
+            }
+        }
+        // drain every MMA the warp issued before the CTA frees its tensor memory
+        if (elect_one()) {
             mma_commit(su32(&bars->drain));
             unsigned long long t0 = gtimer();
             while (!mbar_try(su32(&bars->drain), 0)) {
@@ -247,6 +261,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 }
             }
         }
+        __syncwarp();
     } else if (warp < 10) {
         // ---------------- epilogue ----------------
         const int quarter = warp & 3;           // TMEM lanes (rows) this warp may access
@@ -260,55 +275,37 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const UnitRec x = nx;
             nx = record(k + k_step);
             const int64_t Bp = x.Bp;
-            // mask word of this warp's 32 rows, for the warp's 128 relabelings
-            const uint32_t *wrow = bt.maskT + x.mask_col + ((int64_t)x.I * 8 + x.h * 4 + quarter) * Bp + g0 * 32;
-            uint32_t words[4];
+            // mask words of this warp's 32 rows: the thread's pairs of relabelings (masked_block_sum)
+            const uint32_t *wrow = bt.maskT + x.mask_col + ((int64_t)x.I * 8 + x.h * 4 + quarter) * Bp + g0 * 32 +
+                                   2 * (lane & 3);
+            uint2 w[4], wn[4];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) words[g] = wrow[g * 32 + lane];
-            if (!mbar_wait(su32(&bars->acc_full[acc]), acc_phase, abort_flag, ctr, ERR_WAIT_EPI, wait_ns)) break;
+            for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint2 *>(wrow + 8 * j);
+            // the warp's lanes leave together: the loads below are collective
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait(su32(&bars->acc_full[acc]), acc_phase, abort_flag, ctr, ERR_WAIT_EPI,
+                                                   wait_ns)))
+                break;
             fence_after();
             const uint32_t tbase =
                 tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * TC_N) + (uint32_t)(g0 * 32);
             float *myred = red + (rbuf * 4 + quarter) * TC_N + g0 * 32;
 #pragma unroll 1
             for (int g = 0; g < 4; ++g) {
-                uint32_t v[32];
-                tmem_ld32(tbase + (uint32_t)(g * 32), v);
-                // bit e of `mine` = s_{b_e}[row of this lane], b_e = relabeling 32 (g0 + g) + e:
-                // the 32 x 32 bit matrix (lane = relabeling, bit = row) transposed in five
-                // butterfly stages, each swapping the off-diagonal halves of 2j x 2j blocks
-                uint32_t mine = words[g];
+                if (g < 3) {   // the next block's words arrive while this one is summed
 #pragma unroll
-                for (int j = 16; j >= 1; j >>= 1) {
-                    const uint32_t m = j == 16 ? 0x0000FFFFu
-                                     : j == 8  ? 0x00FF00FFu
-                                     : j == 4  ? 0x0F0F0F0Fu
-                                     : j == 2  ? 0x33333333u
-                                               : 0x55555555u;
-                    const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, mine, j);
-                    mine = (lane & j) ? ((mine & ~m) | ((y & ~m) >> j)) : ((mine & m) | ((y & m) << j));
+                    for (int j = 0; j < 4; ++j)
+                        wn[j] = *reinterpret_cast<const uint2 *>(wrow + 32 * (g + 1) + 8 * j);
                 }
-                float xv[32];
+                myred[g * 32 + masked_sum_col(lane)] = masked_block_sum(tbase + (uint32_t)(g * 32), w, lane);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) xv[e] = ((mine >> e) & 1u) ? __uint_as_float(v[e]) : 0.f;
-                // butterfly transpose-reduce: lane e ends with the sum over the warp's rows of column e
-#pragma unroll
-                for (int off = 16; off >= 1; off >>= 1) {
-                    const bool upper = (lane & off) != 0;
-#pragma unroll
-                    for (int k = 0; k < off; ++k) {
-                        const float send = upper ? xv[k] : xv[k + off];
-                        const float keep = upper ? xv[k + off] : xv[k];
-                        xv[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, off);
-                    }
-                }
-                myred[g * 32 + lane] = xv[0];
+                for (int j = 0; j < 4; ++j) w[j] = wn[j];
             }
             fence_before();
             mbar_arrive(su32(&bars->acc_empty[acc]));
             // the four row quarters' sums, added in a fixed order
             mbar_arrive(su32(&bars->red));
-            if (!mbar_wait(su32(&bars->red), red_phase, abort_flag, ctr, ERR_WAIT_EPI, wait_ns)) break;
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait(su32(&bars->red), red_phase, abort_flag, ctr, ERR_WAIT_EPI, wait_ns)))
+                break;
             const float *rb = red + rbuf * 4 * TC_N;
             float *out = bt.partial + x.out_off;
             out[et] = (rb[et] + rb[TC_N + et]) + (rb[2 * TC_N + et] + rb[3 * TC_N + et]);
@@ -319,58 +316,69 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 acc_phase ^= 1u;
             }
         }
-    } else {
+    } else if (warp != 13 && warp != 17) {
         // ---------------- relabeling-tile producers ----------------
-        // The mask words of a stage are loaded two stages ahead, so that their L2
-        // latency overlaps the expansion of the stages before.
-        const int r = threadIdx.x - 320;   // 0..255: row r of the B tile
+        // A stage costs its mask words from L2, the expansion and eight 16-byte stores a
+        // thread.  Everything but the stores happens before the stage is free: the words are
+        // loaded two stages ahead, across unit boundaries, and expanded in registers (expand_bits).
+        const int r = (warp - 10 - (warp > 13) - (warp > 17)) * 32 + lane;   // 0..255: row r of the B tile
+        // the next K-block to load: its unit's first mask word of relabeling r, or the next unit's
+        struct Words { uint32_t x, y; bool live; };   // words 2 kb and 2 kb + 1; live: the MMA reads the row
+        const uint32_t *fp = nullptr;
+        int64_t f_bp = 0, fk = k_first;
+        int f_kb = 0, f_kb1 = 0;
+        bool f_live = false;
+        UnitRec fn = record(k_first);   // the unit after the one being loaded
+        auto fetch = [&](Words &w) {
+            if (f_kb == f_kb1) {
+                if (fk >= k_end) return false;
+                f_bp = fn.Bp;
+                f_kb = fn.kb0;
+                f_kb1 = fn.kb1;
+                f_live = r < mma_n(fn);   // rows past the tile's columns are not read by the MMA
+                fp = bt.maskT + fn.mask_col + r + (int64_t)(2 * f_kb) * f_bp;
+                fk += k_step;
+                fn = record(fk);
+            }
+            w.x = fp[0];
+            w.y = fp[f_bp];
+            w.live = f_live;
+            fp += 2 * f_bp;
+            ++f_kb;
+            return true;
+        };
         int stage = 0;
         uint32_t phase = 0;
-        bool ok = true;
-        UnitRec nx = record(k_first);
-        for (int64_t k = k_first; k < k_end && ok; k += k_step) {
-            const UnitRec x = nx;
-            nx = record(k + k_step);
-            const int64_t Bp = x.Bp;
-            const uint32_t *maskT = bt.maskT + x.mask_col + r;
-            // words 2 kb and 2 kb + 1 of relabeling r
-            auto load2 = [&](int kb, uint2 &w) {
-                const uint32_t *p0 = maskT + (int64_t)(2 * kb) * Bp;
-                w.x = p0[0];
-                w.y = p0[Bp];
-            };
-            uint2 cur = make_uint2(0, 0), nxt = make_uint2(0, 0);
-            load2(x.kb0, cur);
-            if (x.kb0 + 1 < x.kb1) load2(x.kb0 + 1, nxt);
-            const int ncols = mma_n(x);
-            for (int kb = x.kb0; kb < x.kb1; ++kb) {
-                uint2 nn = make_uint2(0, 0);
-                if (kb + 2 < x.kb1) load2(kb + 2, nn);
-                if (!mbar_wait(su32(&bars->empty[stage]), phase ^ 1u, abort_flag, ctr, ERR_WAIT_MASK, wait_ns)) {
-                    ok = false;
-                    break;
-                }
+        Words cur, nxt;
+        bool has = fetch(cur), has_nxt = has && fetch(nxt);
+        while (has) {
+            Words nn;
+            const bool has_nn = has_nxt && fetch(nn);
+            uint32_t e[32];
+            expand_bits(cur.x, e);
+            expand_bits(cur.y, e + 16);
+            if (!mbar_wait(su32(&bars->empty[stage]), phase ^ 1u, abort_flag, ctr, ERR_WAIT_MASK, wait_ns)) {
+                // giving up: the copies already under way can then complete their stages' phases
+                for (int s2 = 0; s2 < STAGES; ++s2) mbar_arrive(su32(&bars->full[s2]));
+                break;
+            }
+            if (cur.live) {
                 uint8_t *brow = smem + stage * STAGE_BYTES + 2 * A_BYTES + r * 128;
-                if (r < ncols) {   // rows past the tile's columns are not read by the MMA
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint32_t w = c < 4 ? cur.x : cur.y;
-                        const uint2 lo = lut[(w >> (8 * (c & 3))) & 15u];
-                        const uint2 hi = lut[(w >> (8 * (c & 3) + 4)) & 15u];
-                        const uint32_t dst = su32(brow + ((c ^ (r & 7)) << 4));
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(lo.x), "r"(lo.y),
-                                     "r"(hi.x), "r"(hi.y)
-                                     : "memory");
-                    }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mbar_arrive(su32(&bars->b_full[stage]));
-                cur = nxt;
-                nxt = nn;
-                if (++stage == STAGES) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+                for (int c = 0; c < 8; ++c)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(su32(brow + ((c ^ (r & 7)) << 4))),
+                                 "r"(e[4 * c]), "r"(e[4 * c + 1]), "r"(e[4 * c + 2]), "r"(e[4 * c + 3])
+                                 : "memory");
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(su32(&bars->full[stage]));
+            cur = nxt;
+            nxt = nn;
+            has = has_nxt;
+            has_nxt = has_nn;
+            if (++stage == STAGES) {
+                stage = 0;
+                phase ^= 1u;
             }
         }
     }

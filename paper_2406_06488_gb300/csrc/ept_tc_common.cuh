@@ -106,6 +106,17 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void *tmap, int 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// true on one lane of a converged warp (the same one every time)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xFFFFFFFF;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r));
+    return r != 0;
+}
+
 // Shared-memory matrix descriptor, K-major, 128-byte swizzle: start address >> 4
 // (bits 0-13), leading byte offset 16 B (unused for swizzled K-major), stride byte
 // offset 1024 B between 8-row groups (bits 32-45), descriptor version 1 (bit 46),
@@ -157,14 +168,22 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
                  : "memory");
 }
 
-// 0/1 bits of `byte` -> eight FP16 values (1.0 = 0x3C00), element e = bit e.
-__device__ __forceinline__ uint4 expand8(uint32_t byte) {
-    uint4 v;
-    v.x = (byte & 1u) * 0x3C00u + (byte & 2u) * 0x1E000000u;
-    v.y = ((byte >> 2) & 1u) * 0x3C00u + ((byte >> 2) & 2u) * 0x1E000000u;
-    v.z = ((byte >> 4) & 1u) * 0x3C00u + ((byte >> 4) & 2u) * 0x1E000000u;
-    v.w = ((byte >> 6) & 1u) * 0x3C00u + ((byte >> 6) & 2u) * 0x1E000000u;
-    return v;
+// The 32 bits of w as FP16 values (1.0 = 0x3C00 where the bit is set), e[i] = bits 2 i and
+// 2 i + 1.  Sixteen columns at a time, the even bits in z's low half and the odd ones,
+// one place down, in its high half: then one bit of each is a mask away and 0x3C00 >> 2 i
+// times that is the pair (exact while 2 i <= 10; the last two pairs from z >> 4).  On the
+// logic and multiply pipes alone: a table in shared memory competes with the MMAs'
+// operand reads for its bandwidth.
+__device__ __forceinline__ void expand_bits(uint32_t w, uint32_t *e) {
+    const uint32_t z[2] = {__byte_perm(w, w << 15, 0x7610), __byte_perm(w, w >> 1, 0x7632)};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) e[8 * q + i] = (z[q] & (0x00010001u << (2 * i))) * (0x3C00u >> (2 * i));
+        const uint32_t y = z[q] >> 4;
+        e[8 * q + 6] = (y & (0x00010001u << 8)) * (0x3C00u >> 8);
+        e[8 * q + 7] = (y & (0x00010001u << 10)) * (0x3C00u >> 10);
+    }
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
@@ -179,6 +198,64 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
           "=r"(v[30]), "=r"(v[31])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// Sixteen TMEM lanes x 32 columns: thread l of the warp gets row l / 4 (registers 4 j, 4 j + 1)
+// and row l / 4 + 8 (4 j + 2, 4 j + 3) of columns 8 j + 2 (l mod 4) and the next, j = 0..3.
+// Asynchronous: tmem_wait_ld() before the registers are read.
+__device__ __forceinline__ void tmem_ld16x256(uint32_t taddr, uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The masked row sums of a 32 x 32 block of an accumulator (the warp's 32 TMEM lanes = rows at
+// taddr): for each of 32 relabelings the sum over the rows in its group.  w[j]: the mask
+// words of relabelings 8 j + 2 (lane mod 4) and the next for these rows (bit = row).  Returns the
+// sum of relabeling masked_sum_col(lane) of the block.
+// Rows are added in the order of a butterfly over row distances 16, 8, 4, 2, 1.  The 16 x 256-bit
+// load gives a thread rows r, r + 8, r + 16, r + 24 of eight relabelings, so that the first two
+// distances are additions within the thread and the mask bits need no transpose: 7
+// shuffles and about 130 instructions a block, where a thread holding one row of 32 relabelings
+// took 36 and 215.
+__device__ __forceinline__ int masked_sum_col(int lane) {
+    return 8 * (((lane >> 4) & 1) * 2 + ((lane >> 3) & 1)) + 2 * (lane & 3) + ((lane >> 2) & 1);
+}
+__device__ __forceinline__ float masked_block_sum(uint32_t taddr, const uint2 (&w)[4], int lane) {
+    uint32_t a[16], b[16];   // rows 0..15 and 16..31 of the block
+    tmem_ld16x256(taddr, a);
+    tmem_ld16x256(taddr + (16u << 16), b);
+    tmem_wait_ld();
+    const int r = lane >> 2;
+    float s[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t t = (e ? w[j].y : w[j].x) >> r;
+            const float x0 = (t & 0x00000001u) ? __uint_as_float(a[4 * j + e]) : 0.f;
+            const float x1 = (t & 0x00000100u) ? __uint_as_float(a[4 * j + 2 + e]) : 0.f;
+            const float x2 = (t & 0x00010000u) ? __uint_as_float(b[4 * j + e]) : 0.f;
+            const float x3 = (t & 0x01000000u) ? __uint_as_float(b[4 * j + 2 + e]) : 0.f;
+            s[2 * j + e] = (x0 + x2) + (x1 + x3);
+        }
+    }
+#pragma unroll
+    for (int off = 16, n = 4; off >= 4; off >>= 1, n >>= 1) {
+        const bool upper = (lane & off) != 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (k >= n) break;
+            const float send = upper ? s[k] : s[k + n];
+            const float keep = upper ? s[k + n] : s[k];
+            s[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, off);
+        }
+    }
+    return s[0];
 }
 
 }  // namespace tc
