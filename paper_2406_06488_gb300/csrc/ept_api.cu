@@ -2709,6 +2709,7 @@ ept_status ept_perm_masks(ept_ctx *c, uint64_t seed, int64_t nx, int64_t ny, int
     const size_t bytesR = (size_t)count * nwu * 4;
     ept_status st = ensure_arena(c, bytesT + bytesR, s);
     if (st != EPT_OK) return st;
+    c->urec_serial = 0;   // the masks take the arena from its start, over a cached plan's unit records
     uint32_t *maskT = (uint32_t *)c->arena;
     uint32_t *rows = on_device ? out : (uint32_t *)(c->arena + bytesT);
     launch_perm_masks_plain(seed, (int)nx, (int)ny, b0, count, (int)nw, maskT, s);
@@ -2737,6 +2738,7 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     if ((st = ensure_pinned(c, S.total)) != EPT_OK) return st;
     if (s != c->stream) CK(cudaStreamSynchronize(c->stream));
     c->tables_staged = false;   // the staging area now holds this call's tables
+    c->urec_serial = 0;         // and the arena its data, over a cached plan's unit records
     stage_host(c, P, specs, on_device != 0);
     uint8_t *A = c->arena;
     const Batch b = device_view(c, P);
