@@ -126,7 +126,10 @@ struct Plan {
     int64_t nrows = 0, npan = 0, ncols_pad = 0, nunits = 0, nsimt = 0, nblk = 0, nmask = 0, nchunk = 0, npart = 0,
             nstats = 0, p_stride = 0;
     size_t in_bytes = 0;              // host inputs copied into the arena
-    // byte offsets in the arena; the first tab_bytes are the uploaded tables
+    // byte offsets in the arena: the descriptors and zeroed counters (head_bytes, uploaded with every
+    // run), the results behind the counters, the constant tables (off_pre_rows up to tab_bytes,
+    // uploaded when the plan or the arena changes), then the data
+    size_t off_zero = 0, head_bytes = 0;   // (off_zero: the head's counters)
     size_t off_desc, off_pre_rows, off_pre_panels, off_pre_cols, off_pre_units, off_pre_simt, off_blk, off_tiles,
         off_chunks, off_sched, off_sched_off, off_urec, off_urec_pair, tab_bytes;
     size_t off_in, off_norms, off_iscale, off_u, off_Zh, off_Zl, off_D, off_Chi, off_rowpart, off_colpart,
@@ -329,6 +332,12 @@ void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host
     };
     const size_t nt1 = (size_t)P.n_tests + 1;
     P.off_desc = take(sizeof(TestDesc) * P.n_tests);
+    P.off_zero = P.off_ctr = take(sizeof(Counters) * P.n_tests);
+    P.head_bytes = o;
+    in_data = true;
+    P.off_observed = take((size_t)P.n_tests * 8);   // counters, observed, statistics: read back together
+    P.off_stats = take((size_t)P.nstats * 8);
+    in_data = false;
     P.off_pre_rows = take(8 * nt1);
     P.off_pre_panels = take(8 * nt1);
     P.off_pre_cols = take(8 * nt1);
@@ -367,11 +376,8 @@ void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host
     P.off_Stpart = take((size_t)P.npan * 8);
     P.off_maskT = take((size_t)P.nmask * 4);
     P.off_partial = take((size_t)P.npart * 4);
-    P.off_stats = take((size_t)P.nstats * 8);
     P.off_errest = take((size_t)P.nstats * 8);
     P.off_flags = take((size_t)P.nstats);
-    P.off_observed = take((size_t)P.n_tests * 8);
-    P.off_ctr = take(sizeof(Counters) * P.n_tests);
     P.off_sel_hist = P.any_median ? take((size_t)P.n_tests * 2048 * 4) : 0;
     P.total = o;
 }
@@ -632,6 +638,8 @@ struct ept_ctx {
     std::vector<int64_t> plan_key;
     bool tables_staged = false;
     uint64_t urec_serial = 0;           // plan whose unit records the arena holds (0: none)
+    uint64_t tab_serial = 0;            // plan whose constant tables it holds, and which arena
+    uint8_t *tab_arena = nullptr;
     uint8_t *urec_arena = nullptr;      // the arena they were uploaded to
     // host-to-device copies of this run's inputs: from the caller's buffers when they
     // are page-locked, else from the pinned staging area
@@ -732,7 +740,7 @@ ept_status ensure_arena(ept_ctx *c, size_t bytes, cudaStream_t s, bool exact = f
     if (st != EPT_OK) return st;
     c->arena = (uint8_t *)p;
     c->arena_cap = cap;
-    c->urec_serial = 0;   // a new arena holds no unit records
+    c->urec_serial = c->tab_serial = 0;   // a new arena holds neither records nor tables
     return EPT_OK;
 }
 
@@ -754,26 +762,34 @@ ept_status ensure_pinned(ept_ctx *c, size_t bytes) {
     return EPT_OK;
 }
 
-// Pinned staging layout: [tables (tab_bytes)] [inputs (in_bytes)] [results].
+// Pinned staging layout: [head] [constant tables] [inputs (in_bytes)] [results, laid out as in the arena].
 struct Staging {
-    size_t tables, inputs, res_ctr, res_obs, res_stats, total;
+    size_t head, tables, inputs, res_ctr, res_obs, res_stats, res_bytes, total;
 };
 
 Staging staging_layout(const Plan &P) {
     Staging S;
     size_t o = 0;
+    S.head = o;
+    o = align_up(o + P.head_bytes, 256);
     S.tables = o;
-    o = align_up(o + P.tab_bytes, 256);
+    o = align_up(o + P.tab_bytes - P.off_pre_rows, 256);
     S.inputs = o;
     o = align_up(o + P.in_bytes, 256);
     S.res_ctr = o;
-    o = align_up(o + sizeof(Counters) * P.n_tests, 256);
-    S.res_obs = o;
-    o = align_up(o + 8 * (size_t)P.n_tests, 256);
-    S.res_stats = o;
-    o = align_up(o + (P.host_in ? 8 * (size_t)P.nstats : 0), 256);
-    S.total = o;
+    S.res_obs = o + (P.off_observed - P.off_ctr);
+    S.res_stats = o + (P.off_stats - P.off_ctr);
+    S.res_bytes = P.host_in ? P.off_stats - P.off_ctr + 8 * (size_t)P.nstats
+                            : P.off_observed - P.off_ctr + 8 * (size_t)P.n_tests;
+    S.total = align_up(o + S.res_bytes, 256);
     return S;
+}
+
+// counters, observed statistics and (host outputs) permuted statistics in one copy
+ept_status read_back(ept_ctx *c, const Plan &P, cudaStream_t s) {
+    const Staging S = staging_layout(P);
+    CK(cudaMemcpyAsync(c->pinned + S.res_ctr, c->arena + P.off_ctr, S.res_bytes, cudaMemcpyDeviceToHost, s));
+    return EPT_OK;
 }
 
 bool page_locked(const void *p) {
@@ -846,9 +862,10 @@ void stage_host(ept_ctx *c, Plan &P, const std::vector<TestSpec> &specs, bool on
         c->in_copies.clear();
         c->in_copies.push_back({P.off_in, pin + S.inputs, P.in_bytes});
     }
-    uint8_t *tab = pin + S.tables;
-    memcpy(tab + P.off_desc, P.desc.data(), sizeof(TestDesc) * P.n_tests);
+    memcpy(pin + S.head + P.off_desc, P.desc.data(), sizeof(TestDesc) * P.n_tests);
     if (!tables) return;   // the shape-dependent tables are already in place
+    memset(pin + S.head + P.off_zero, 0, P.head_bytes - P.off_zero);   // uploaded as the run's zeroed counters
+    uint8_t *tab = pin + S.tables - P.off_pre_rows;
     memcpy(tab + P.off_pre_rows, P.pre_rows.data(), 8 * P.pre_rows.size());
     memcpy(tab + P.off_pre_panels, P.pre_panels.data(), 8 * P.pre_panels.size());
     memcpy(tab + P.off_pre_cols, P.pre_cols.data(), 8 * P.pre_cols.size());
@@ -933,21 +950,45 @@ int draw_mode_for(const ept_ctx *c, const Plan &P) {
 // The run's input copies on the copy stream (after `after`'s prior work), then ev_in:
 // the relabeling draws, which do not read the inputs, start while the copies run
 // (caller relabelings in host memory are inputs: their kernel waits for ev_in too).
+// Small inputs, and none, stay on `after`: crossing to the copy stream and back costs more
+// than it hides (small calls: about 3 us of 100).
+constexpr size_t SMALL_INPUT_BYTES = 256 << 10;
+
 ept_status enqueue_inputs(ept_ctx *c, cudaStream_t after) {
-    CK(cudaEventRecord(c->ev_user, after));
-    CK(cudaStreamWaitEvent(c->copy, c->ev_user, 0));
+    size_t bytes = 0;
+    for (const ept_ctx::InputCopy &k : c->in_copies) bytes += k.bytes;
+    cudaStream_t s = after;
+    if (bytes > SMALL_INPUT_BYTES) {
+        s = c->copy;
+        CK(cudaEventRecord(c->ev_user, after));
+        CK(cudaStreamWaitEvent(s, c->ev_user, 0));
+    }
     for (const ept_ctx::InputCopy &k : c->in_copies)
-        CK(cudaMemcpyAsync(c->arena + k.dst, k.src, k.bytes, cudaMemcpyHostToDevice, c->copy));
-    CK(cudaEventRecord(c->ev_in, c->copy));
+        CK(cudaMemcpyAsync(c->arena + k.dst, k.src, k.bytes, cudaMemcpyHostToDevice, s));
+    CK(cudaEventRecord(c->ev_in, s));
+    return EPT_OK;
+}
+
+// The descriptors and the zeroed counters, and the constant tables unless the arena holds
+// this plan's from its last run (any other use of the arena resets tab_serial).
+ept_status upload_tables(ept_ctx *c, const Plan &P, cudaStream_t s) {
+    const Staging S = staging_layout(P);
+    CK(cudaMemcpyAsync(c->arena, c->pinned + S.head, P.head_bytes, cudaMemcpyHostToDevice, s));
+    if (c->tab_serial != P.serial || c->tab_arena != c->arena) {
+        CK(cudaMemcpyAsync(c->arena + P.off_pre_rows, c->pinned + S.tables, P.tab_bytes - P.off_pre_rows,
+                           cudaMemcpyHostToDevice, s));
+        c->tab_serial = P.serial;
+        c->tab_arena = c->arena;
+    }
     return EPT_OK;
 }
 
 // The run's host-to-device traffic: the tables on s first (the copy engine takes
 // copies in order, so the small upload that the draws wait for goes ahead), then the
-// inputs on the copy stream.
+// inputs.
 ept_status enqueue_uploads(ept_ctx *c, const Plan &P, cudaStream_t s) {
-    const Staging S = staging_layout(P);
-    CK(cudaMemcpyAsync(c->arena, c->pinned + S.tables, P.tab_bytes, cudaMemcpyHostToDevice, s));
+    const ept_status st = upload_tables(c, P, s);
+    if (st != EPT_OK) return st;
     // the unit records stay in the arena while the same plan runs on it; a run of any
     // other plan may overwrite them
     if (P.urec.empty() && P.urec_pair.empty()) {
@@ -970,13 +1011,10 @@ ept_status enqueue_uploads(ept_ctx *c, const Plan &P, cudaStream_t s) {
 // waits for the inputs through ev_in as an external event.
 ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed, bool with_inputs = true) {
     ept_status st = EPT_OK;
-    const Staging S = staging_layout(P);
-    uint8_t *pin = c->pinned;
     const Batch b = device_view(c, P);
     const bool tc = P.prec == EPT_PREC_SPLIT_BF16;
     if (timed) CK(cudaEventRecord(c->ev[0], s));
     if (with_inputs && (st = enqueue_uploads(c, P, s)) != EPT_OK) return st;
-    CK(cudaMemsetAsync(b.ctr, 0, sizeof(Counters) * P.n_tests, s));
     if (P.any_median) CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)P.n_tests * 2048 * 4, s));
     if (P.debug) launch_guards(c->arena, P.guards, false, b.ctr, s);
     CK(cudaEventRecord(c->ev[1], s));
@@ -1035,9 +1073,7 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
     if (P.debug) launch_guards(c->arena, P.guards, true, b.ctr, s);   // after every write of the run
     if (timed) CK(cudaEventRecord(c->ev[3], s));
 
-    CK(cudaMemcpyAsync(pin + S.res_ctr, b.ctr, sizeof(Counters) * P.n_tests, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(pin + S.res_obs, b.observed, 8 * (size_t)P.n_tests, cudaMemcpyDeviceToHost, s));
-    if (P.host_in) CK(cudaMemcpyAsync(pin + S.res_stats, b.stats, 8 * (size_t)P.nstats, cudaMemcpyDeviceToHost, s));
+    if ((st = read_back(c, P, s)) != EPT_OK) return st;
     if (timed) CK(cudaEventRecord(c->ev[4], s));
     return EPT_OK;
 }
@@ -1356,10 +1392,7 @@ ept_status refine_after(ept_ctx *c, const Plan &P, const std::vector<TestSpec> &
     launch_reset_counts(b, s);
     launch_combine_count(b, s);
     CK(cudaGetLastError());
-    uint8_t *pin = c->pinned;
-    CK(cudaMemcpyAsync(pin + S.res_ctr, b.ctr, sizeof(Counters) * P.n_tests, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(pin + S.res_obs, b.observed, 8 * (size_t)P.n_tests, cudaMemcpyDeviceToHost, s));
-    if (P.host_in) CK(cudaMemcpyAsync(pin + S.res_stats, b.stats, 8 * (size_t)P.nstats, cudaMemcpyDeviceToHost, s));
+    if ((st = read_back(c, P, s)) != EPT_OK) return st;
     CK(cudaStreamSynchronize(s));
     const ept_status st2 = collect(c, P, specs, out, timed, per_test);
     for (int t = 0; st2 == EPT_OK && t < P.n_tests; ++t) out[t].refine_launches = launches;
@@ -1734,9 +1767,9 @@ void stream_layout(Plan &P, size_t tab_bytes_resident) {
     P.off_Stpart = take((size_t)P.npan * 8);
     P.off_maskT = take((size_t)P.nmask * 4);
     P.off_sacc = take((size_t)d.Bp * 8);
-    P.off_stats = take((size_t)P.nstats * 8);
-    P.off_observed = take(8);
     P.off_ctr = take(sizeof(Counters));
+    P.off_observed = take(8);
+    P.off_stats = take((size_t)P.nstats * 8);
     P.off_D = take((size_t)P.win_blk * PANEL * KB * 4);
     P.off_Chi = P.off_D;
     P.off_rowpart = take((size_t)P.win_blk * PANEL * 8);
@@ -1890,7 +1923,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
         g.user_masks = P.desc[0].user_masks;
         g.out_stats = P.desc[0].out_stats;
     }
-    uint8_t *tab = c->pinned + S.tables;
+    uint8_t *tab = c->pinned + S.tables - P.off_pre_rows;
     memcpy(tab + P.off_gdesc, P.gdesc.data(), sizeof(TestDesc) * P.gdesc.size());
     memcpy(tab + P.off_gpre, P.gpre.data(), 8 * P.gpre.size());
 
@@ -1957,9 +1990,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     CK(cudaGetLastError());
     if (P.debug) launch_guards(c->arena, P.guards, true, bf.ctr, s);
     CK(cudaEventRecord(c->ev[3], s));
-    CK(cudaMemcpyAsync(c->pinned + S.res_ctr, bf.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(c->pinned + S.res_obs, bf.observed, 8, cudaMemcpyDeviceToHost, s));
-    if (P.host_in) CK(cudaMemcpyAsync(c->pinned + S.res_stats, bf.stats, 8 * (size_t)P.nstats, cudaMemcpyDeviceToHost, s));
+    if ((st = read_back(c, P, s)) != EPT_OK) return st;
     CK(cudaEventRecord(c->ev[4], s));
     c->inject_stall = false;   // the hook is one-shot
     CK(cudaStreamSynchronize(s));
@@ -2001,9 +2032,9 @@ void pooled_layout(Plan &P, int num_sms) {
     P.off_maskT = take((size_t)P.nmask * 4);
     P.win_part = pooled_row_chunks(d.n, d.ncols, num_sms);   // row chunks of the sums
     P.off_partial = take((size_t)P.win_part * 3 * d.ncols * 8);
-    P.off_stats = take((size_t)P.nstats * 8);
-    P.off_observed = take(8);
     P.off_ctr = take(sizeof(Counters));
+    P.off_observed = take(8);
+    P.off_stats = take((size_t)P.nstats * 8);
     P.total = L.o;
 }
 
@@ -2070,9 +2101,7 @@ ept_status run_pooled(ept_ctx *c, const std::vector<TestSpec> &specs, bool on_de
     launch_combine_count(b, s);
     CK(cudaGetLastError());
     if (P.debug) launch_guards(c->arena, P.guards, true, b.ctr, s);
-    CK(cudaMemcpyAsync(c->pinned + S.res_ctr, b.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(c->pinned + S.res_obs, b.observed, 8, cudaMemcpyDeviceToHost, s));
-    if (P.host_in) CK(cudaMemcpyAsync(c->pinned + S.res_stats, b.stats, 8 * (size_t)P.nstats, cudaMemcpyDeviceToHost, s));
+    if ((st = read_back(c, P, s)) != EPT_OK) return st;
     CK(cudaEventRecord(c->ev[4], s));
     CK(cudaStreamSynchronize(s));
     if ((st = collect(c, P, specs, out, false)) != EPT_OK) return st;
@@ -2709,7 +2738,7 @@ ept_status ept_perm_masks(ept_ctx *c, uint64_t seed, int64_t nx, int64_t ny, int
     const size_t bytesR = (size_t)count * nwu * 4;
     ept_status st = ensure_arena(c, bytesT + bytesR, s);
     if (st != EPT_OK) return st;
-    c->urec_serial = 0;   // the masks take the arena from its start, over a cached plan's unit records
+    c->urec_serial = c->tab_serial = 0;   // the masks take the arena from its start, over a cached plan's
     uint32_t *maskT = (uint32_t *)c->arena;
     uint32_t *rows = on_device ? out : (uint32_t *)(c->arena + bytesT);
     launch_perm_masks_plain(seed, (int)nx, (int)ny, b0, count, (int)nw, maskT, s);
@@ -2738,11 +2767,11 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     if ((st = ensure_pinned(c, S.total)) != EPT_OK) return st;
     if (s != c->stream) CK(cudaStreamSynchronize(c->stream));
     c->tables_staged = false;   // the staging area now holds this call's tables
-    c->urec_serial = 0;         // and the arena its data, over a cached plan's unit records
+    c->urec_serial = c->tab_serial = 0;   // and the arena its data, over a cached plan's tables and records
     stage_host(c, P, specs, on_device != 0);
     uint8_t *A = c->arena;
     const Batch b = device_view(c, P);
-    CK(cudaMemcpyAsync(A, c->pinned + S.tables, P.tab_bytes, cudaMemcpyHostToDevice, s));
+    if ((st = upload_tables(c, P, s)) != EPT_OK) return st;
     if ((st = enqueue_inputs(c, s)) != EPT_OK) return st;
     CK(cudaStreamWaitEvent(s, c->ev_in, 0));
     CK(cudaMemsetAsync(b.ctr, 0, sizeof(Counters), s));
