@@ -1308,10 +1308,11 @@ ept_status refine_after(ept_ctx *c, const Plan &P, const std::vector<TestSpec> &
             if (f[j] == 2) list2.push_back((int32_t)j);
         }
         const int32_t nkc = (int32_t)refine_packed_chunks(d.NKB);
-        for (int64_t j = first1; j < (int64_t)list1.size(); j += REFINE_JOB_COLS) {
+        const int64_t job_cols = P.prec == EPT_PREC_SPLIT_BF16 ? REFINE_SPLIT_COLS : REFINE_JOB_COLS;
+        for (int64_t j = first1; j < (int64_t)list1.size(); j += job_cols) {
             RefineJob J;
             J.t = t;
-            J.ncol = (int32_t)std::min<int64_t>(REFINE_JOB_COLS, (int64_t)list1.size() - j);
+            J.ncol = (int32_t)std::min<int64_t>(job_cols, (int64_t)list1.size() - j);
             J.np = (int32_t)d.NP;
             J.nkc = nkc;
             J.list0 = j;
@@ -1347,7 +1348,7 @@ ept_status refine_after(ept_ctx *c, const Plan &P, const std::vector<TestSpec> &
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(djobs, jobs.data(), sizeof(RefineJob) * jobs.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) {
-            launch_refine_packed(b, djobs, (int64_t)jobs.size(), max_ctas, dlist1, dpart1, s);
+            launch_refine_packed(b, P.prec == EPT_PREC_SPLIT_BF16, djobs, (int64_t)jobs.size(), max_ctas, dlist1, dpart1, s);
             e = cudaGetLastError();
         }
     }

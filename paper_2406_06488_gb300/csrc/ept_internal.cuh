@@ -405,18 +405,20 @@ void launch_refine_finish(const Batch &b, int t, const int32_t *list, int64_t nf
                           const double *spart, int64_t ntiles, cudaStream_t s);
 void launch_reset_counts(const Batch &b, cudaStream_t s);   // n_ge = n_near = 0 before a recount
 // The statistics of flagged columns from the packed operand the contraction read,
-// summed exactly: one job per group of up to REFINE_JOB_COLS columns of one test
+// summed exactly: one job per group of up to REFINE_JOB_COLS (tensor-core path:
+// REFINE_SPLIT_COLS, what a thread sums at once) columns of one test
 // (list[list0 ..] test-local column indexes; part[part0 + g * ncol + k] for the
 // test's np x nkc (panel, chunk) pairs g, nkc = refine_packed_chunks(NKB)); every job
 // of a run in one launch (max_ctas = the largest np x nkc).
 constexpr int REFINE_JOB_COLS = 16;
+constexpr int REFINE_SPLIT_COLS = 8;
 struct RefineJob {
     int32_t t, ncol;
     int32_t np, nkc;
     int64_t list0, part0;
 };
 int64_t refine_packed_chunks(int64_t NKB);
-void launch_refine_packed(const Batch &b, const RefineJob *jobs, int64_t njobs, int64_t max_ctas,
+void launch_refine_packed(const Batch &b, bool split, const RefineJob *jobs, int64_t njobs, int64_t max_ctas,
                           const int32_t *list, double *part, cudaStream_t s);
 
 // single-draw-stream export (ept_perm_masks): columns 0..count-1 = draws b0..b0+count-1

@@ -236,31 +236,106 @@ __global__ void __launch_bounds__(256) k_refine_finish(const Batch bt, int t, co
 // recomputed from the packed, centred operand the contraction read, T = s'Cs, with
 // no accumulation error: on the tensor-core path every entry is c C_ij = hi + lo, two
 // FP16 numbers that are both multiples of 2^-24 with |hi + lo| < 2^15, so 2^24 c C_ij
-// is an integer below 2^39 and a row of up to 2^22 entries sums exactly in int64; on
+// is an integer below 2^39 and a panel's chunk of 256 x 512 entries sums exactly in int64; on
 // the plain path the FP32 entries are summed with TwoSum-compensated FP32 pairs.  The
-// rows' sums meet in FP64.  One launch serves every flagged test of a run: a job is
-// a group of up to 16 flagged columns of one test; CTA = (row panel I, chunk of RK
-// K-blocks) x job; thread = (row r of a 64-row quarter, 4 of the 16 columns).
+// parts meet in FP64.  One launch serves every flagged test of a run: a job is
+// a group of up to 8 (plain: 16) flagged columns of one test; CTA = (row panel I, chunk of RK
+// K-blocks) x job.
 constexpr int PCOLS = REFINE_JOB_COLS;
 constexpr int RK = 8;   // K-blocks per CTA
 
-// 2^24 x (an FP16 number), exactly, from its bits with integer operations: a normal
-// number (exponent field e >= 1) is (1024 + f) 2^(e - 25), a subnormal one f 2^-24
-// (f the 10-bit fraction); infinities and NaNs do not occur in the packed operand
-__device__ __forceinline__ long long fp16_fixed24(uint16_t bits) {
-    const int e = (bits >> 10) & 31, f = bits & 1023;
-    const long long mag = e ? (long long)(1024 + f) << (e - 1) : (long long)f;
-    return (bits & 0x8000u) ? -mag : mag;
+// 2^24 (hi + lo), exactly: the sum is exact in FP32 (lo is at most half a unit of hi's last place
+// and has 11 bits), 2^7 times it rounded to an integer A by adding 1.5 2^23 (|A| <= 2^22), and
+// the rest, at most 2^-8, is a multiple B of 2^-24 taken the same way.
+__device__ __forceinline__ long long packed_fixed24(__half hi, __half lo) {
+    const float magic = 12582912.f;
+    const float x = __half2float(hi) + __half2float(lo);
+    const float a = fmaf(x, 128.f, magic);
+    const float rest = fmaf(a - magic, -0.0078125f, x);
+    const float b = fmaf(rest, 16777216.f, magic);
+    const int A = __float_as_int(a) - 0x4B400000, B = __float_as_int(b) - 0x4B400000;
+    return ((long long)A << 17) + B;
 }
 
+// Tensor-core path.  Thread = (row of a 64-row quarter, 16 of a K-block's 64 columns): its 16
+// entries come in four 16-byte loads, become integers in registers, and each of the job's columns
+// adds those its mask selects; a row counts where its own bit is set.  All in integers, so the
+// order does not matter.  Flagged columns are few (28 of 2.5 million in a batch of 512
+// uneven tests, one or two to a test): four threads to a row share one column's work, where
+// a thread per row and four columns left most of them idle (that batch: 1.14 ms, now 0.10).
+__global__ void __launch_bounds__(256) k_refine_split(const Batch bt, const RefineJob *__restrict__ jobs,
+                                                      const int32_t *__restrict__ list, double *__restrict__ part) {
+    __shared__ uint32_t words[REFINE_SPLIT_COLS][2 * RK + PANEL / 32];   // the chunk's mask words, then the rows'
+    __shared__ long long tot_s[REFINE_SPLIT_COLS][8];
+    const RefineJob J = jobs[blockIdx.y];
+    if ((int64_t)blockIdx.x >= (int64_t)J.np * J.nkc) return;
+    const TestDesc &d = bt.desc[J.t];
+    const int64_t nkc = J.nkc;
+    const int64_t I = blockIdx.x / nkc, kc = blockIdx.x % nkc;
+    const int64_t nkb = contract_nkb(d);
+    const int64_t kb_lo = KB_PER_PANEL * I + kc * RK;
+    const int64_t kb_hi = kb_lo + RK < nkb ? kb_lo + RK : nkb;
+    for (int x = threadIdx.x; x < REFINE_SPLIT_COLS * (2 * RK + PANEL / 32); x += 256) {
+        const int k = x / (2 * RK + PANEL / 32), w = x % (2 * RK + PANEL / 32);
+        const int64_t word = w < 2 * RK ? 2 * kb_lo + w : I * (PANEL / 32) + w - 2 * RK;
+        words[k][w] = (k < J.ncol && word < d.nw) ? bt.maskT[d.mask0 + word * d.Bp + list[J.list0 + k]] : 0u;
+    }
+    __syncthreads();
+    const int r = threadIdx.x >> 2, q16 = threadIdx.x & 3;   // row of the quarter, 16-column part
+    long long tot[REFINE_SPLIT_COLS];
+#pragma unroll
+    for (int k = 0; k < REFINE_SPLIT_COLS; ++k) tot[k] = 0;
+    for (int64_t kb = kb_lo; kb < kb_hi; ++kb) {
+        const int64_t blk = d.blk0 + blk_index(I, kb, d.NKB);
+        const int w = (int)(kb - kb_lo) * 2 + (q16 >> 1), sh = (q16 & 1) * 16;
+#pragma unroll 1
+        for (int qr = 0; qr < 4; ++qr) {
+            const int64_t off = blk * bt.c_stride + (int64_t)(64 * qr + r) * KB + q16 * 16;
+            uint4 hv[2], lv[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                hv[e] = reinterpret_cast<const uint4 *>(bt.Chi + off)[e];
+                lv[e] = reinterpret_cast<const uint4 *>(bt.Clo + off)[e];
+            }
+            long long v[16];
+            const __half *hp = reinterpret_cast<const __half *>(hv), *lp = reinterpret_cast<const __half *>(lv);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = packed_fixed24(hp[e], lp[e]);
+#pragma unroll
+            for (int k = 0; k < REFINE_SPLIT_COLS; ++k) {
+                if (k >= J.ncol) break;   // uniform
+                const bool row = (words[k][2 * RK + 2 * qr + (r >> 5)] >> (r & 31)) & 1u;
+                const uint32_t m = row ? words[k][w] >> sh : 0u;
+                long long sum = 0;
+#pragma unroll
+                for (int e = 0; e < 16; ++e) sum += ((m >> e) & 1u) ? v[e] : 0ll;
+                tot[k] += sum;
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < REFINE_SPLIT_COLS; ++k) {
+        for (int off = 16; off; off >>= 1) tot[k] += __shfl_xor_sync(0xFFFFFFFFu, tot[k], off);
+        if ((threadIdx.x & 31) == 0) tot_s[k][threadIdx.x >> 5] = tot[k];
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < J.ncol) {
+        long long T = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) T += tot_s[threadIdx.x][w];
+        const double inv_c = (double)(1.f / packed_scale(bt.ctr[J.t]));   // a power of two
+        part[J.part0 + (I * nkc + kc) * J.ncol + threadIdx.x] = ldexp((double)T, -24) * inv_c;
+    }
+}
+
+// Plain path: thread = (row r of a 64-row quarter, 4 of the 16 columns).
 __global__ void __launch_bounds__(256) k_refine_packed(const Batch bt, const RefineJob *__restrict__ jobs,
                                                        const int32_t *__restrict__ list, double *__restrict__ part) {
-    // the values of 64 rows x 64 columns (int64 fixed point or FP32), then the sums
+    // the values of 64 rows x 64 columns, then the sums
     __shared__ __align__(16) uint8_t sm[PANEL * (PCOLS + 1) * 8];
-    long long(*vi)[KB + 1] = reinterpret_cast<long long(*)[KB + 1]>(sm);
     float(*vf)[KB + 1] = reinterpret_cast<float(*)[KB + 1]>(sm);
     double(*red)[PCOLS + 1] = reinterpret_cast<double(*)[PCOLS + 1]>(sm);
-    static_assert(64 * (KB + 1) * 8 <= PANEL * (PCOLS + 1) * 8, "value buffer");
+    static_assert(64 * (KB + 1) * 4 <= PANEL * (PCOLS + 1) * 8, "value buffer");
     const RefineJob J = jobs[blockIdx.y];
     if ((int64_t)blockIdx.x >= (int64_t)J.np * J.nkc) return;
     const int t = J.t;
@@ -268,7 +343,6 @@ __global__ void __launch_bounds__(256) k_refine_packed(const Batch bt, const Ref
     const int64_t nkc = J.nkc;
     const int64_t I = blockIdx.x / nkc, kc = blockIdx.x % nkc;
     const int r = threadIdx.x & 63, cg = threadIdx.x >> 6;   // row r of a 64-row quarter, columns 4 cg ..
-    const bool split = d.scaled != 0;
     const int64_t nkb = contract_nkb(d);
     const int64_t kb_lo = KB_PER_PANEL * I + kc * RK;
     const int64_t kb_hi = kb_lo + RK < nkb ? kb_lo + RK : nkb;
@@ -286,58 +360,32 @@ __global__ void __launch_bounds__(256) k_refine_packed(const Batch bt, const Ref
 #pragma unroll
     for (int qr = 0; qr < 4; ++qr) {   // the panel's four 64-row quarters
         const int64_t i = I * PANEL + 64 * qr + r;
-        long long si[4] = {0, 0, 0, 0};
         float sf[4] = {0.f, 0.f, 0.f, 0.f}, ef[4] = {0.f, 0.f, 0.f, 0.f};
         for (int64_t kb = kb_lo; kb < kb_hi; ++kb) {
             const int64_t blk = d.blk0 + blk_index(I, kb, d.NKB);
             __syncthreads();
             for (int x = threadIdx.x; x < 64 * KB; x += 256) {
                 const int rr = x / KB, cc = x % KB;
-                const int64_t off = (int64_t)(64 * qr + rr) * KB + cc;
-                if (split) {
-                    vi[rr][cc] = fp16_fixed24(bt.Chi[blk * bt.c_stride + off]) +
-                                 fp16_fixed24(bt.Clo[blk * bt.c_stride + off]);
-                } else {
-                    vf[rr][cc] = bt.D[blk * (int64_t)(PANEL * KB) + off];
-                }
+                vf[rr][cc] = bt.D[blk * (int64_t)(PANEL * KB) + (int64_t)(64 * qr + rr) * KB + cc];
             }
             __syncthreads();
             const int64_t w0 = kb * KB / 32;
-            uint32_t mw[4][2];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                mw[q][0] = col[q] < 0 ? 0u : bt.maskT[d.mask0 + w0 * d.Bp + col[q]];
-                mw[q][1] = col[q] < 0 ? 0u : bt.maskT[d.mask0 + (w0 + 1) * d.Bp + col[q]];
-            }
-            if (split) {
-                // each value read once from shared memory for the four columns
-#pragma unroll
-                for (int h2 = 0; h2 < 2; ++h2) {
-#pragma unroll 8
-                    for (int sh = 0; sh < 32; ++sh) {
-                        const long long x = vi[r][32 * h2 + sh];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) si[q] += ((mw[q][h2] >> sh) & 1u) ? x : 0ll;
-                    }
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 4 && !split; ++q) {
                 if (col[q] < 0) continue;
-                const uint32_t m0 = mw[q][0], m1 = mw[q][1];
-                {
-                    float sq = sf[q], eq = ef[q];
-                    for (int cc = 0; cc < KB; ++cc) {
-                        const uint32_t bit = cc < 32 ? (m0 >> cc) & 1u : (m1 >> (cc - 32)) & 1u;
-                        const float a = bit ? vf[r][cc] : 0.f;
-                        const float t2 = sq + a;   // TwoSum
-                        const float bb = t2 - sq;
-                        eq += (sq - (t2 - bb)) + (a - bb);
-                        sq = t2;
-                    }
-                    sf[q] = sq;
-                    ef[q] = eq;
+                const uint32_t m0 = bt.maskT[d.mask0 + w0 * d.Bp + col[q]];
+                const uint32_t m1 = bt.maskT[d.mask0 + (w0 + 1) * d.Bp + col[q]];
+                float sq = sf[q], eq = ef[q];
+                for (int cc = 0; cc < KB; ++cc) {
+                    const uint32_t bit = cc < 32 ? (m0 >> cc) & 1u : (m1 >> (cc - 32)) & 1u;
+                    const float a = bit ? vf[r][cc] : 0.f;
+                    const float t2 = sq + a;   // TwoSum
+                    const float bb = t2 - sq;
+                    eq += (sq - (t2 - bb)) + (a - bb);
+                    sq = t2;
                 }
+                sf[q] = sq;
+                ef[q] = eq;
             }
         }
         // this row's masked sum counts when the row is in the column's group
@@ -345,7 +393,7 @@ __global__ void __launch_bounds__(256) k_refine_packed(const Batch bt, const Ref
         for (int q = 0; q < 4; ++q) {
             if (col[q] < 0 || i >= d.n) continue;
             const uint32_t bit = (bt.maskT[d.mask0 + (i / 32) * d.Bp + col[q]] >> (i & 31)) & 1u;
-            if (bit) rowT[qr][q] = split ? ldexp((double)si[q], -24) : (double)sf[q] + (double)ef[q];
+            if (bit) rowT[qr][q] = (double)sf[q] + (double)ef[q];
         }
     }
     __syncthreads();
@@ -358,8 +406,7 @@ __global__ void __launch_bounds__(256) k_refine_packed(const Batch bt, const Ref
     if (threadIdx.x < J.ncol) {
         double T = 0.0;
         for (int rr = 0; rr < PANEL; ++rr) T += red[rr][threadIdx.x];
-        const double inv_c = split ? 1.0 / (double)packed_scale(bt.ctr[t]) : 1.0;
-        part[J.part0 + (I * nkc + kc) * J.ncol + threadIdx.x] = T * inv_c;
+        part[J.part0 + (I * nkc + kc) * J.ncol + threadIdx.x] = T;
     }
 }
 
@@ -388,11 +435,13 @@ __global__ void __launch_bounds__(32 * REFINE_JOB_COLS) k_refine_packed_finish(c
 
 int64_t refine_packed_chunks(int64_t NKB) { return (NKB + RK - 1) / RK; }
 
-void launch_refine_packed(const Batch &b, const RefineJob *jobs, int64_t njobs, int64_t max_ctas,
+void launch_refine_packed(const Batch &b, bool split, const RefineJob *jobs, int64_t njobs, int64_t max_ctas,
                           const int32_t *list, double *part, cudaStream_t s) {
     for (int64_t j0 = 0; j0 < njobs; j0 += 65535) {   // grid.y holds at most 65535 jobs
         const int64_t nj = njobs - j0 < 65535 ? njobs - j0 : 65535;
-        k_refine_packed<<<dim3((unsigned)max_ctas, (unsigned)nj), 256, 0, s>>>(b, jobs + j0, list, part);
+        const dim3 grid((unsigned)max_ctas, (unsigned)nj);
+        if (split) k_refine_split<<<grid, 256, 0, s>>>(b, jobs + j0, list, part);
+        else k_refine_packed<<<grid, 256, 0, s>>>(b, jobs + j0, list, part);
         k_refine_packed_finish<<<(unsigned)nj, 32 * REFINE_JOB_COLS, 0, s>>>(b, jobs + j0, list, part);
     }
 }
