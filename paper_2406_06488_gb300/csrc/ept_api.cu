@@ -124,7 +124,7 @@ struct Plan {
     int tc_grid = 0;                         // contraction CTAs
     std::vector<size_t> in_off;       // per test: byte offset of its X (then Y, then masks) in the input region
     int64_t nrows = 0, npan = 0, ncols_pad = 0, nunits = 0, nsimt = 0, nblk = 0, nmask = 0, nchunk = 0, npart = 0,
-            nstats = 0, p_stride = 0;
+            nstats = 0, p_stride = 0, parts_min = 0, parts_max = 0;
     size_t in_bytes = 0;              // host inputs copied into the arena
     // byte offsets in the arena: the descriptors and zeroed counters (head_bytes, uploaded with every
     // run), the results behind the counters, the constant tables (off_pre_rows up to tab_bytes,
@@ -289,6 +289,8 @@ void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host
         P.npart += d.nparts * d.Bp;
         P.nstats += d.ncols;
         P.p_stride = std::max(P.p_stride, d.p_pad);
+        P.parts_min = t == 0 ? d.nparts : std::min(P.parts_min, d.nparts);
+        P.parts_max = std::max(P.parts_max, d.nparts);
         push_pre(P.pre_rows, d.n_pad);
         push_pre(P.pre_panels, d.NP);
         push_pre(P.pre_cols, d.Bp);
@@ -907,6 +909,8 @@ Batch device_view(ept_ctx *c, const Plan &P) {
     b.nunits_total = P.nunits;
     b.nsimt_total = P.nsimt;
     b.p_stride = P.p_stride;
+    b.parts_min = P.parts_min;
+    b.parts_max = P.parts_max;
     b.norms = (float *)(A + P.off_norms);
     b.iscale = (float *)(A + P.off_iscale);
     b.u = (float *)(A + P.off_u);
@@ -1068,7 +1072,7 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
         CK(cudaGetLastError());
     }
     if (timed) CK(cudaEventRecord(c->ev[6], s));
-    launch_combine(b, s);
+    launch_combine(b, c->num_sms, s);
     CK(cudaGetLastError());
     if (P.debug) launch_guards(c->arena, P.guards, true, b.ctr, s);   // after every write of the run
     if (timed) CK(cudaEventRecord(c->ev[3], s));

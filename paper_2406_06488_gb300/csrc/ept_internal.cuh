@@ -209,6 +209,7 @@ struct Batch {
     int tc_grid;                         // contraction CTAs when scheduled
     int64_t nblk_total, ntiles, nrows_total, npan_total, ncols_total, nunits_total, nsimt_total;
     int64_t p_stride;                    // row stride of the FP16 rows (max p_pad)
+    int64_t parts_min, parts_max;        // fewest and most partials per column of a test
     float *norms, *iscale, *u;
     uint16_t *Zh, *Zl, *Chi, *Clo;       // Chi / Clo: the split parts of block b start at b * c_stride
     int64_t c_stride;
@@ -387,7 +388,7 @@ inline int draw_mode_auto(int64_t cols, int num_sms) {
 }
 void launch_masks(const Batch &b, int num_sms, int mode, cudaStream_t s);   // draws or caller masks
 void launch_contract_simt(const Batch &b, cudaStream_t s);
-void launch_combine(const Batch &b, cudaStream_t s);                     // statistics, flags, counts, outputs
+void launch_combine(const Batch &b, int num_sms, cudaStream_t s);                     // statistics, flags, counts, outputs
 void launch_combine_count(const Batch &b, cudaStream_t s);               // counts and outputs alone (recount)
 
 // ---- FP64 refinement of flagged statistics (ept_refine.cu): one test ----

@@ -1128,20 +1128,79 @@ void launch_contract_simt(const Batch &b, cudaStream_t s) {
 
 // ---------------------------------------------------------------------------
 // Final combination (Algorithm 1, statistic and p-value lines): per relabeling
-// column b, Q_b = sum of its partials, stat_b = sign * (cT Q_b + S~/o^2).  A CTA
-// covers 32 columns of one test (the column padding is a multiple of 256): lane l of
-// each of its 16 warps reads column l of every 16th partial (one coalesced 128-byte
-// row per load, eight loads in flight), and the 16 warp sums are added in a fixed
-// order (deterministic).
+// column b, Q_b = sum of its partials, stat_b = sign * (cT Q_b + S~/o^2).  The partials are summed
+// as unevaluated FP32 pairs (TwoSum: each addition's rounding error is kept exactly) of a
+// few each, which then meet in FP64 in a fixed order: this GPU's FP64 pipe takes 16 cycles for a
+// warp's operation, so that with FP64 per partial, or per few of them, it is the limit.
 // Then k_combine_count compares against stat_0 (the identity, evaluated by the same
 // kernels): stat_b >= stat_0 and near-ties |stat_b - stat_0| <= 1e-5 |stat_0|.
-__global__ void __launch_bounds__(512) k_combine_stats(const Batch bt) {
+// the statistic and the accumulation part of its error estimate (ept_internal.cuh, refine_ka)
+// from the sum q of a column's partials and the sum a of their magnitudes
+__device__ __forceinline__ void finish_stat(const Batch &bt, int t, const TestDesc &d, int64_t c, double q, double a,
+                                            double St) {
+    // the tensor-core path accumulates c Q (packed operand scaled by c); 1/c is exact
+    const double inv_c = d.scaled ? (double)(1.f / packed_scale(bt.ctr[t])) : 1.0;
+    bt.stats[d.col0 + c] = d.sign * (d.cT * (q * inv_c) + St * d.inv_o2);
+    if (bt.errest) bt.errest[d.col0 + c] = d.ka * REFINE_U * d.cT * (a * inv_c);
+}
+
+// Many columns (a batch): a thread per column (256 per CTA), eight partials at a time in one
+// pair (their loads in flight together), the pairs in FP64: three FP64 operations per eight
+// partials.  The kernel below makes 16 FP64 merges per column whatever its partials, 1.08 ms for 512
+// uneven tests (2.6 million columns, 50 partials on average, 0.5 GB); this one takes 0.29 ms.  It
+// needs two CTAs per SM to pay (COMBINE_COLUMNS_PER_SM): with few columns a thread's chain of loads
+// is longer than the sixteen warps' (5000 columns of 50 partials: 8 us against 6).  Tests of more
+// partials than COMBINE_THREAD_PARTS keep the other.
+constexpr int64_t COMBINE_THREAD_PARTS = 1024;
+constexpr int64_t COMBINE_COLUMNS_PER_SM = 512;
+__global__ void __launch_bounds__(256) k_combine_columns(const Batch bt) {
+    __shared__ double bSt;
+    const int64_t gc0 = (int64_t)blockIdx.x * 256;
+    const int t = find_test(bt.pre.cols, bt.n_tests, gc0);
+    const TestDesc &d = bt.desc[t];
+    const int64_t nparts = d.nparts;
+    if (nparts > COMBINE_THREAD_PARTS) return;
+    if (threadIdx.x < 32) {
+        const double St = warp_ordered_sum(bt.Stpart + d.pan0, d.NP);
+        if (threadIdx.x == 0) bSt = St;
+    }
+    __syncthreads();
+    const int64_t c = gc0 + threadIdx.x - bt.pre.cols[t];
+    if (c >= d.ncols) return;
+    const int64_t Bp = d.Bp;
+    const float *part = bt.partial + d.part0 + c;
+    double q = 0.0;
+    float aabs = 0.f;
+    for (int64_t k0 = 0; k0 < nparts; k0 += 8) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = k0 + k < nparts ? part[(k0 + k) * Bp] : 0.f;
+        float h = 0.f, l = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            float s2, e;
+            two_sum(h, v[k], s2, e);
+            h = s2;
+            l += e;
+            aabs += fabsf(v[k]);
+        }
+        q += (double)h + (double)l;
+    }
+    finish_stat(bt, t, d, c, q, (double)aabs, bSt);
+}
+
+// Tests of more partials: a CTA covers 32 columns of one test (the column padding is a multiple of
+// 256): lane l of each of its 16 warps reads column l of every 16th partial (one coalesced 128-byte
+// row per load, eight loads in flight), and the 16 warp sums are added in a fixed
+// order (deterministic).
+__global__ void __launch_bounds__(512) k_combine_stats(const Batch bt, int64_t above) {
     constexpr int NW = 16;   // warps: parts k = warp, warp + NW, ...
     __shared__ double bSt;
     __shared__ double ws[NW][32], wa[NW][32];
     const int64_t gc0 = (int64_t)blockIdx.x * 32;
     const int t = find_test(bt.pre.cols, bt.n_tests, gc0);
     const TestDesc &d = bt.desc[t];
+    if (d.nparts <= above) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {
         const double St = warp_ordered_sum(bt.Stpart + d.pan0, d.NP);
@@ -1260,10 +1319,13 @@ __global__ void __launch_bounds__(256) k_combine_count(const Batch bt, int flag)
     }
 }
 
-void launch_combine(const Batch &b, cudaStream_t s) {
+void launch_combine(const Batch &b, int num_sms, cudaStream_t s) {
     if (b.ncols_total <= 0) return;
     if (b.n_tests > 1) k_batch_status<<<1, 256, 0, s>>>(b);
-    k_combine_stats<<<(unsigned)(b.ncols_total / 32), 512, 0, s>>>(b);
+    const bool columns = b.ncols_total >= COMBINE_COLUMNS_PER_SM * num_sms && b.parts_min <= COMBINE_THREAD_PARTS;
+    if (columns) k_combine_columns<<<(unsigned)(b.ncols_total / 256), 256, 0, s>>>(b);
+    if (!columns || b.parts_max > COMBINE_THREAD_PARTS)
+        k_combine_stats<<<(unsigned)(b.ncols_total / 32), 512, 0, s>>>(b, columns ? COMBINE_THREAD_PARTS : 0);
     k_combine_count<<<(unsigned)(b.ncols_total / 256), 256, 0, s>>>(b, 1);
 }
 

@@ -211,6 +211,7 @@ extern "C" ept_status ept_test_static(const float *X, int64_t nx, const float *Y
     b.nrows_total = d.n_pad;
     b.npan_total = d.NP;
     b.ncols_total = d.Bp;
+    b.parts_min = b.parts_max = d.nparts;
     b.nunits_total = tc_units(d);
     b.norms = (float *)(A + P.norms);
     b.iscale = (float *)(A + P.iscale);
@@ -248,7 +249,7 @@ extern "C" ept_status ept_test_static(const float *X, int64_t nx, const float *Y
     if (!encode_block_tmaps(&th, &tl, b.Chi, b.Clo, d.nblk, b.c_stride, emsg, sizeof(emsg)))
         return err(EPT_ECUDA, "%s", emsg);
     SCK(launch_contract_tc(b, &th, &tl, sd->num_sms, s));
-    launch_combine(b, s);
+    launch_combine(b, sd->num_sms, s);
     SCK(cudaGetLastError());
     Counters h;
     double observed = 0.0;
