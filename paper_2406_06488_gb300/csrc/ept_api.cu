@@ -1046,7 +1046,7 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
         launch_norms(b, s);
         launch_build_simt(b, s);
     }
-    launch_median_select(b, s);
+    launch_median_select(b, c->num_sms, s);
     launch_blocksums(b, s);
     launch_rowsum_reduce(b, s);
     launch_center(b, s);
@@ -2793,7 +2793,7 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     if (P.any_median) {
         // median bandwidth: select it, then the block-sum pass turns distances into kernel values
         CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)2048 * 4, s));
-        launch_median_select(b, s);
+        launch_median_select(b, c->num_sms, s);
         launch_blocksums(b, s);
     }
     float *dout = on_device ? D_out : (float *)(A + P.total);

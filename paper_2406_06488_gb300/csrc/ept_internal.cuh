@@ -69,9 +69,11 @@ struct Counters {
     unsigned int max_d_bits;         // max |D_ij| over the stored blocks (FP32 bits; non-negative values
     unsigned int max_u_bits;         //   order like their bit patterns), max |u_i|,
     unsigned int max_dc_bits;        //   max |dcorr_i|: they bound |C| for the FP16 scale of the packing
-    unsigned int sel_prefix;         // median heuristic: radix-selection prefix, then the median's bits
+    unsigned int sel_prefix;         // median heuristic: start of the bracket, then the median's bits
+    unsigned int sel_shift, sel_bins, sel_state, sel_blocks;   //   its bins, the selection's state, blocks of the pass done
     unsigned int never_set;          // stays 0: the failure-path test hook waits for it
-    unsigned long long sel_k;        //   rank still to find within the prefix
+    unsigned long long sel_k;        //   rank still to find within the bracket
+    unsigned long long sel_below;    //   entries below the first bracket
     unsigned long long guard_bad;    // debug checks: words of the guard bands found overwritten
     unsigned long long batch_failed; // (test 0) some test of a batched call has an error: device outputs
                                      //   of the call are then left unwritten
@@ -366,7 +368,7 @@ __device__ __forceinline__ UnitRec unit_at_position(const Batch &bt, int64_t k) 
 void launch_norms(const Batch &b, cudaStream_t s);                       // plain path: norms + finite check
 void launch_build_simt(const Batch &b, cudaStream_t s);
 void launch_blocksums(const Batch &b, cudaStream_t s);   // median-heuristic tests: kernel transform first
-void launch_median_select(const Batch &b, cudaStream_t s);   // exact radix selection of the median distance
+void launch_median_select(const Batch &b, int num_sms, cudaStream_t s);   // exact selection of the median distance
 void launch_rowsum_reduce(const Batch &b, cudaStream_t s);
 void launch_center(const Batch &b, cudaStream_t s);
 void launch_pack(const Batch &b, bool split, cudaStream_t s);   // split: FP16 hi/lo (tensor-core path)

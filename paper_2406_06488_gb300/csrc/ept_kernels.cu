@@ -759,102 +759,243 @@ void launch_blocksums(const Batch &b, cudaStream_t s) {
 // Median heuristic (bandwidth of the MMD kernels): the lower median, rank
 // k = floor((N - 1) / 2) in ascending order, of the N = n (n - 1) / 2 distances
 // between distinct pooled rows (the strictly upper entries of the stored blocks).
-// Exact radix selection on the FP32 bit patterns (non-negative floats order like
-// their bits): three passes over digits of 11, 11 and 10 bits, most significant
-// first; each pass histograms the digit of the entries whose higher bits match the
-// prefix found so far (k_median_hist, one CTA per stored block, lanes with equal
-// digits aggregated before the shared-memory atomics) and then finds the bin that
-// holds rank k (k_median_pick, one CTA per test), which extends the prefix.  After
-// the last pass the prefix is the median's bit pattern (Counters::sel_prefix).
-__device__ __forceinline__ void sel_digit(int pass, uint32_t &mask, int &shift, uint32_t &dmask) {
-    mask = pass == 0 ? 0u : (pass == 1 ? 0xFFE00000u : 0xFFFFFC00u);
-    shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-    dmask = pass == 2 ? 0x3FFu : 0x7FFu;
+// Exact selection on the FP32 bit patterns (non-negative floats order like their
+// bits).  k_median_sample takes 16,384 entries at random and brackets the median six
+// standard deviations of its sample rank to either side, about 5 % of the entries.  A pass
+// (k_median_pass) counts the entries below the bracket in registers and
+// histograms those inside in 2048 equal bins; the last CTA of the test finds the bin
+// that holds rank k, which is the next pass's bracket, until the bins are single values.  The
+// first bracket is usually within 2^22 values, so two passes do it; a median outside it
+// (or a test with few pairs) starts again from all values, which takes three.  Four
+// passes are launched, those left return at once.
+// A pass reads every stored entry once (n = 10,500: 224 MB) and adds to shared memory for one
+// entry in twenty; histograms of the leading digits of every entry took 167 us a pass,
+// three times, since distances share a few leading digits; now 28 us for the sample, 84 and 73 us for the
+// passes that do the work and 7 us for the two that return.
+constexpr int MED_SAMPLES = 16384, MED_BINS = 2048, MED_PASSES = 4;
+
+// state of a test's selection (Counters): values [lo, lo + nbins << shift), rank k among
+// the entries from `lo` on (first pass: from 0 on)
+enum { MED_SAMPLED = 1, MED_INSIDE = 2, MED_DONE = 3 };
+
+__device__ __forceinline__ uint32_t mix32(uint32_t x) {
+    x ^= x >> 16;
+    x *= 0x85EBCA6Bu;
+    x ^= x >> 13;
+    x *= 0xC2B2AE35u;
+    return x ^ (x >> 16);
 }
 
-__global__ void __launch_bounds__(256) k_median_hist(const Batch bt, int pass) {
-    __shared__ uint32_t hist[2048];
-    const int64_t gb = blockIdx.x;
-    const BlkInfo bi = bt.blk[gb];
-    const TestDesc &d = bt.desc[bi.t];
-    if (!d.median) return;
-    for (int k = threadIdx.x; k < 2048; k += 256) hist[k] = 0u;
+// The bin of h[0 .. MED_BINS) that holds rank k, and the number of entries in the bins before it
+// (bin -1: k is past the end); every thread of the CTA (T threads, a multiple of 32) gets both.
+template <int T>
+__device__ __forceinline__ int find_bin(const uint32_t *h, unsigned long long k, unsigned long long &before) {
+    constexpr int PER = MED_BINS / T;
+    __shared__ unsigned long long wsum[T / 32];
+    __shared__ int bin_s;
+    __shared__ unsigned long long before_s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long mine = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) mine += h[threadIdx.x * PER + q];
+    unsigned long long inc = mine;   // inclusive over the warp
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+        if (lane >= off) inc += o;
+    }
+    if (threadIdx.x == 0) bin_s = -1;
+    if (lane == 31) wsum[warp] = inc;
     __syncthreads();
-    uint32_t mask, dmask;
-    int shift;
-    sel_digit(pass, mask, shift, dmask);
-    const uint32_t prefix = bt.ctr[bi.t].sel_prefix;
-    const int64_t n = d.n;
-    const float *base = bt.D + gb * (int64_t)(PANEL * KB);
-    for (int e = threadIdx.x; e < PANEL * KB; e += 256) {
-        const int64_t i = (int64_t)bi.I * PANEL + (e >> 6), j = (int64_t)bi.kb * KB + (e & 63);
-        const uint32_t v = __float_as_uint(base[e]);
-        const bool take = i < n && j < n && j > i && (v & mask) == prefix;
-        const uint32_t bin = take ? ((v >> shift) & dmask) : 0xFFFFFFFFu;
-        const uint32_t peers = __match_any_sync(0xFFFFFFFFu, bin);
-        if (take && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&hist[bin], (uint32_t)__popc(peers));
+    unsigned long long base = 0;
+    for (int w = 0; w < warp; ++w) base += wsum[w];
+    unsigned long long cum = base + inc - mine;   // entries before this thread's bins
+    if (k >= cum && k < cum + mine) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const unsigned long long c = h[threadIdx.x * PER + q];
+            if (k >= cum && k < cum + c) {
+                bin_s = threadIdx.x * PER + q;
+                before_s = cum;
+            }
+            cum += c;
+        }
     }
     __syncthreads();
-    uint32_t *gh = bt.sel_hist + (int64_t)bi.t * 2048;
-    for (int k = threadIdx.x; k < 2048; k += 256)
-        if (hist[k]) atomicAdd(&gh[k], hist[k]);
+    before = before_s;
+    const int bin = bin_s;
+    __syncthreads();
+    return bin;
 }
 
-__global__ void __launch_bounds__(256) k_median_pick(const Batch bt, int pass) {
-    __shared__ unsigned long long part[256];
-    __shared__ int owner;
-    __shared__ unsigned long long before;
+__global__ void __launch_bounds__(1024) k_median_sample(const Batch bt) {
+    __shared__ uint32_t h[2][MED_BINS];
     const int t = blockIdx.x;
     const TestDesc &d = bt.desc[t];
     if (!d.median) return;
-    uint32_t mask, dmask;
-    int shift;
-    sel_digit(pass, mask, shift, dmask);
-    const int nbins = (int)dmask + 1, per = nbins / 256;
-    uint32_t *gh = bt.sel_hist + (int64_t)t * 2048;
     Counters *c = bt.ctr + t;
+    constexpr int PER = MED_SAMPLES / 1024;
+    uint32_t v[PER];
+    int cnt = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const uint32_t s = (uint32_t)(q * 1024 + threadIdx.x);
+        const int64_t gb = d.blk0 + (int64_t)(((uint64_t)mix32(s * 2u + 1u) * (uint64_t)d.nblk) >> 32);
+        const int e = (int)(mix32(s * 2u + 2u) & (PANEL * KB - 1));
+        const BlkInfo bi = bt.blk[gb];
+        const int64_t i = (int64_t)bi.I * PANEL + (e >> 6), j = (int64_t)bi.kb * KB + (e & 63);
+        const bool take = i < d.n && j < d.n && j > i;
+        v[q] = take ? __float_as_uint(bt.D[gb * (int64_t)(PANEL * KB) + e]) : 0xFFFFFFFFu;
+        cnt += take;
+    }
+    for (int k = threadIdx.x; k < MED_BINS; k += 1024) h[0][k] = 0u;
+    __shared__ int cnt_s;
+    if (threadIdx.x == 0) cnt_s = 0;
+    __syncthreads();
+    for (int off = 16; off; off >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, off);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&cnt_s, cnt);
+    // leading 11 of 31 bits: lanes with equal digits aggregated
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const uint32_t bin = v[q] >> 20;
+        const uint32_t peers = __match_any_sync(0xFFFFFFFFu, bin);
+        if (bin < MED_BINS && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&h[0][bin], (uint32_t)__popc(peers));
+    }
+    __syncthreads();
+    const int m = cnt_s;
+    const int spread = (int)(3.f * sqrtf((float)m)) + 2;   // six standard deviations of the median's sample rank
+    const int r0 = m / 2 - spread, r1 = m / 2 + spread;
     const unsigned long long npairs = (unsigned long long)d.n * (unsigned long long)(d.n - 1) / 2ull;
-    const unsigned long long k = pass == 0 ? (npairs - 1ull) / 2ull : c->sel_k;
-    unsigned long long mine = 0;
-    for (int q = 0; q < per; ++q) mine += gh[threadIdx.x * per + q];
-    part[threadIdx.x] = mine;
-    if (threadIdx.x == 0) owner = -1;
-    __syncthreads();
+    uint32_t lo = 0, width = 0x80000000u;
+    if (r0 > 0 && r1 < m) {
+        unsigned long long b0, b1;
+        const int p0 = find_bin<1024>(h[0], (unsigned long long)r0, b0);
+        const int p1 = find_bin<1024>(h[0], (unsigned long long)r1, b1);
+        for (int k = threadIdx.x; k < MED_BINS; k += 1024) h[0][k] = h[1][k] = 0u;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {   // the next 11 bits of the entries that share either digit
+            const uint32_t lead = v[q] >> 20, next = (v[q] >> 9) & (MED_BINS - 1);
+            if (lead == (uint32_t)p0) atomicAdd(&h[0][next], 1u);
+            if (lead == (uint32_t)p1) atomicAdd(&h[1][next], 1u);
+        }
+        __syncthreads();
+        unsigned long long x;
+        const int q0 = find_bin<1024>(h[0], (unsigned long long)r0 - b0, x);
+        const int q1 = find_bin<1024>(h[1], (unsigned long long)r1 - b1, x);
+        lo = ((uint32_t)p0 << 20) | ((uint32_t)q0 << 9);
+        width = (((uint32_t)p1 << 20) | ((uint32_t)q1 << 9)) + 512u - lo;
+    }
     if (threadIdx.x == 0) {
-        unsigned long long cum = 0;
-        for (int q = 0; q < 256; ++q) {
-            if (k < cum + part[q]) {
-                owner = q;
-                before = cum;
-                break;
-            }
-            cum += part[q];
-        }
+        int shift = 0;
+        while (((width - 1u) >> shift) >= (uint32_t)MED_BINS) ++shift;
+        c->sel_prefix = lo;
+        c->sel_shift = shift;
+        c->sel_bins = ((width - 1u) >> shift) + 1u;
+        c->sel_k = (npairs - 1ull) / 2ull;
+        c->sel_state = MED_SAMPLED;
     }
-    __syncthreads();
-    if ((int)threadIdx.x == owner) {
-        unsigned long long cum = before;
-        for (int q = 0; q < per; ++q) {
-            const unsigned long long h = gh[threadIdx.x * per + q];
-            if (k < cum + h) {
-                c->sel_prefix |= (uint32_t)(threadIdx.x * per + q) << shift;
-                c->sel_k = k - cum;
-                break;
-            }
-            cum += h;
-        }
-    }
-    if (owner < 0 && threadIdx.x == 0) c->sel_prefix = 0u;   // counts do not add up: reported as a zero bandwidth
-    __syncthreads();
-    for (int q = 0; q < per; ++q) gh[threadIdx.x * per + q] = 0u;   // ready for the next pass
 }
 
-void launch_median_select(const Batch &b, cudaStream_t s) {
-    if (!b.sel_hist || b.nblk_total <= 0) return;
-    for (int pass = 0; pass < 3; ++pass) {
-        k_median_hist<<<(unsigned)b.nblk_total, 256, 0, s>>>(b, pass);
-        k_median_pick<<<(unsigned)b.n_tests, 256, 0, s>>>(b, pass);
+// One pass over the stored entries: a CTA takes a run of consecutive blocks, and hands its
+// histogram over where the test changes and at the end.
+__global__ void __launch_bounds__(256) k_median_pass(const Batch bt) {
+    __shared__ uint32_t hist[MED_BINS];
+    __shared__ bool last_s;
+    const int64_t b0 = bt.nblk_total * (int64_t)blockIdx.x / gridDim.x;
+    const int64_t b1 = bt.nblk_total * (int64_t)(blockIdx.x + 1) / gridDim.x;
+    int64_t gb = b0;
+    while (gb < b1) {
+        const int t = bt.blk[gb].t;
+        const TestDesc &d = bt.desc[t];
+        const int64_t end = d.blk0 + d.nblk < b1 ? d.blk0 + d.nblk : b1;   // this test's blocks of the run
+        Counters *c = bt.ctr + t;
+        if (!d.median || c->sel_state == MED_DONE) {
+            gb = end;
+            continue;
+        }
+        const uint32_t lo = c->sel_prefix, shift = c->sel_shift, bins = c->sel_bins;
+        const int64_t n = d.n;
+        for (int k = threadIdx.x; k < MED_BINS; k += 256) hist[k] = 0u;
+        __syncthreads();
+        uint32_t below = 0;
+        const unsigned int nb = (unsigned int)(end - gb);
+        for (; gb < end; ++gb) {
+            const BlkInfo bi = bt.blk[gb];
+            const int64_t i0 = (int64_t)bi.I * PANEL, j0 = (int64_t)bi.kb * KB;
+            const bool inside = i0 + PANEL <= n && j0 + KB <= n && j0 >= i0 + PANEL;   // every entry counts
+            const float4 *base = reinterpret_cast<const float4 *>(bt.D + gb * (int64_t)(PANEL * KB));
+#pragma unroll 1
+            for (int q0 = 0; q0 < PANEL * KB / 4 / 256; q0 += 8) {
+                float4 f[8];   // the loads first: they do not move past the histogram's atomics
+#pragma unroll
+                for (int q = 0; q < 8; ++q) f[q] = base[(q0 + q) * 256 + threadIdx.x];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int x = (q0 + q) * 256 + threadIdx.x;
+                    const uint32_t u[4] = {__float_as_uint(f[q].x), __float_as_uint(f[q].y), __float_as_uint(f[q].z),
+                                           __float_as_uint(f[q].w)};
+                    const int64_t i = i0 + (x >> 4), j = j0 + (x & 15) * 4;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (!inside && !(i < n && j + e < n && j + e > i)) continue;
+                        const uint32_t bin = (u[e] - lo) >> shift;   // below `lo`: wraps past the bins
+                        below += u[e] < lo;
+                        if (u[e] >= lo && bin < bins) atomicAdd(&hist[bin], 1u);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        uint32_t *gh = bt.sel_hist + (int64_t)t * MED_BINS;
+        for (int k = threadIdx.x; k < MED_BINS; k += 256)
+            if (hist[k]) atomicAdd(&gh[k], hist[k]);
+        for (int off = 16; off; off >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, off);
+        if ((threadIdx.x & 31) == 0 && below) atomicAdd(&c->sel_below, (unsigned long long)below);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last_s = atomicAdd(&c->sel_blocks, nb) + nb == (unsigned int)d.nblk;
+        __syncthreads();
+        if (!last_s) continue;
+        // the test's last CTA: the bin of rank k
+        __threadfence();
+        for (int k = threadIdx.x; k < MED_BINS; k += 256) {
+            hist[k] = __ldcg(&gh[k]);
+            gh[k] = 0u;   // ready for the next pass
+        }
+        __syncthreads();
+        const bool first = c->sel_state == MED_SAMPLED;
+        const unsigned long long under = first ? __ldcg(&c->sel_below) : 0ull, k = c->sel_k;
+        unsigned long long before = 0;
+        const int bin = k >= under ? find_bin<256>(hist, k - under, before) : -1;   // uniform
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            c->sel_blocks = 0u;
+            if (bin < 0) {
+                // outside the sampled bracket: from all values; else the counts do not add up
+                // (reported as a zero bandwidth)
+                c->sel_state = first ? MED_INSIDE : MED_DONE;
+                c->sel_prefix = 0u;
+                c->sel_shift = 20;
+                c->sel_bins = MED_BINS;
+            } else {
+                c->sel_prefix = lo + ((uint32_t)bin << shift);
+                c->sel_k = k - under - before;
+                c->sel_state = shift == 0 ? MED_DONE : MED_INSIDE;
+                c->sel_shift = shift > 11 ? shift - 11 : 0;
+                c->sel_bins = 1u << (shift < 11 ? shift : 11);
+            }
+        }
+        __syncthreads();
     }
+}
+
+void launch_median_select(const Batch &b, int num_sms, cudaStream_t s) {
+    if (!b.sel_hist || b.nblk_total <= 0) return;
+    k_median_sample<<<(unsigned)b.n_tests, 1024, 0, s>>>(b);
+    // as many CTAs as are resident at once (five of 48 registers a thread): 84 + 73 us with five per SM,
+    // 117 + 102 with six (a second wave), 113 + 101 with three
+    const int64_t full = (int64_t)5 * num_sms, grid = b.nblk_total < full ? b.nblk_total : full;
+    for (int pass = 0; pass < MED_PASSES; ++pass) k_median_pass<<<(unsigned)grid, 256, 0, s>>>(b);
 }
 
 // r_i = sum over the stored blocks of row i's panel (its own row segments) + sum
