@@ -1015,8 +1015,9 @@ ept_status enqueue_uploads(ept_ctx *c, const Plan &P, cudaStream_t s) {
 // waits for the inputs through ev_in as an external event.
 ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed, bool with_inputs = true) {
     ept_status st = EPT_OK;
-    const Batch b = device_view(c, P);
+    Batch b = device_view(c, P);
     const bool tc = P.prec == EPT_PREC_SPLIT_BF16;
+    b.build_sums = tc ? 1 : 0;
     if (timed) CK(cudaEventRecord(c->ev[0], s));
     if (with_inputs && (st = enqueue_uploads(c, P, s)) != EPT_OK) return st;
     if (P.any_median) CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)P.n_tests * 2048 * 4, s));
@@ -1047,7 +1048,7 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
         launch_build_simt(b, s);
     }
     launch_median_select(b, c->num_sms, s);
-    launch_blocksums(b, s);
+    if (!tc || P.any_median) launch_blocksums(b, tc, s);
     launch_rowsum_reduce(b, s);
     launch_center(b, s);
     launch_pack(b, tc, s);
@@ -1966,9 +1967,10 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     }
     // pass 1: the row sums r (and max |D| for the FP16 scale)
     for (int g = 0; g < nwin; ++g) {
-        const Batch gv = stream_view(c, P, g);
+        Batch gv = stream_view(c, P, g);
+        gv.build_sums = 1;
+        CK(cudaMemsetAsync(gv.colpart, 0, (size_t)P.gnblk[(size_t)g] * KB * 8, s));
         CK(launch_build_tc(gv, tm, c->num_sms, s));
-        launch_blocksums(gv, s);
         launch_stream_rowsums(gv, P.gI0[(size_t)g], P.gI1[(size_t)g], d.n_pad, s);
         CK(cudaGetLastError());
     }
@@ -2794,7 +2796,7 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
         // median bandwidth: select it, then the block-sum pass turns distances into kernel values
         CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)2048 * 4, s));
         launch_median_select(b, c->num_sms, s);
-        launch_blocksums(b, s);
+        launch_blocksums(b, true, s);
     }
     float *dout = on_device ? D_out : (float *)(A + P.total);
     launch_expand_blocks(b.D, nx + ny, P.desc[0].NKB, dout, s);

@@ -32,9 +32,13 @@
 // swizzle, conflict-free 16-byte stores) and one TMA store writes it, two buffers per
 // warp.  Three stages of 48 KB (K = 32) leave the 64 KB for that; two of 96 KB did
 // not.  The entries are formed in pairs with packed FP32 arithmetic (the same roundings).
-// n = 20,000, p = 100: Gaussian 483 -> 265 us (3.1 TB/s of entries), distances 218 us; n = 5000,
-// p = 200: 43 -> 28 us, p = 1000 (tensor pipe 70 % busy) 65 -> 59 us; n = 200, p = 10 (close
-// pairs recomputed) 27 -> 16 us.
+// The epilogue also sums the entries it holds: a thread its row (two pairs at once), a warp the columns
+// of each group from its buffer, the four warps of a column half through shared memory, the
+// two row halves of a panel by two additions to a zeroed FP64 sum (two terms commute).  That
+// spares k_blocksums and its pass over every stored entry.
+// n = 20,000, p = 100: Gaussian 483 us and 197 for the sums -> 265 without sums, 434 with them; n = 5000,
+// p = 200: 43 + 17 -> 38 us, p = 1000 (tensor pipe 70 % busy) 65 + 21 -> 62 us; n = 200, p = 10 (close
+// pairs recomputed) 27 + 11 -> 21 us.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -61,11 +65,12 @@ constexpr int OUT_BYTES = 32 * 32 * 4;                // a staged 32 x 32 group 
 constexpr int NUM_THREADS = 320;   // TMA warp, MMA warp, 8 epilogue warps
 constexpr int EPI_THREADS = 256;
 // stages | per-epilogue-warp output groups (8 x 2 x 4 KB) | barriers (1 KB) | per-epilogue-warp column norms and
-// scales (8 x 1 KB) | alignment slack
+// scales (8 x 1 KB) | per-epilogue-warp column sums (8 x 1 KB) | alignment slack
 constexpr int OUT_OFF = STAGES * STAGE_BYTES;
 constexpr int BAR_OFF = OUT_OFF + 8 * 2 * OUT_BYTES;
 constexpr int COL_OFF = BAR_OFF + 1024;
-constexpr int SMEM_BYTES = COL_OFF + 8 * (PANEL / 2) * 8 + 1024;
+constexpr int SUM_OFF = COL_OFF + 8 * (PANEL / 2) * 8;
+constexpr int SMEM_BYTES = SUM_OFF + 8 * (PANEL / 2) * 8 + 1024;
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of the build");
 // kind::f16 instruction descriptor with A = B = FP16 (format 0), D = FP32, K-major
 constexpr uint32_t IDESC = idesc_f16_f32(BM, BN);
@@ -104,6 +109,11 @@ __global__ void __launch_bounds__(256) k_split_rows(const Batch bt) {
     const int64_t i = gr - d.row0;
     const int64_t p = d.p, p_pad = d.p_pad;
     const float *z = (i < d.n) ? row_ptr(d, i) : nullptr;
+    if (bt.build_sums) {   // the column sums that the build adds to
+        const int64_t threads = (int64_t)gridDim.x * blockDim.x;
+        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < bt.nblk_total * KB; k += threads)
+            bt.colpart[k] = 0.0;
+    }
     uint32_t mx = 0;
     bool bad = false;
     if (z) {
@@ -183,6 +193,40 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     f32x2 r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// (h, l) += v on two sums at once, each an unevaluated pair (TwoSum, the rounding error kept in l)
+__device__ __forceinline__ void pair_add2(f32x2 &h, f32x2 &l, f32x2 v) {
+    const f32x2 s = add2(h, v), bb = sub2(s, h);
+    l = add2(l, add2(sub2(h, sub2(s, bb)), sub2(v, bb)));
+    h = s;
+}
+// the two sums added: the pair's value
+__device__ __forceinline__ void pair_join(f32x2 h, f32x2 l, float &hs, float &ls) {
+    float h0, h1, l0, l1, e;
+    unpack2(h, h0, h1);
+    unpack2(l, l0, l1);
+    two_sum(h0, h1, hs, e);
+    ls = (l0 + l1) + e;
+}
+
+// Barriers of the four warps that share a half of the tile's columns: 0, before a tile's column
+// sums are written (the last tile's are read); 1, when they are.  A warp that gives up arrives at both.
+__device__ __forceinline__ void half_sync(int half, int which) {
+    if (half == 0 && which == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+    else if (half == 0) asm volatile("bar.sync 2, 128;" ::: "memory");
+    else if (which == 0) asm volatile("bar.sync 3, 128;" ::: "memory");
+    else asm volatile("bar.sync 4, 128;" ::: "memory");
+}
+__device__ __forceinline__ void half_leave(int half) {
+    if (half == 0) asm volatile("bar.arrive 1, 128;\n\tbar.arrive 2, 128;" ::: "memory");
+    else asm volatile("bar.arrive 3, 128;\n\tbar.arrive 4, 128;" ::: "memory");
 }
 
 // exp_cw of two arguments x in [-87, 0] (its operations in its order; outside the
@@ -470,6 +514,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         float *colv = reinterpret_cast<float *>(smem + COL_OFF) + (warp - 2) * PANEL;
         uint8_t *outb = smem + OUT_OFF + (warp - 2) * 2 * OUT_BYTES;
         int ob = 0;   // output buffer of the next group
+        float2 *colsum = reinterpret_cast<float2 *>(smem + SUM_OFF);   // [warp][column of the half]
         int acc = 0;
         uint32_t acc_phase = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -484,6 +529,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             // first row of the warp's 32 in the block array (rows of 64 entries)
             const int64_t drow = (d.blk0 + blk_index(tile.I, (int64_t)tile.J * KB_PER_PANEL, NKB)) * PANEL +
                                  tile.h * BM + quarter * 32;
+            // the blocks' row and column sums and largest entry (a median test's come from its
+            // kernel values, in k_blocksums)
+            const bool sums = bt.build_sums && !d.median;
+            f32x2 rh = 0, rl = 0;   // the row's even and odd columns of a K-block
+            float mx = 0.f;
+            if (sums) half_sync(half, 0);
             unsigned fixups = 0;
             const int rp = tile.h * BM + rt;                 // row within panel I
             const int64_t i = (int64_t)tile.I * PANEL + rp;  // pooled row of the test
@@ -500,8 +551,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             __syncwarp();
             // the warp's lanes leave together (the group loop below synchronises them)
             if (!__all_sync(0xFFFFFFFFu, mbar_wait(su32(&bars->acc_full[acc]), acc_phase, abort_flag, ctr, ERR_WAIT_EPI,
-                                                   wait_ns)))
+                                                   wait_ns))) {
+                half_leave(half);
                 break;
+            }
             fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
@@ -543,6 +596,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     *reinterpret_cast<float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4)) =
                         make_float4(out[4 * c], out[4 * c + 1], out[4 * c + 2], out[4 * c + 3]);
                 // cancellation-prone pairs: d^2 by direct differences
+                const bool fixed = fix != 0u;
                 while (fix) {
                     const int e = __ffs(fix) - 1;
                     fix &= fix - 1u;
@@ -553,6 +607,29 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     *reinterpret_cast<float *>(buf + lane * 128 + (((e >> 2) ^ (lane & 7)) << 4) + (e & 3) * 4) =
                         entry_direct(zi, zj, p, kern, neg_inv_2s2, inv_sigma);
                 }
+                if (sums) {
+                    if (fixed) {   // this lane's row changed in the buffer
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            const float4 x = *reinterpret_cast<const float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4));
+                            out[4 * c] = x.x;
+                            out[4 * c + 1] = x.y;
+                            out[4 * c + 2] = x.z;
+                            out[4 * c + 3] = x.w;
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2) {
+                        pair_add2(rh, rl, pack2(out[e], out[e + 1]));
+                        mx = fmaxf(mx, fmaxf(out[e], out[e + 1]));
+                    }
+                    if (gl & 1) {   // a K-block is complete
+                        float h, l;
+                        pair_join(rh, rl, h, l);
+                        bt.rowpart[drow + lane + (int64_t)(g >> 1) * PANEL] = (double)h + (double)l;
+                        rh = rl = 0;
+                    }
+                }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
@@ -562,10 +639,48 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                                  : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
+                if (sums && tile.I != tile.J) {   // (the diagonal square's row sums have both triangles)
+                    // column `lane` of the group over the warp's rows, even and odd rows at once
+                    f32x2 ch = 0, cl = 0;
+#pragma unroll 8
+                    for (int r = 0; r < 32; r += 2) {
+                        const float x0 = *reinterpret_cast<const float *>(buf + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) +
+                                                                          (lane & 3) * 4);
+                        const float x1 = *reinterpret_cast<const float *>(
+                            buf + (r + 1) * 128 + (((lane >> 2) ^ ((r + 1) & 7)) << 4) + (lane & 3) * 4);
+                        pair_add2(ch, cl, pack2(x0, x1));
+                    }
+                    float h, l;
+                    pair_join(ch, cl, h, l);
+                    colsum[(warp - 2) * (PANEL / 2) + gl * 32 + lane] = make_float2(h, l);
+                }
                 ob ^= 1;
             }
             fence_before();
             mbar_arrive(su32(&bars->acc_empty[acc]));
+            if (sums) {
+                for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
+                if (lane == 0) atomicMax(&bt.ctr[tile.t].max_d_bits, __float_as_uint(mx));
+                half_sync(half, 1);
+                if (tile.I != tile.J) {
+                    // column c of the half: the four quarters in order; the panel's two row
+                    // halves (two tiles) meet in the zeroed sum, whose two terms commute
+                    const int c = quarter * 32 + lane;
+                    float h = 0.f, l = 0.f;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        // quarter q of this half: warps 2..9, quarter = warp mod 4, half = (warp - 2) / 4
+                        const int w = 4 * half + ((q + 2) & 3);
+                        const float2 x = colsum[w * (PANEL / 2) + c];
+                        float sum, e;
+                        two_sum(h, x.x, sum, e);
+                        h = sum;
+                        l += x.y + e;
+                    }
+                    const int64_t blk = drow / PANEL + half * 2 + (c >> 6);
+                    atomicAdd(&bt.colpart[blk * KB + (c & 63)], (double)h + (double)l);
+                }
+            }
             if (fixups) atomicAdd(&bt.ctr[tile.t].n_fixup, (unsigned long long)fixups);
             if (++acc == 2) {
                 acc = 0;

@@ -223,6 +223,7 @@ struct Batch {
     Counters *ctr;
     uint32_t *sel_hist;                  // median heuristic: 2048 bins per test (null if no test needs it)
     double *sacc;                        // streaming mode: FP64 sums of the windows' partials (Bp)
+    int build_sums;                      // the tensor-core build also sums its blocks' rows and columns
     int inject_stall;                    // failure-path test hook: the contraction's MMA issuer waits on a
                                          //   flag that nothing sets until its bounded wait expires
     unsigned long long wait_ns;          // limit of the tensor-core kernels' bounded waits (0: 2 s)
@@ -367,7 +368,9 @@ __device__ __forceinline__ UnitRec unit_at_position(const Batch &bt, int64_t k) 
 // ---- launchers (ept_kernels.cu) ----
 void launch_norms(const Batch &b, cudaStream_t s);                       // plain path: norms + finite check
 void launch_build_simt(const Batch &b, cudaStream_t s);
-void launch_blocksums(const Batch &b, cudaStream_t s);   // median-heuristic tests: kernel transform first
+// row and column sums of the blocks (median-heuristic tests: kernel transform first); median_only: of
+// those tests alone (the tensor-core build has done the others')
+void launch_blocksums(const Batch &b, bool median_only, cudaStream_t s);
 void launch_median_select(const Batch &b, int num_sms, cudaStream_t s);   // exact selection of the median distance
 void launch_rowsum_reduce(const Batch &b, cudaStream_t s);
 void launch_center(const Batch &b, cudaStream_t s);

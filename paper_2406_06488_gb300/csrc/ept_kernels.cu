@@ -640,6 +640,7 @@ void launch_build_simt(const Batch &b, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
+// (The tensor-core build sums its own entries but for median-heuristic tests.)
 // Row and column partial sums of each stored block, for the row sums r = W 1
 // (the lower part of W is the transpose of the stored strictly-upper blocks, so
 // their column sums supply it).  Sums are accumulated as unevaluated FP32 pairs
@@ -659,7 +660,7 @@ __device__ __forceinline__ void pair_add(float &h, float &l, float h2, float l2)
     l += l2 + e;
 }
 
-__global__ void __launch_bounds__(256) k_blocksums(const Batch bt) {
+__global__ void __launch_bounds__(256) k_blocksums(const Batch bt, int median_only) {
     constexpr int QR = 64, LD = KB + 1;   // rows per quarter, padded row length
     __shared__ float tile[QR * LD];
     __shared__ float wmax[8];
@@ -670,6 +671,7 @@ __global__ void __launch_bounds__(256) k_blocksums(const Batch bt) {
     const TestDesc &d = bt.desc[bi.t];
     // median-heuristic tests: the build wrote distances; now that the bandwidth is
     // known, they become kernel values in place as they are read (padding stays 0)
+    if (median_only && !d.median) return;   // the tensor-core build has summed its entries
     const bool median = d.median != 0;
     float neg = 0.f, inv = 0.f;
     if (median) {
@@ -750,9 +752,9 @@ __global__ void __launch_bounds__(256) k_blocksums(const Batch bt) {
     }
 }
 
-void launch_blocksums(const Batch &b, cudaStream_t s) {
+void launch_blocksums(const Batch &b, bool median_only, cudaStream_t s) {
     if (b.nblk_total <= 0) return;
-    k_blocksums<<<(unsigned)b.nblk_total, 256, 0, s>>>(b);
+    k_blocksums<<<(unsigned)b.nblk_total, 256, 0, s>>>(b, median_only ? 1 : 0);
 }
 
 // ---------------------------------------------------------------------------

@@ -238,7 +238,7 @@ extern "C" ept_status ept_test_static(const float *X, int64_t nx, const float *Y
                                                                       (BlkInfo *)(A + P.blk), (Chunk *)(A + P.chunks));
     launch_norms(b, s);
     launch_build_simt(b, s);
-    launch_blocksums(b, s);
+    launch_blocksums(b, false, s);
     launch_rowsum_reduce(b, s);
     launch_center(b, s);
     launch_pack(b, true, s);
