@@ -48,22 +48,39 @@ __global__ void __launch_bounds__(256) k_stream_rowsums(const Batch bt, int64_t 
     if (sub == 0 && i < d.n) bt.r[d.row0 + i] += acc;
 }
 
-// sacc[b] += the window's partials of relabeling b (FP64, fixed order).  CTA = 32
-// columns, warp w takes every eighth partial row.
-__global__ void __launch_bounds__(256) k_stream_accum(const Batch bt) {
-    __shared__ double ws[8][32];
+// sacc[b] += the window's partials of relabeling b (fixed order).  CTA = 32 columns, warp w
+// takes every 32nd partial row: eight at a time (their loads in flight together) as an
+// unevaluated FP32 pair (TwoSum), the pairs in FP64.  Bound by the loads; with an FP64 addition per
+// partial on eight warps this GPU's FP64 rate was the limit (n = 100,000, B = 4000, 1.3 GB of
+// partials in three windows: 2.87 ms, now 1.00).
+__global__ void __launch_bounds__(1024) k_stream_accum(const Batch bt) {
+    constexpr int NW = 32;
+    __shared__ double ws[NW][32];
     const TestDesc &d = bt.desc[0];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t c = (int64_t)blockIdx.x * 32 + lane, Bp = d.Bp;
     const float *part = bt.partial + d.part0 + c;
     double acc = 0.0;
-    for (int64_t k = warp; k < d.nparts; k += 8) acc += (double)part[k * Bp];
+    for (int64_t k0 = warp; k0 < d.nparts; k0 += 8 * NW) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = k0 + k * NW < d.nparts ? part[(k0 + k * NW) * Bp] : 0.f;
+        float h = 0.f, l = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            float s2, e;
+            two_sum(h, v[k], s2, e);
+            h = s2;
+            l += e;
+        }
+        acc += (double)h + (double)l;
+    }
     ws[warp][lane] = acc;
     __syncthreads();
     if (warp == 0) {
         double q = 0.0;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) q += ws[w][lane];
+#pragma unroll 8
+        for (int w = 0; w < NW; ++w) q += ws[w][lane];
         bt.sacc[c] += q;
     }
 }
@@ -113,7 +130,7 @@ void launch_stream_rowsums(const Batch &g, int64_t I0, int64_t I1, int64_t n_pad
 
 void launch_stream_accum(const Batch &g, cudaStream_t s) {
     if (g.ncols_total <= 0) return;
-    k_stream_accum<<<(unsigned)(g.ncols_total / 32), 256, 0, s>>>(g);
+    k_stream_accum<<<(unsigned)(g.ncols_total / 32), 1024, 0, s>>>(g);
 }
 
 void launch_stream_stats(const Batch &b, cudaStream_t s) {
