@@ -91,59 +91,107 @@ __device__ __forceinline__ const float *row_ptr(const TestDesc &d, int64_t i) {
     return (i < d.nx) ? d.X + i * d.p : d.Y + (i - d.nx) * d.p;
 }
 
+// Squared norm of a row by one warp, lane l taking elements 2l, 2l + 1 of each 64: the order that
+// decides whether a row near FP32's limit overflows within a lane (NaN) or only in the rounding (inf).
+__device__ __noinline__ double row_norm_by_warp(const float *z, int64_t p, int lane) {
+    float sh = 0.f, sl = 0.f;
+    for (int64_t k = 2 * lane; k < p; k += 64) {
+        #pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float v = (k + j < p) ? z[k + j] : 0.f;
+            if (!isfinite(v)) v = 0.f;
+            const float q = v * v, e = fmaf(v, v, -q);
+            float s2, f;
+            two_sum(sh, q, s2, f);
+            sh = s2;
+            sl += f + e;
+        }
+    }
+    double acc = (double)sh + (double)sl;
+    for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
+    return acc;
+}
+
 // Pooled row i of a test -> FP16 hi / lo parts of c_i z_i (zero padding up to the
 // test's p_pad), the inverse scale 1/c_i, and the squared norm of the unscaled row
 // (each product split exactly into p + e by an FMA, the p summed with TwoSum and
 // every rounding error carried in a second FP32 sum: about FP64 accuracy without
-// FP64 arithmetic per element; the lanes' pairs are added in FP64 and rounded once).
+// FP64 arithmetic; the lanes' pairs are added the same way and rounded once).
 // c_i = 2^k with
 // max |c_i z_i| < 2^14, k clamped to [-60, 60] so that 1/c_i 1/c_j stays a normal
 // FP32 number (rows above 2^74 would overflow the FP32 norms in any case).
-// Non-finite inputs are counted.  One warp per row of the batch.
+// Non-finite inputs are counted, once a row.
+//
+// L lanes per row, 4 elements of it a lane and step (16 bytes read, 8 bytes written to each part; element by
+// element where a row is not 16-byte aligned); the first KEEP steps stay in registers between the maximum and
+// the split, so that a row of up to 16 L elements is read once.  A warp's fixed work (finding the test, scale,
+// reductions: with an FP64 tree and one row a warp about 250 SM cycles, half of them FP64) was what bounded it:
+// four rows a warp share it, and the pairs are added as pairs.  500 tests of 400 x 100 (212 MB of traffic,
+// 31 us at the copy rate): 148 -> 57 us; 512 tests of up to 4,000 x 500: 772 -> 533 us.
+template <int L>
 __global__ void __launch_bounds__(256) k_split_rows(const Batch bt) {
-    const int lane = threadIdx.x & 31;
-    const int64_t gr = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (gr >= bt.nrows_total) return;
-    const int t = find_test(bt.pre.rows, bt.n_tests, gr);
-    const TestDesc &d = bt.desc[t];
-    const int64_t i = gr - d.row0;
-    const int64_t p = d.p, p_pad = d.p_pad;
-    const float *z = (i < d.n) ? row_ptr(d, i) : nullptr;
+    constexpr int R = 32 / L, KEEP = 4;
+    constexpr int STEP = 4 * L;
+    const int lane = threadIdx.x & 31, sub = lane % L;
     if (bt.build_sums) {   // the column sums that the build adds to
         const int64_t threads = (int64_t)gridDim.x * blockDim.x;
         for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < bt.nblk_total * KB; k += threads)
             bt.colpart[k] = 0.0;
     }
+    const int64_t gr = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * R + lane / L;
+    const bool row = gr < bt.nrows_total;   // every lane stays for the warp's shuffles
+    const int t = row ? find_test(bt.pre.rows, bt.n_tests, gr) : 0;
+    const TestDesc &d = bt.desc[t];
+    const int64_t i = gr - d.row0;
+    const int p = (row && i < d.n) ? (int)d.p : 0, p_pad = row ? (int)d.p_pad : 0;   // padding rows: zeros
+    const float *z = p ? row_ptr(d, i) : nullptr;
+    const bool vec = (p & 3) == 0 && ((uintptr_t)z & 15) == 0;   // 16-byte loads; else element by element
+    auto load = [&](int k) -> float4 {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (vec) {
+            if (k < p) v = __ldg(reinterpret_cast<const float4 *>(z + k));
+        } else {
+            if (k < p) v.x = z[k];
+            if (k + 1 < p) v.y = z[k + 1];
+            if (k + 2 < p) v.z = z[k + 2];
+            if (k + 3 < p) v.w = z[k + 3];
+        }
+        return v;
+    };
     uint32_t mx = 0;
     bool bad = false;
-    if (z) {
-        for (int64_t k = lane; k < p; k += 32) {
-            const float v = z[k];
-            if (isfinite(v)) mx = max(mx, __float_as_uint(fabsf(v)));
+    auto take_max = [&](float4 v) {
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t m = __float_as_uint((&v.x)[j]) & 0x7FFFFFFFu;
+            if (m < 0x7F800000u) mx = max(mx, m);
             else bad = true;
         }
-    }
-    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-    if (__any_sync(0xFFFFFFFFu, bad)) {
-        if (lane == 0) atomicAdd(&bt.ctr[t].nonfinite, 1ull);
-    }
-    int k2 = 0;
-    if (mx) {
-        int e;
-        frexpf(__uint_as_float(mx), &e);   // max = f 2^e, 0.5 <= f < 1
-        k2 = 14 - e;
-        k2 = k2 < -60 ? -60 : (k2 > 60 ? 60 : k2);
-    }
-    const float c = ldexpf(1.f, k2);
+    };
+    float4 keep[KEEP];
+    #pragma unroll
+    for (int q = 0; q < KEEP; ++q) keep[q] = load(4 * sub + q * STEP);
+    #pragma unroll
+    for (int q = 0; q < KEEP; ++q)
+        if (q * STEP < p) take_max(keep[q]);
+    for (int k = 4 * sub + KEEP * STEP; k < p; k += STEP) take_max(load(k));
+    #pragma unroll
+    for (int off = L / 2; off; off >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
+    const uint32_t bads = __ballot_sync(0xFFFFFFFFu, bad) >> (lane - sub) & (uint32_t)((1ull << L) - 1);
+    if (bads && sub == 0) atomicAdd(&bt.ctr[t].nonfinite, 1ull);
+    // 2^(e - 1) <= max < 2^e; below the normal range the clamp takes over
+    int k2 = mx ? 14 - ((int)(mx >> 23) - 126) : 0;
+    k2 = k2 < -60 ? -60 : (k2 > 60 ? 60 : k2);
+    const float c = __uint_as_float((uint32_t)(127 + k2) << 23);
     __half *zh = (__half *)bt.Zh + gr * bt.p_stride, *zl = (__half *)bt.Zl + gr * bt.p_stride;
     float sh = 0.f, sl = 0.f;
-    for (int64_t k = 2 * lane; k < p_pad; k += 64) {
-        float v0 = 0.f, v1 = 0.f;
-        if (z && k < p) v0 = z[k];
-        if (z && k + 1 < p) v1 = z[k + 1];
-        if (!isfinite(v0)) v0 = 0.f;
-        if (!isfinite(v1)) v1 = 0.f;
-        {
+    auto split = [&](int k, float4 v4) {
+        __half2 h[2], l[2];
+        #pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float v0 = (&v4.x)[2 * j], v1 = (&v4.x)[2 * j + 1];
+            if (!isfinite(v0)) v0 = 0.f;
+            if (!isfinite(v1)) v1 = 0.f;
             const float p0 = v0 * v0, e0 = fmaf(v0, v0, -p0);
             const float p1 = v1 * v1, e1 = fmaf(v1, v1, -p1);
             float s2, f;
@@ -153,19 +201,40 @@ __global__ void __launch_bounds__(256) k_split_rows(const Batch bt) {
             two_sum(sh, p1, s2, f);
             sh = s2;
             sl += f + e1;
+            const float w0 = v0 * c, w1 = v1 * c;
+            h[j] = __floats2half2_rn(w0, w1);
+            const float2 hf = __half22float2(h[j]);
+            l[j] = __floats2half2_rn(w0 - hf.x, w1 - hf.y);
         }
-        const float w0 = v0 * c, w1 = v1 * c;
-        const __half h0 = __float2half_rn(w0), h1 = __float2half_rn(w1);
-        const __half l0 = __float2half_rn(w0 - __half2float(h0));
-        const __half l1 = __float2half_rn(w1 - __half2float(h1));
-        *reinterpret_cast<__half2 *>(zh + k) = __halves2half2(h0, h1);
-        *reinterpret_cast<__half2 *>(zl + k) = __halves2half2(l0, l1);
+        *reinterpret_cast<uint2 *>(zh + k) = *reinterpret_cast<const uint2 *>(h);
+        *reinterpret_cast<uint2 *>(zl + k) = *reinterpret_cast<const uint2 *>(l);
+    };
+    #pragma unroll
+    for (int q = 0; q < KEEP; ++q)
+        if (4 * sub + q * STEP < p_pad) split(4 * sub + q * STEP, keep[q]);
+    for (int k = 4 * sub + KEEP * STEP; k < p_pad; k += STEP) split(k, load(k));
+    #pragma unroll
+    for (int off = L / 2; off; off >>= 1) {
+        const float oh = __shfl_xor_sync(0xFFFFFFFFu, sh, off), ol = __shfl_xor_sync(0xFFFFFFFFu, sl, off);
+        float s2, f;
+        two_sum(sh, oh, s2, f);
+        sh = s2;
+        sl += ol;
+        sl += f;
     }
-    double acc = (double)sh + (double)sl;
-    for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
-    if (lane == 0) {
-        bt.norms[gr] = (float)acc;
-        bt.iscale[gr] = ldexpf(1.f, -k2);
+    float norm = sh + sl;
+    // near FP32's limit (or past it within a lane): once more, by the whole warp
+    uint32_t over = __ballot_sync(0xFFFFFFFFu, sub == 0 && !(norm <= 1e38f));
+    while (over) {
+        const int src = __ffs(over) - 1;
+        over &= over - 1;
+        const float *zr = (const float *)__shfl_sync(0xFFFFFFFFu, (unsigned long long)z, src);
+        const double a = row_norm_by_warp(zr, __shfl_sync(0xFFFFFFFFu, p, src), lane);
+        if (lane - sub == src) norm = (float)a;
+    }
+    if (row && sub == 0) {
+        bt.norms[gr] = norm;
+        bt.iscale[gr] = __uint_as_float((uint32_t)(127 - k2) << 23);
     }
 }
 
@@ -700,9 +769,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 
 }  // namespace
 
+// Eight lanes a row once the rows fill the chip that way; with fewer rows, or long ones, a row's own steps
+// are what is waited for and the whole warp takes them.  Measured, 8 lanes against 32 (us): 4,000 rows of
+// 64 features 3.9 / 4.3, 16,000 of 64 5.8 / 11.1, 400 of 500 7.8 / 3.8, 16,000 of 300 13.4 / 14.2, 32,000 of
+// 300 22 / 25, 32,000 of 1,000 81 / 62.
+constexpr int64_t SPLIT_NARROW_ROWS = 4096, SPLIT_WIDE_ROWS = 32768;
+
 void launch_split_rows(const Batch &b, cudaStream_t s) {
     if (b.nrows_total <= 0) return;
-    k_split_rows<<<(unsigned)((b.nrows_total + 7) / 8), 256, 0, s>>>(b);
+    const unsigned warps = 256 / 32;
+    if (b.p_stride <= 128 ? b.nrows_total >= SPLIT_NARROW_ROWS : b.p_stride <= 512 && b.nrows_total >= SPLIT_WIDE_ROWS)
+        k_split_rows<8><<<(unsigned)((b.nrows_total + 4 * warps - 1) / (4 * warps)), 256, 0, s>>>(b);
+    else
+        k_split_rows<32><<<(unsigned)((b.nrows_total + warps - 1) / warps), 256, 0, s>>>(b);
 }
 
 cudaError_t launch_build_tc(const Batch &b, const void *tmaps, int num_sms, cudaStream_t s) {
