@@ -244,8 +244,13 @@ void plan_schedule(Plan &P, int num_sms, int unit_order = 0) {
     }
 }
 
-void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host_in, int chunk_kb,
-                int num_sms = 160, bool debug = false, bool schedule = true, int order = 0, bool pair_records = false) {
+// How much of the contraction's schedule a plan holds: nothing, all of it, or only the space that it takes
+// (the same layout and total without visiting the units: what admission needs; a burst of 16 requests of up to
+// 10^4 rows is submitted in 1.5 ms instead of 5.2).
+enum Schedule { SCHED_NONE, SCHED_FULL, SCHED_SPACE };
+
+void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host_in, int chunk_kb, int num_sms = 160,
+                bool debug = false, Schedule schedule = SCHED_FULL, int order = 0, bool pair_records = false) {
     P = Plan();
     static std::atomic<uint64_t> plans{0};
     P.serial = ++plans;
@@ -307,8 +312,11 @@ void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host
     }
     P.ncols_pad = P.pre_cols.back();
     P.nunits = P.pre_units.back();
-    if (tc && schedule) plan_schedule(P, num_sms, order);
-    if (tc && pair_records) {   // the pair kernel takes pair units in order (unit 2 pu: row half 0)
+    if (tc && schedule == SCHED_FULL) plan_schedule(P, num_sms, order);
+    const size_t nsched = tc && schedule != SCHED_NONE ? (size_t)P.nunits : 0;
+    const size_t ngrid = nsched ? (size_t)std::min<int64_t>(std::max(num_sms, 1), P.nunits) + 1 : 0;
+    const size_t npairs = tc && pair_records ? (size_t)(P.nunits / 2) : 0;
+    if (npairs && schedule != SCHED_SPACE) {   // the pair kernel takes pair units in order (unit 2 pu: row half 0)
         P.urec_pair.resize((size_t)(P.nunits / 2));
         for (int64_t pu = 0; pu < P.nunits / 2; ++pu) {
             const int64_t u = 2 * pu;
@@ -348,14 +356,14 @@ void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host
     P.off_blk = take(sizeof(BlkInfo) * P.blk.size());
     P.off_tiles = take(sizeof(Tile) * P.tiles.size());
     P.off_chunks = take(sizeof(Chunk) * P.chunks.size());
-    P.off_sched = take(8 * P.sched.size());
-    P.off_sched_off = take(8 * P.sched_off.size());
+    P.off_sched = take(8 * nsched);
+    P.off_sched_off = take(8 * ngrid);
     P.tab_bytes = o;
     o = align_up(o, 1024);
     in_data = true;
     // the unit records: uploaded with the first run of the plan, not with every run
-    P.off_urec = take(sizeof(UnitRec) * P.urec.size());
-    P.off_urec_pair = take(sizeof(UnitRec) * P.urec_pair.size());
+    P.off_urec = take(sizeof(UnitRec) * nsched);
+    P.off_urec_pair = take(sizeof(UnitRec) * npairs);
     if (P.debug) {   // a band right after the tables as well
         P.guards.off[P.guards.n++] = o;
         o += GUARD_BYTES;
@@ -524,8 +532,18 @@ public:
         const void *src;
         size_t bytes;
     };
-    explicit HostCopier(int workers) {
-        for (int k = 0; k < workers; ++k) th_.emplace_back([this] { worker(); });
+    // a copier of up to 8 workers, half the machine's cores; null where no thread can be started
+    static std::unique_ptr<HostCopier> create() {
+        const unsigned hw = std::thread::hardware_concurrency();
+        std::unique_ptr<HostCopier> c(new (std::nothrow) HostCopier());
+        if (!c) return c;
+        try {
+            for (unsigned k = std::max(1u, std::min(8u, hw / 2)); k > 0; --k)
+                c->th_.emplace_back([p = c.get()] { p->worker(); });
+        } catch (const std::exception &) {   // fewer workers, or none
+            if (c->th_.empty()) c.reset();
+        }
+        return c;
     }
     ~HostCopier() {
         {
@@ -536,7 +554,9 @@ public:
         for (std::thread &t : th_) t.join();
     }
     void run(const std::vector<Job> &jobs) {
-        constexpr size_t PIECE = 1 << 20;
+        size_t total = 0;
+        for (const Job &j : jobs) total += j.bytes;
+        const size_t PIECE = total >= ((size_t)32 << 20) ? (size_t)1 << 20 : (size_t)1 << 18;
         {
             std::unique_lock<std::mutex> lk(mu_);
             cv_done_.wait(lk, [this] { return active_ == 0; });   // a late worker of the last run has left
@@ -851,10 +871,9 @@ void stage_host(ept_ctx *c, Plan &P, const std::vector<TestSpec> &specs, bool on
         }
     }
     if (gather_bytes >= ((size_t)4 << 20)) {
-        if (!c->copier) {
-            const unsigned hw = std::thread::hardware_concurrency();
-            c->copier.reset(new HostCopier((int)std::max(1u, std::min(8u, hw / 2))));
-        }
+        if (!c->copier) c->copier = HostCopier::create();
+    }
+    if (gather_bytes >= ((size_t)4 << 20) && c->copier) {
         c->copier->run(gather);
     } else {
         for (const HostCopier::Job &j : gather) memcpy(j.dst, j.src, j.bytes);
@@ -1419,7 +1438,7 @@ ept_status run_once(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, bo
         if (!c->plan) return fail(EPT_ENOMEM, "host allocation failed");
     }
     if (c->plan_key != pkey) {
-        plan_batch(*c->plan, specs, prec, !on_device, chunk_kb, c->num_sms, c->debug, true, tn.order,
+        plan_batch(*c->plan, specs, prec, !on_device, chunk_kb, c->num_sms, c->debug, SCHED_FULL, tn.order,
                    (tn.kernel ? tn.kernel : contraction_kernel(c)) == 2);
         c->plan->draw_mode = tn.draw_mode;
         c->plan->contraction = tn.kernel;
@@ -1871,7 +1890,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     std::unique_ptr<Plan> hold(new (std::nothrow) Plan());
     if (!hold) return fail(EPT_ENOMEM, "host allocation failed");
     Plan &P = *hold;
-    plan_batch(P, specs, prec, !on_device, unit_kb(c), c->num_sms, c->debug, false);
+    plan_batch(P, specs, prec, !on_device, unit_kb(c), c->num_sms, c->debug, SCHED_NONE);
     P.stream = true;
     const size_t tab0 = P.tab_bytes;
     const TestDesc &d = P.desc[0];
@@ -2046,7 +2065,7 @@ void pooled_layout(Plan &P, int num_sms) {
 }
 
 void plan_pooled(Plan &P, const std::vector<TestSpec> &specs, bool host_in, int num_sms, bool debug = false) {
-    plan_batch(P, specs, EPT_PREC_PLAIN_FP32, host_in, CHUNK_KB_DEFAULT, num_sms, debug, false);
+    plan_batch(P, specs, EPT_PREC_PLAIN_FP32, host_in, CHUNK_KB_DEFAULT, num_sms, debug, SCHED_NONE);
     TestDesc &d = P.desc[0];
     d.comp = 0;   // the relabelings mark x*
     d.m = d.nx;
@@ -2147,10 +2166,15 @@ enum ReqState { REQ_PENDING = 0, REQ_RUNNING = 1, REQ_DONE = 2, REQ_CANCELLED = 
 
 using Clock = std::chrono::steady_clock;
 
+struct HostBuffer {
+    std::unique_ptr<float[]> data;
+    size_t cap = 0;   // floats
+};
+
 struct Request {
     uint64_t ticket = 0;
     TestSpec spec;
-    std::vector<float> X, Y;
+    HostBuffer samples;    // X, then Y
     std::vector<double> stats;
     ept_result res;
     int prec = 0;
@@ -2168,6 +2192,7 @@ struct Lane {
     std::vector<Request *> reqs;
     std::vector<TestSpec> specs;
     Plan plan;
+    bool pair_records = false;
     size_t bytes = 0;   // device scratch held by the lane's run
     uint8_t *arena = nullptr;
     cudaEvent_t done = nullptr;
@@ -2190,7 +2215,66 @@ struct Server {
     size_t max_pending = 1 << 16;
     int64_t peak_busy = 0;         // the most lanes that held a running batch at the same time
     int64_t submits_busy = 0;      // requests submitted while some lane held a running batch
+    // Sample memory of finished requests, for the next ones (guarded by mu; at most SPARE_BYTES, freed with the
+    // server).  Copying the samples is most of a burst's time, and into fresh memory half of the copy is
+    // page faults: 88 MB take one core 9 ms, into used memory 5, and with the workers below 1.3.
+    std::vector<HostBuffer> spare;
+    size_t spare_bytes = 0;
+    // Worker threads for the samples' copies; a submitter that finds them taken copies by itself.
+    std::mutex copy_mu;
+    std::unique_ptr<HostCopier> copier;
 };
+
+constexpr size_t SPARE_BYTES = (size_t)256 << 20;
+constexpr size_t SPARE_MIN = (size_t)128 << 10;     // smaller buffers are the heap's own business
+constexpr size_t PARALLEL_COPY = (size_t)1 << 20;   // below, waking the workers costs what they would save
+
+// Memory for `floats` values: a spare buffer of up to twice that, else a new one (data == nullptr: none to be had).
+HostBuffer take_buffer(Server *S, size_t floats) {
+    {
+        std::lock_guard<std::mutex> lk(S->mu);
+        size_t best = S->spare.size();
+        for (size_t k = 0; k < S->spare.size(); ++k) {
+            const size_t cap = S->spare[k].cap;
+            if (cap >= floats && cap / 2 <= floats && (best == S->spare.size() || cap < S->spare[best].cap)) best = k;
+        }
+        if (best < S->spare.size()) {
+            HostBuffer b = std::move(S->spare[best]);
+            S->spare[best] = std::move(S->spare.back());
+            S->spare.pop_back();
+            S->spare_bytes -= b.cap * sizeof(float);
+            return b;
+        }
+    }
+    HostBuffer b;
+    b.data.reset(new (std::nothrow) float[floats]);
+    b.cap = b.data ? floats : 0;
+    return b;
+}
+
+// Keeps a finished request's memory (lock held); what does not fit is freed by the caller, without the lock.
+void give_buffer(Server *S, HostBuffer &b) {
+    const size_t bytes = b.cap * sizeof(float);
+    if (bytes < SPARE_MIN || S->spare_bytes + bytes > SPARE_BYTES) return;
+    S->spare_bytes += bytes;
+    S->spare.push_back(std::move(b));
+    b.cap = 0;
+}
+
+void copy_samples(Server *S, const std::vector<HostCopier::Job> &jobs) {
+    size_t bytes = 0;
+    for (const HostCopier::Job &j : jobs) bytes += j.bytes;
+    std::unique_lock<std::mutex> lk(S->copy_mu, std::try_to_lock);
+    if (bytes >= PARALLEL_COPY && lk.owns_lock()) {
+        if (!S->copier) S->copier = HostCopier::create();
+        if (S->copier) {
+            S->copier->run(jobs);
+            return;
+        }
+    }
+    if (lk.owns_lock()) lk.unlock();
+    for (const HostCopier::Job &j : jobs) memcpy(j.dst, j.src, j.bytes);
+}
 
 void CUDART_CB lane_finished(void *arg) {
     Server *S = (Server *)arg;
@@ -2215,6 +2299,9 @@ ept_status lane_release(Server *S, Lane &L) {
 ept_status lane_enqueue(Server *S, Lane &L) {
     ept_ctx *c = L.ctx;
     cudaStream_t s = c->stream;
+    // the schedule, without the server lock: submissions go on meanwhile
+    plan_batch(L.plan, L.specs, L.reqs[0]->prec, true, unit_kb(c), c->num_sms, false, SCHED_FULL, 0, L.pair_records);
+    if (L.plan.total != L.bytes) return fail(EPT_EINTERNAL, "serving plan differs from the admitted one");
     const Staging SL = staging_layout(L.plan);
     ept_status st = ensure_pinned(c, SL.total);
     if (st != EPT_OK) return st;
@@ -2282,7 +2369,7 @@ void finish_requests(Server *S, Lane &L, ept_status st, const std::string &msg, 
 // Takes the next batch from the queue for a free lane (lock held): requests of the
 // first request's precision in arrival order, while slots and memory allow.  The
 // batch's exact scratch size is planned; requests are handed back from the end
-// until it fits.
+// until it fits.  The schedule itself is planned by lane_enqueue.
 bool form_batch(Server *S, Lane &L) {
     if (S->pending.empty()) return false;
     const int prec = S->pending.front()->prec;
@@ -2303,8 +2390,8 @@ bool form_batch(Server *S, Lane &L) {
     std::vector<TestSpec> specs;
     for (Request *r : batch) specs.push_back(r->spec);
     while (!batch.empty()) {
-        plan_batch(L.plan, specs, prec, true, unit_kb(L.ctx), L.ctx->num_sms, false, true, 0,
-                   contraction_kernel(S->owner) == 2);
+        L.pair_records = contraction_kernel(S->owner) == 2;
+        plan_batch(L.plan, specs, prec, true, unit_kb(L.ctx), L.ctx->num_sms, false, SCHED_SPACE, 0, L.pair_records);
         if (S->in_use + L.plan.total <= S->budget) break;
         // hand the last one back, at its place in arrival order
         Request *r = batch.back();
@@ -2610,7 +2697,7 @@ ept_status ept_plan_check(const int64_t *nx, const int64_t *ny, const int64_t *p
     if (!hold) return fail(EPT_ENOMEM, "host allocation failed");
     Plan &P = *hold;
     const bool streaming = stream_blocks > 0;
-    plan_batch(P, specs, EPT_PREC_SPLIT_BF16, true, unit_kb, num_sms, true, !streaming);
+    plan_batch(P, specs, EPT_PREC_SPLIT_BF16, true, unit_kb, num_sms, true, streaming ? SCHED_NONE : SCHED_FULL);
     if (streaming) {
         // as the streaming run plans it: windows of panels, chunks of each window by first K-block
         P.stream = true;
@@ -2900,14 +2987,20 @@ ept_status ept_submit(ept_ctx *c, const ept_test_desc *q, int prec, uint64_t *ti
     Server *S = c->server;
     Request *r = new (std::nothrow) Request();
     if (!r) return fail(EPT_ENOMEM, "host allocation failed");
-    r->X.assign(q->X, q->X + q->nx * q->p);
-    r->Y.assign(q->Y, q->Y + q->ny * q->p);
+    const size_t fx = (size_t)q->nx * q->p, fy = (size_t)q->ny * q->p;
+    r->samples = take_buffer(S, fx + fy);
+    if (!r->samples.data) {
+        delete r;
+        return fail(EPT_ENOMEM, "host allocation failed");
+    }
+    float *const X = r->samples.data.get(), *const Y = X + fx;
+    copy_samples(S, {{X, q->X, fx * sizeof(float)}, {Y, q->Y, fy * sizeof(float)}});
     r->stats.assign((size_t)q->B, 0.0);
-    r->spec = one_test(r->X.data(), q->nx, r->Y.data(), q->ny, q->p, q->stat, q->sigma, q->B, q->seed, nullptr,
+    r->spec = one_test(X, q->nx, Y, q->ny, q->p, q->stat, q->sigma, q->B, q->seed, nullptr,
                        q->B > 0 ? r->stats.data() : nullptr)[0];
     r->prec = prec;
     Plan P;
-    plan_batch(P, std::vector<TestSpec>(1, r->spec), prec, true, unit_kb(c));
+    plan_batch(P, std::vector<TestSpec>(1, r->spec), prec, true, unit_kb(c), 160, false, SCHED_SPACE);
     r->bytes = P.total;
     std::lock_guard<std::mutex> lk(S->mu);
     if (r->bytes > S->budget) {
@@ -2966,6 +3059,8 @@ ept_status ept_wait(ept_ctx *c, uint64_t ticket, double *perm_stats, ept_result 
         if (out) *out = r->res;
         if (perm_stats && !r->stats.empty()) memcpy(perm_stats, r->stats.data(), r->stats.size() * 8);
     }
+    give_buffer(S, r->samples);
+    lk.unlock();
     delete r;
     if (state == REQ_CANCELLED) return fail(EPT_ECANCELLED, "request %llu was cancelled", (unsigned long long)ticket);
     if (st != EPT_OK) return fail(st, "%s", msg.c_str());
