@@ -1003,18 +1003,20 @@ void launch_median_select(const Batch &b, int num_sms, cudaStream_t s) {
 // r_i = sum over the stored blocks of row i's panel (its own row segments) + sum
 // over the earlier panels J < panel(i) of column i's segments.  Eight threads per
 // row take every eighth term and combine by a fixed shuffle tree (deterministic).
-// CTA = 32 rows of one test (256 threads); Spart[CTA] = sum of its rows' r_i.
+// CTA = 32 rows of one test (256 threads); Spart[CTA] = sum of its rows' r_i, by one warp's tree: as one
+// thread's 32 additions in a row it was most of a small test's time (n = 200: 4.5 -> 3.5 us; 500 tests of
+// n = 400: 58 -> 43 us).
 __global__ void __launch_bounds__(256) k_rowsum_reduce(const Batch bt) {
     __shared__ double sh[32];
     const int sub = threadIdx.x & 7, rl = threadIdx.x >> 3;
     const int64_t gr = (int64_t)blockIdx.x * 32 + rl;
     const int t = find_test(bt.pre.rows, bt.n_tests, (int64_t)blockIdx.x * 32);
-    const TestDesc d = bt.desc[t];
+    const TestDesc &d = bt.desc[t];
     const int64_t i = gr - d.row0;
     const int64_t I = i / PANEL, rr = i % PANEL, NKB = d.NKB;
     double acc = 0.0;
     if (i < d.n) {
-        const int64_t nkb = NKB - KB_PER_PANEL * I;
+        const int64_t nkb = contract_nkb(d) - KB_PER_PANEL * I;   // those with real columns
         const int64_t base = d.blk0 + blk_off(I, NKB);
         for (int64_t k = sub; k < nkb; k += 8) acc += bt.rowpart[(base + k) * PANEL + rr];
         const int64_t kbi = i / KB, ci = i % KB;
@@ -1028,10 +1030,10 @@ __global__ void __launch_bounds__(256) k_rowsum_reduce(const Batch bt) {
         sh[rl] = acc;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int k = 0; k < 32; ++k) s += sh[k];
-        bt.Spart[blockIdx.x] = s;
+    if (threadIdx.x < 32) {
+        double s = sh[threadIdx.x];
+        for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+        if (threadIdx.x == 0) bt.Spart[blockIdx.x] = s;
     }
 }
 
@@ -1135,41 +1137,54 @@ void launch_center(const Batch &b, cudaStream_t s) {
 // (packed_scale): |c C - hi - lo| <= 2^-22 |c C|, written over the block's own FP32
 // storage (Batch::Chi / Clo with block stride c_stride), so the packed operand needs
 // no memory of its own.  One CTA per block.
+//
+// Bound by the copy (8 bytes an entry) once there are blocks enough, by the latency of one block below.
+// An FP64 instruction takes a warp 16 cycles of its SM, so the diagonal's three, issued row by row for one
+// lane each, were the longest part of a diagonal block: now one row a lane.  n = 200: 8.7 -> 4.8 us;
+// 500 tests of n = 400 (786 MB, 116 us at the copy rate): 170 -> 120 us; 512 tests of up to 4,000 rows
+// 2,085 -> 1,845 us; n = 20,000: 267 -> 257 us (of 240).
 template <bool SPLIT>
 __global__ void __launch_bounds__(512) k_pack(const Batch bt) {
     const int64_t gb = blockIdx.x;
-    const BlkInfo bi = bt.blk[gb];
-    const TestDesc d = bt.desc[bi.t];
-    const int64_t n = d.n;
-    const float *u = bt.u + d.row0;
-    const double *dcorr = bt.dcorr + d.row0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t j0 = (int64_t)bi.kb * KB + 2 * lane;
-    const float uj[2] = {(j0 < n) ? u[j0] : 0.f, (j0 + 1 < n) ? u[j0 + 1] : 0.f};
-    const int64_t row0 = (int64_t)bi.I * PANEL + warp * 16;   // 16 warps x 16 rows
-    const float cs = SPLIT ? packed_scale(bt.ctr[bi.t]) : 1.f;
     // the whole block is read before any of it is rewritten: the split parts are
-    // written over the block's own FP32 storage (hi in its first half, lo in its second)
+    // written over the block's own FP32 storage (hi in its first half, lo in its second).
+    // Its loads do not wait for the block's test, descriptor and vectors.
     float2 dv[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q)
-        dv[q] = *reinterpret_cast<const float2 *>(bt.D + (gb * PANEL + warp * 16 + q) * KB + 2 * lane);
+        dv[q] = __ldcs(reinterpret_cast<const float2 *>(bt.D + (gb * PANEL + warp * 16 + q) * KB + 2 * lane));
+    const BlkInfo bi = bt.blk[gb];
+    const TestDesc &d = bt.desc[bi.t];
+    const int64_t n = d.n;
+    const int64_t j0 = (int64_t)bi.kb * KB + 2 * lane;
+    if ((int64_t)bi.kb * KB >= n) return;   // a K-block of padding: the build's zeros are also the split's
+    const float *u = bt.u + d.row0;
+    const double *dcorr = bt.dcorr + d.row0;
+    const float uj[2] = {(j0 < n) ? u[j0] : 0.f, (j0 + 1 < n) ? u[j0 + 1] : 0.f};
+    const int64_t row0 = (int64_t)bi.I * PANEL + warp * 16;   // 16 warps x 16 rows
+    const float cs = SPLIT ? packed_scale(bt.ctr[bi.t]) : 1.f;
+    // diagonal entries, one row a lane: FP64 arithmetic once for the warp's 16 rows, not row by row
+    const bool on_diag = row0 / KB == bi.kb;   // the warp's rows cross the diagonal in this block, or none does
+    float diag = 0.f;
+    if (on_diag && lane < 16 && row0 + lane < n) {
+        const int64_t i = row0 + lane;
+        const float dii = bt.D[(gb * PANEL + warp * 16 + lane) * KB + (i - (int64_t)bi.kb * KB)];
+        diag = (float)((double)dii - 2.0 * (double)u[i] - dcorr[i]);
+    }
     if (SPLIT) __syncthreads();
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
         const int64_t i = row0 + q;
         const float ui = (i < n) ? u[i] : 0.f;
         const float dq[2] = {dv[q].x, dv[q].y};
+        const float di = on_diag ? __shfl_sync(0xFFFFFFFFu, diag, q) : 0.f;
         float w[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int64_t j = j0 + e;
-            float v = 0.f;
-            if (i < n && j < n && j >= i) {
-                if (j == i) v = (float)((double)dq[e] - 2.0 * (double)ui - dcorr[i]);
-                else v = 2.f * ((dq[e] - ui) - uj[e]);
-            }
-            w[e] = v;
+            const float v = j == i ? di : 2.f * ((dq[e] - ui) - uj[e]);
+            w[e] = (i < n && j < n && j >= i) ? v : 0.f;
         }
         const int64_t r = warp * 16 + q;
         if (SPLIT) {
