@@ -1057,11 +1057,12 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
     CK(cudaStreamWaitEvent(s, c->ev_in, with_inputs ? cudaEventWaitDefault : cudaEventWaitExternal));
     if (tc) {
         launch_split_rows(b, s);
+        const int split = build_split(b.ntiles, c->num_sms);
         alignas(64) CUtensorMap tm[5];
         char emsg[160];
-        if (!encode_build_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, b.D, P.nblk, emsg, sizeof(emsg)))
+        if (!encode_build_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, b.D, P.nblk, split, emsg, sizeof(emsg)))
             return fail(EPT_ECUDA, "%s", emsg);
-        CK(launch_build_tc(b, tm, c->num_sms, s));
+        CK(launch_build_tc(b, tm, split, c->num_sms, s));
     } else {
         launch_norms(b, s);
         launch_build_simt(b, s);
@@ -1973,7 +1974,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     alignas(64) CUtensorMap tm[5];
     alignas(64) CUtensorMap th, tl;
     char emsg[160];
-    if (!encode_build_tmaps(tm, bf.Zh, bf.Zl, P.nrows, P.p_stride, bf.D, P.win_blk, emsg, sizeof(emsg)))
+    if (!encode_build_tmaps(tm, bf.Zh, bf.Zl, P.nrows, P.p_stride, bf.D, P.win_blk, 0, emsg, sizeof(emsg)))
         return fail(EPT_ECUDA, "%s", emsg);
     if (!encode_block_tmaps(&th, &tl, bf.Chi, bf.Clo, P.win_blk, bf.c_stride, emsg, sizeof(emsg)))
         return fail(EPT_ECUDA, "%s", emsg);
@@ -1989,7 +1990,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
         Batch gv = stream_view(c, P, g);
         gv.build_sums = 1;
         CK(cudaMemsetAsync(gv.colpart, 0, (size_t)P.gnblk[(size_t)g] * KB * 8, s));
-        CK(launch_build_tc(gv, tm, c->num_sms, s));
+        CK(launch_build_tc(gv, tm, 0, c->num_sms, s));
         launch_stream_rowsums(gv, P.gI0[(size_t)g], P.gI1[(size_t)g], d.n_pad, s);
         CK(cudaGetLastError());
     }
@@ -2002,7 +2003,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     // pass 2: build again, pack, contract, fold the partials
     for (int g = 0; g < nwin; ++g) {
         const Batch gv = stream_view(c, P, g);
-        CK(launch_build_tc(gv, tm, c->num_sms, s));
+        CK(launch_build_tc(gv, tm, 0, c->num_sms, s));
         launch_pack(gv, true, s);
         CK(cudaGetLastError());
         if (g < ntimed) CK(cudaEventRecord(c->ev_win[2 * (size_t)g], s));
@@ -2871,10 +2872,12 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     CK(cudaMemsetAsync(b.ctr, 0, sizeof(Counters), s));
     if (prec == EPT_PREC_SPLIT_BF16) {
         launch_split_rows(b, s);
+        const int split = build_split(b.ntiles, c->num_sms);
         alignas(64) CUtensorMap tm[5];
         char emsg[160];
-        if (!encode_build_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, b.D, P.nblk, emsg, sizeof(emsg))) return fail(EPT_ECUDA, "%s", emsg);
-        CK(launch_build_tc(b, tm, c->num_sms, s));
+        if (!encode_build_tmaps(tm, b.Zh, b.Zl, P.nrows, P.p_stride, b.D, P.nblk, split, emsg, sizeof(emsg)))
+            return fail(EPT_ECUDA, "%s", emsg);
+        CK(launch_build_tc(b, tm, split, c->num_sms, s));
     } else {
         launch_norms(b, s);
         launch_build_simt(b, s);

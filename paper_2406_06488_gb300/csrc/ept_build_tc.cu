@@ -37,8 +37,9 @@
 // two row halves of a panel by two additions to a zeroed FP64 sum (two terms commute).  That
 // spares k_blocksums and its pass over every stored entry.
 // n = 20,000, p = 100: Gaussian 483 us and 197 for the sums -> 265 without sums, 434 with them; n = 5000,
-// p = 200: 43 + 17 -> 38 us, p = 1000 (tensor pipe 70 % busy) 65 + 21 -> 62 us; n = 200, p = 10 (close
-// pairs recomputed) 27 + 11 -> 21 us.
+// p = 200: 43 + 17 -> 38 us, p = 1000 (tensor pipe 70 % busy) 65 + 21 -> 60 us; n = 200, p = 10 (close
+// pairs recomputed) 27 + 11 -> 12.5 us.  With few tiles each is shared by several CTAs (build_split).
+// Sixteen epilogue warps, a K-block each, issue no more (96 registers spill; 434 -> 447 us).
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -72,9 +73,6 @@ constexpr int COL_OFF = BAR_OFF + 1024;
 constexpr int SUM_OFF = COL_OFF + 8 * (PANEL / 2) * 8;
 constexpr int SMEM_BYTES = SUM_OFF + 8 * (PANEL / 2) * 8 + 1024;
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of the build");
-// kind::f16 instruction descriptor with A = B = FP16 (format 0), D = FP32, K-major
-constexpr uint32_t IDESC = idesc_f16_f32(BM, BN);
-
 constexpr unsigned long long ERR_WAIT_TMA = 0x201, ERR_WAIT_MMA = 0x202, ERR_WAIT_EPI = 0x203, ERR_DRAIN = 0x205;
 
 struct Bars {
@@ -436,13 +434,15 @@ __device__ __forceinline__ float entry_direct(const float *zi, const float *zj, 
     return s + (fmaf(-s, s, h) + l) * (0.5f / s);   // the residual h + l - s s is exact up to l's last bits
 }
 
+template <bool SHARED>   // tiles shared by several CTAs (build_split); whole ones keep their constants
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     k_build_tc(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ CUtensorMap tm_al,
                const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CUtensorMap tm_bl,
-               const __grid_constant__ CUtensorMap tm_d, const Batch bt) {
+               const __grid_constant__ CUtensorMap tm_d, const Batch bt, const int parts_log) {
+    const int split = SHARED ? parts_log : 0;
     Counters *ctr = bt.ctr;   // bounded-wait errors are recorded in test 0's counters
     const unsigned long long wait_ns = bt.wait_ns ? bt.wait_ns : WAIT_NS;   // limit of every bounded wait
-    const int ntiles = (int)bt.ntiles;
+    const int nitems = (int)bt.ntiles << split;   // item t: tile t >> split, part t mod 2^split of its columns
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     Bars *bars = reinterpret_cast<Bars *>(smem + BAR_OFF);
@@ -480,11 +480,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             int armed[STAGES];
             for (int s2 = 0; s2 < STAGES; ++s2) armed[s2] = -1;
             bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const Tile tile = bt.tiles[t];
+            for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
+                const Tile tile = bt.tiles[t >> split];
                 const int64_t row0 = bt.desc[tile.t].row0;
                 const int rowA = (int)row0 + tile.I * PANEL + tile.h * BM;
-                const int rowB = (int)row0 + tile.J * PANEL;
+                const int rowB = (int)row0 + tile.J * PANEL + (t & ((1 << split) - 1)) * (BN >> split);
                 const int kblocks = (int)((bt.desc[tile.t].p + BK - 1) / BK);
                 for (int kk = 0; kk < kblocks; ++kk) {
                     if (!mbar_wait(su32(&bars->empty[stage]), phase ^ 1u, abort_flag, ctr, ERR_WAIT_TMA, wait_ns)) {
@@ -492,11 +492,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         break;
                     }
                     const uint32_t full = su32(&bars->full[stage]);
-                    mbar_arrive_tx(full, STAGE_BYTES);
+                    mbar_arrive_tx(full, 2 * A_BYTES + ((2 * B_BYTES) >> split));
                     uint8_t *st = smem + stage * STAGE_BYTES;
                     tma_load_2d(su32(st), &tm_ah, kk * BK, rowA, full);
                     tma_load_2d(su32(st + A_BYTES), &tm_al, kk * BK, rowA, full);
-                    tma_load_2d(su32(st + 2 * A_BYTES), &tm_bh, kk * BK, rowB, full);
+                    tma_load_2d(su32(st + 2 * A_BYTES), &tm_bh, kk * BK, rowB, full);   // boxes of BN >> split rows
                     tma_load_2d(su32(st + 2 * A_BYTES + B_BYTES), &tm_bl, kk * BK, rowB, full);
                     armed[stage] = (int)phase;
                     if (++stage == STAGES) {
@@ -522,9 +522,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (lane == 0) {
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
+            const uint32_t idesc = idesc_f16_f32(BM, BN >> split);
             bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const int kblocks = (int)((bt.desc[bt.tiles[t].t].p + BK - 1) / BK);
+            for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
+                const int kblocks = (int)((bt.desc[bt.tiles[t >> split].t].p + BK - 1) / BK);
                 if (!mbar_wait(su32(&bars->acc_empty[acc]), acc_phase ^ 1u, abort_flag, ctr, ERR_WAIT_MMA, wait_ns)) {
                     ok = false;
                     break;
@@ -542,9 +543,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     const uint64_t dbh = desc_sw64(sa + 2 * A_BYTES), dbl = desc_sw64(sa + 2 * A_BYTES + B_BYTES);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
-                        mma_f16(d_tmem, dah + 2 * k, dbh + 2 * k, IDESC, (kk == 0 && k == 0) ? 0u : 1u);
-                        mma_f16(d_tmem, dah + 2 * k, dbl + 2 * k, IDESC, 1u);
-                        mma_f16(d_tmem, dal + 2 * k, dbh + 2 * k, IDESC, 1u);
+                        mma_f16(d_tmem, dah + 2 * k, dbh + 2 * k, idesc, (kk == 0 && k == 0) ? 0u : 1u);
+                        mma_f16(d_tmem, dah + 2 * k, dbl + 2 * k, idesc, 1u);
+                        mma_f16(d_tmem, dal + 2 * k, dbh + 2 * k, idesc, 1u);
                     }
                     mma_commit(su32(&bars->empty[stage]));
                     if (++stage == STAGES) {
@@ -586,8 +587,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         float2 *colsum = reinterpret_cast<float2 *>(smem + SUM_OFF);   // [warp][column of the half]
         int acc = 0;
         uint32_t acc_phase = 0;
-        for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-            const Tile tile = bt.tiles[t];
+        for (int t = blockIdx.x; t < nitems; t += gridDim.x) {
+            const Tile tile = bt.tiles[t >> split];
+            // The item's groups of 32 columns start at gi of the tile's; the warp takes `ng` from gi + gw:
+            // half of the item's, or (a part is one K-block) all of them for one of the halves.
+            const int part = t & ((1 << split) - 1), gi = part * (BN / 32 >> split);
+            const int gw = split < 2 ? half * (BN / 64 >> split) : 0;
+            const int ng = split < 2 ? BN / 64 >> split : (part & 1) == half ? 2 : 0;
             const TestDesc &d = bt.desc[tile.t];
             const int64_t n = d.n, p = d.p, NKB = d.NKB, nx = d.nx;
             const float *X = d.X, *Y = d.Y;
@@ -611,8 +617,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const float si = (i < n) ? inv_scale[i] : 0.f;
             __syncwarp();
 #pragma unroll
-            for (int c = lane; c < PANEL / 2; c += 32) {
-                const int64_t j = (int64_t)tile.J * PANEL + half * (PANEL / 2) + c;
+            for (int k = 0; k < BN / 64; ++k) {
+                const int c = 32 * k + lane;
+                if (k >= ng) break;
+                const int64_t j = (int64_t)tile.J * PANEL + (gi + gw) * 32 + c;
                 float *cp = colv + (c >> 1) * 4 + (c & 1);
                 cp[0] = (j < n) ? norms[j] : 0.f;
                 cp[2] = (j < n) ? inv_scale[j] : 0.f;
@@ -627,10 +635,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
-            for (int gl = 0; gl < BN / 64; ++gl) {
-                const int g = half * (BN / 64) + gl;   // column group of the tile
+            for (int gl = 0; gl < ng; ++gl) {
+                const int g = gi + gw + gl;   // column group of the tile
                 uint32_t v[32];
-                tmem_ld32(tbase + (uint32_t)(g * 32), v);
+                tmem_ld32(tbase + (uint32_t)((gw + gl) * 32), v);
                 const int64_t j0 = (int64_t)tile.J * PANEL + g * 32;
                 float out[32];
                 const float4 *cg = reinterpret_cast<const float4 *>(colv) + gl * 16;
@@ -639,7 +647,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                                                  : group_entries<2>(v, cg, ni, si, tau, neg_inv_2s2, inv_sigma, out);
                 uint32_t fix = 0;
                 if (__any_sync(0xFFFFFFFFu, patch)) {
-                    tmem_ld32(tbase + (uint32_t)(g * 32), v);   // read again: no registers held for this case
+                    tmem_ld32(tbase + (uint32_t)((gw + gl) * 32), v);   // read again: no registers held for this case
                     fix = group_patch(v, cg, ni, si, tau, kern, neg_inv_2s2, inv_sigma, out);
                 }
                 // padding rows / columns hold 0; the diagonal is exactly 0 (ED) / 1 (MMD)
@@ -731,9 +739,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
                 if (lane == 0) atomicMax(&bt.ctr[tile.t].max_d_bits, __float_as_uint(mx));
                 half_sync(half, 1);
-                if (tile.I != tile.J) {
-                    // column c of the half: the four quarters in order; the panel's two row
-                    // halves (two tiles) meet in the zeroed sum, whose two terms commute
+                if (tile.I != tile.J && quarter < ng) {
+                    // column c of the warps' (in their group `quarter`): the four quarters in order; the panel's
+                    // two row halves (two tiles) meet in the zeroed sum, whose two terms commute
                     const int c = quarter * 32 + lane;
                     float h = 0.f, l = 0.f;
 #pragma unroll
@@ -746,7 +754,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         h = sum;
                         l += x.y + e;
                     }
-                    const int64_t blk = drow / PANEL + half * 2 + (c >> 6);
+                    const int64_t blk = drow / PANEL + ((gi + gw) >> 1) + (c >> 6);
                     atomicAdd(&bt.colpart[blk * KB + (c & 63)], (double)h + (double)l);
                 }
             }
@@ -784,14 +792,16 @@ void launch_split_rows(const Batch &b, cudaStream_t s) {
         k_split_rows<32><<<(unsigned)((b.nrows_total + warps - 1) / warps), 256, 0, s>>>(b);
 }
 
-cudaError_t launch_build_tc(const Batch &b, const void *tmaps, int num_sms, cudaStream_t s) {
-    static unsigned long long smem_set = 0;   // one bit per device
-    cudaError_t e = smem_limit_once((const void *)k_build_tc, SMEM_BYTES, &smem_set);
+cudaError_t launch_build_tc(const Batch &b, const void *tmaps, int split, int num_sms, cudaStream_t s) {
+    static unsigned long long smem_set[2] = {0, 0};   // one bit per device
+    const auto kernel = split ? k_build_tc<true> : k_build_tc<false>;
+    cudaError_t e = smem_limit_once((const void *)kernel, SMEM_BYTES, &smem_set[split ? 1 : 0]);
     if (e != cudaSuccess) return e;
     if (b.ntiles < 1) return cudaSuccess;
     const CUtensorMap *tm = (const CUtensorMap *)tmaps;
-    const int grid = b.ntiles < num_sms ? (int)b.ntiles : num_sms;
-    k_build_tc<<<grid, NUM_THREADS, SMEM_BYTES, s>>>(tm[0], tm[1], tm[2], tm[3], tm[4], b);
+    const int64_t items = b.ntiles << split;
+    const int grid = items < num_sms ? (int)items : num_sms;
+    kernel<<<grid, NUM_THREADS, SMEM_BYTES, s>>>(tm[0], tm[1], tm[2], tm[3], tm[4], b, split);
     return cudaGetLastError();
 }
 

@@ -427,13 +427,13 @@ static EncodeTiledFn encode_fn(char *err, size_t errlen) {
 }
 
 bool encode_build_tmaps(void *tmaps5, const uint16_t *Zh, const uint16_t *Zl, int64_t nrows, int64_t p_stride,
-                        float *D, int64_t nblk, char *err, size_t errlen) {
+                        float *D, int64_t nblk, int split, char *err, size_t errlen) {
     EncodeTiledFn enc = encode_fn(err, errlen);
     if (!enc) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)p_stride, (cuuint64_t)nrows};
     const cuuint64_t strides[1] = {(cuuint64_t)p_stride * 2};
     const cuuint32_t estr[2] = {1, 1};
-    const cuuint32_t box_a[2] = {BUILD_STAGE_K, 128}, box_b[2] = {BUILD_STAGE_K, 256};
+    const cuuint32_t box_a[2] = {BUILD_STAGE_K, 128}, box_b[2] = {BUILD_STAGE_K, 256u >> split};
     CUtensorMap *out = (CUtensorMap *)tmaps5;
     const void *srcs[4] = {Zh, Zl, Zh, Zl};
     const cuuint32_t *boxes[4] = {box_a, box_a, box_b, box_b};

@@ -436,7 +436,14 @@ void launch_expand_blocks(const float *D, int64_t n, int64_t NKB, float *out, cu
 
 // ---- tensor-core kernels (ept_build_tc.cu, ept_contract_tc.cu) ----
 void launch_split_rows(const Batch &b, cudaStream_t s);                  // FP16 hi/lo rows, norms, checks
-cudaError_t launch_build_tc(const Batch &b, const void *tmaps5, int num_sms, cudaStream_t s);
+// A tile of the build is shared by 2^split CTAs, each with its part of the tile's 256 columns, while there are
+// CTAs enough for all parts: a CTA's epilogue (about 10 us a tile) and, with many features, its MMAs are all
+// that a small test waits for.  Whole tiles against quarters: n = 200, p = 10 19.5 -> 12.5 us, n = 400,
+// p = 500 17.0 -> 12.5.  Beyond, the parts would take turns and load A once each.
+inline int build_split(int64_t ntiles, int num_sms) {
+    return 4 * ntiles <= num_sms ? 2 : 2 * ntiles <= num_sms ? 1 : 0;
+}
+cudaError_t launch_build_tc(const Batch &b, const void *tmaps5, int split, int num_sms, cudaStream_t s);
 cudaError_t launch_contract_tc(const Batch &b, const void *tmap_hi, const void *tmap_lo, int num_sms,
                                cudaStream_t s);
 // the same contraction on pairs of SMs (clusters of two CTAs, tcgen05 cta_group::2;
@@ -450,11 +457,11 @@ cudaError_t launch_contract_tm(const Batch &b, const void *tmap_hi, const void *
                                cudaStream_t s);
 // TMA descriptors: the packed hi/lo blocks [nblk_total x 256 x 64], block stride
 // c_stride halves; for the build the FP16 rows [nrows x p_stride] (hi, lo with boxes of
-// BUILD_STAGE_K x 128, then hi, lo with BUILD_STAGE_K x 256) and the FP32 entries of nblk blocks
+// BUILD_STAGE_K x 128, then hi, lo with BUILD_STAGE_K x 256 >> split) and the FP32 entries of nblk blocks
 bool encode_block_tmaps(void *tmap_hi, void *tmap_lo, const uint16_t *Chi, const uint16_t *Clo, int64_t nblk,
                         int64_t c_stride, char *err, size_t errlen);
 bool encode_build_tmaps(void *tmaps5, const uint16_t *Zh, const uint16_t *Zl, int64_t nrows, int64_t p_stride,
-                        float *D, int64_t nblk, char *err, size_t errlen);
+                        float *D, int64_t nblk, int split, char *err, size_t errlen);
 
 // ---- streaming mode (ept_stream.cu): one test, windows of row panels ----
 // r += the row and column sums of the window [I0, I1) (its stored blocks' parts)

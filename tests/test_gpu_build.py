@@ -81,3 +81,22 @@ def test_equal_and_close_rows(ctx, scale, stat):
     got, want = _compare(ctx, X, Y, stat, 3.0 * scale)
     same = np.arange(20)
     assert (got[same, 80 + same] == (0.0 if stat == "ed" else 1.0)).all()
+
+
+@pytest.mark.parametrize("stat", ["ed", "mmd"])
+@pytest.mark.parametrize("nx,ny", [(300, 500), (800, 700), (1000, 1048), (1000, 1049), (1100, 1200)])
+def test_tiles_shared_by_several_blocks(ctx, nx, ny, stat):
+    """A quarter, half or all of a tile's columns to a thread block (up to 38, up to 76 and more tiles on 152
+    SMs).  The row and column sums show in the statistic of the stored entries: the centred entries (at most
+    16 times the largest) are packed to 2^-22, and no statistic's weights sum to more than 4; a K-block's
+    missing sum would move it by more than 1e-3."""
+    p = 5
+    rng = np.random.default_rng(nx)
+    X = rng.standard_normal((nx, p), dtype=np.float32)
+    Y = rng.standard_normal((ny, p), dtype=np.float32) + np.float32(0.3)
+    sigma = float(np.sqrt(p))
+    got, _ = _compare(ctx, X, Y, stat, sigma)
+    xx, yy, xy = got[:nx, :nx].sum() / nx ** 2, got[nx:, nx:].sum() / ny ** 2, got[:nx, nx:].sum() / (nx * ny)
+    want = 2.0 * xy - xx - yy if stat == "ed" else xx + yy - 2.0 * xy
+    r = ctx.test(X, Y, B=30, seed=1, stat=stat, sigma=sigma)
+    assert abs(r.observed - want) <= 4.0 * 16.0 * 2.0 ** -22 * got.max()
