@@ -1069,8 +1069,9 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
     }
     launch_median_select(b, c->num_sms, s);
     if (!tc || P.any_median) launch_blocksums(b, tc, s);
-    launch_rowsum_reduce(b, s);
-    launch_center(b, s);
+    int64_t max_rows = 0;
+    for (const TestDesc &d : P.desc) max_rows = std::max(max_rows, d.n_pad);
+    launch_rowsums_center(b, max_rows, s);
     launch_pack(b, tc, s);
     CK(cudaGetLastError());
     if (timed) CK(cudaEventRecord(c->ev[2], s));

@@ -50,8 +50,8 @@ constexpr int BUILD_KB = 64;     // p is padded to a multiple of this for the te
 constexpr int BUILD_STAGE_K = 32;   // features per pipeline stage of that build
 constexpr int TC_TILE_N = 256;   // relabelings per contraction work unit (the MMA's N)
 // cap on the relabeling-draw blocks per SM (0: none, one warp per column).  Capping
-// lets the draws share SMs with the tensor-core build, but the draws are
-// latency-bound and run fastest at full occupancy, which measured best overall.
+// lets the draws share SMs with the tensor-core build, but both are issue-bound and the
+// build slows by what the draws hide (n = 5000: 514 us uncapped, 536 capped).
 constexpr int MASK_CTAS_PER_SM = 0;
 
 __host__ __device__ inline int64_t blk_off(int64_t I, int64_t NKB) { return I * NKB - 2 * I * (I - 1); }
@@ -374,6 +374,8 @@ void launch_blocksums(const Batch &b, bool median_only, cudaStream_t s);
 void launch_median_select(const Batch &b, int num_sms, cudaStream_t s);   // exact selection of the median distance
 void launch_rowsum_reduce(const Batch &b, cudaStream_t s);
 void launch_center(const Batch &b, cudaStream_t s);
+// both, in one launch where no test has more than 1,024 (max_rows) padded rows
+void launch_rowsums_center(const Batch &b, int64_t max_rows, cudaStream_t s);
 void launch_pack(const Batch &b, bool split, cudaStream_t s);   // split: FP16 hi/lo (tensor-core path)
 // draw kernels: a warp per relabeling column (caller relabelings, or few columns), a
 // lane per column with groups of 16 columns to a ring of four warps, and a lane per
