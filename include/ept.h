@@ -285,7 +285,8 @@ ept_status ept_test_batch(ept_ctx *ctx, const ept_test_desc *tests, int64_t n_te
    shapes M = 256 across a pair of SMs and N = 128 -- each with its recomputation of
    flagged statistics, keeps the fastest for the shape (ept_result.tuning,
    .tune_candidates) and uses it from then on; every candidate computes the same
-   statistics except for the accumulation order.
+   statistics except for the accumulation order, and one with another order has to be
+   3 % faster, twice, so that timing noise alone does not change the returned bits.
    EPT_OPT_DRAW_MODE (default 0): relabeling-draw kernel, 0 = automatic (by columns per
    SM: a warp per column below 36, groups of 16 columns below 400, a lane per column
    from there), 1 = a warp per column, 2 = a lane per column, 3 = groups of 16 columns,

@@ -143,15 +143,17 @@ def metrics_markdown(table):
 
 
 # the tuned path's kernels by phase (the plain path's k_contract_simt, k_build_simt,
-# k_norms and k_pack<0>, and the bench's own kernels, are not part of a tuned step)
+# k_norms, k_blocksums, k_refine_packed and k_pack<0>, and the bench's own kernels, are not part of a tuned step;
+# k_blocksums belongs to a tuned median-bandwidth step too, but its launches share one name)
 PHASES = [
     ("contraction", ["k_contract_tc", "k_contract_tc2", "k_contract_tm"]),
-    ("relabeling draws (side stream)", ["k_masks", "k_masks_lanes"]),
+    ("relabeling draws (side stream)", ["k_masks", "k_masks_group"]),
     ("block build", ["k_split_rows", "k_build_tc"]),
-    ("centring / packing", ["k_blocksums", "k_rowsum_reduce", "k_center_u", "k_center_r", "k_pack<1>"]),
-    ("combination", ["k_combine_stats", "k_combine_count", "k_batch_status", "k_reset_counts"]),
-    ("recomputation of flagged statistics", ["k_refine_packed", "k_refine_packed_finish", "k_refine_w",
-                                             "k_refine_rows", "k_refine_finish"]),
+    ("median bandwidth", ["k_median_sample", "k_median_pass"]),
+    ("centring / packing", ["k_rowsum_reduce", "k_center_u", "k_center_r", "k_center_small", "k_pack<1>"]),
+    ("combination", ["k_combine_stats", "k_combine_columns", "k_combine_count", "k_batch_status", "k_reset_counts"]),
+    ("recomputation of flagged statistics", ["k_refine_split", "k_refine_packed_finish",
+                                             "k_refine_w", "k_refine_rows", "k_refine_finish"]),
 ]
 
 
@@ -167,7 +169,7 @@ def phase_table(rows):
     means = {_short(k): mean for k, n, t, mean, share in launch_table(rows)}
     out = []
     for phase, kernels in PHASES:
-        present = [k for k in kernels if k in means]
+        present = [m for k in kernels for m in means if m == k or m.split("<")[0] == k]
         if present:
             out.append((phase, present, sum(means[k] for k in present)))
     total = sum(us for _, _, us in out) or 1.0
