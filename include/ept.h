@@ -296,7 +296,8 @@ ept_status ept_test_batch(ept_ctx *ctx, const ept_test_desc *tests, int64_t n_te
    of device scratch (a run's arena, a serving batch's pool allocation) fail with
    EPT_ENOMEM on the host, without touching the GPU, to exercise error paths.
    EPT_OPT_FAULT_INJECT_STALL (test hook, default 0): in the next run (tensor-core
-   path, launched directly) the contraction's MMA issuer waits on a device flag that
+   path, launched directly) the contraction's MMA issuer (value 2: one epilogue warp of
+   the block build) waits on a device flag that
    nothing sets; its bounded wait expires after 2 s, every role of the kernel takes
    the abort path (drain copies, free tensor memory, return) and the call returns
    EPT_ETIMEOUT; the context stays usable.  One-shot.

@@ -647,7 +647,7 @@ struct ept_ctx {
     size_t refine_cap = 0;
     ept_allocator alloc{};              // caller-supplied device memory (alloc.alloc == nullptr: cudaMalloc)
     std::atomic<int> inject_alloc{0};   // test hook: the next N scratch acquisitions fail (host side)
-    bool inject_stall = false;          // test hook: the next run's contraction waits out its limit
+    int inject_stall = 0;               // test hook: the next run's contraction (or build) waits out its limit
     int serve_lanes = 3;                // serving: batches in flight at once
     int serve_slots = 256;              // serving: requests in flight at once
     cudaEvent_t ev_user = nullptr;      // orders the context's stream after a caller's stream
@@ -955,7 +955,7 @@ Batch device_view(ept_ctx *c, const Plan &P) {
     b.ctr = (Counters *)(A + P.off_ctr);
     b.sel_hist = P.any_median ? (uint32_t *)(A + P.off_sel_hist) : nullptr;
     b.sacc = nullptr;
-    b.inject_stall = c->inject_stall ? 1 : 0;
+    b.inject_stall = c->inject_stall;
     b.wait_ns = c->wait_ns;
     return b;
 }
@@ -1507,7 +1507,7 @@ ept_status run_once(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, bo
         return EPT_OK;
     }
     st = enqueue_device(c, P, s, true);
-    c->inject_stall = false;   // the hook is one-shot
+    c->inject_stall = 0;   // the hook is one-shot
     if (st != EPT_OK) return st;
     CK(cudaStreamSynchronize(s));
     if ((st = collect(c, P, specs, out, true)) != EPT_OK) return st;
@@ -1875,7 +1875,7 @@ Batch stream_view(ept_ctx *c, const Plan &P, int g) {
     b.maskT = (uint32_t *)(A + P.off_maskT);
     b.ctr = (Counters *)(A + P.off_ctr);
     b.sacc = (double *)(A + P.off_sacc);
-    b.inject_stall = (g == 0 && c->inject_stall) ? 1 : 0;
+    b.inject_stall = g == 0 ? c->inject_stall : 0;
     b.wait_ns = c->wait_ns;
     return b;
 }
@@ -2020,7 +2020,7 @@ ept_status run_stream(ept_ctx *c, const std::vector<TestSpec> &specs, int prec, 
     CK(cudaEventRecord(c->ev[3], s));
     if ((st = read_back(c, P, s)) != EPT_OK) return st;
     CK(cudaEventRecord(c->ev[4], s));
-    c->inject_stall = false;   // the hook is one-shot
+    c->inject_stall = 0;   // the hook is one-shot
     CK(cudaStreamSynchronize(s));
     if ((st = collect(c, P, specs, out, false)) != EPT_OK) return st;
     float ms = 0.f;
@@ -2866,7 +2866,8 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     c->urec_serial = c->tab_serial = 0;   // and the arena its data, over a cached plan's tables and records
     stage_host(c, P, specs, on_device != 0);
     uint8_t *A = c->arena;
-    const Batch b = device_view(c, P);
+    Batch b = device_view(c, P);
+    b.inject_stall = 0;   // the hook is for runs
     if ((st = upload_tables(c, P, s)) != EPT_OK) return st;
     if ((st = enqueue_inputs(c, s)) != EPT_OK) return st;
     CK(cudaStreamWaitEvent(s, c->ev_in, 0));
@@ -2919,7 +2920,7 @@ ept_status ept_set_option(ept_ctx *c, int option, int64_t value) {
         c->inject_alloc.store((int)value);
         return EPT_OK;
     case EPT_OPT_FAULT_INJECT_STALL:
-        c->inject_stall = value != 0;
+        c->inject_stall = value == STALL_BUILD ? STALL_BUILD : value != 0 ? STALL_CONTRACTION : 0;
         return EPT_OK;
     case EPT_OPT_DEBUG_CHECKS:
         c->debug = value != 0;

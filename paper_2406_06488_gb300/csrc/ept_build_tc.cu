@@ -22,8 +22,8 @@
 // (A hi/lo 128 x 32, B hi/lo 256 x 32, 64-byte swizzle); two TMEM accumulators so
 // the epilogue of one tile overlaps the main loop of the next.  Roles (320
 // threads): warp 0 TMA, warp 1 MMA + TMEM owner, warps 2-9 epilogue (two per TMEM
-// lane quarter, each taking half of the tile's columns).  All waits are bounded as
-// in the contraction kernel.
+// lane quarter, each taking half of the tile's columns).  Every wait on an mbarrier is bounded as
+// in the contraction kernel; the epilogue's named barriers follow from those (half_sync).
 //
 // What bounds it: up to a few hundred features the epilogue, 32768 entries a tile on
 // eight warps, beyond that the tensor pipe.  A thread holds a row, so storing its entries itself
@@ -73,7 +73,8 @@ constexpr int COL_OFF = BAR_OFF + 1024;
 constexpr int SUM_OFF = COL_OFF + 8 * (PANEL / 2) * 8;
 constexpr int SMEM_BYTES = SUM_OFF + 8 * (PANEL / 2) * 8 + 1024;
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of the build");
-constexpr unsigned long long ERR_WAIT_TMA = 0x201, ERR_WAIT_MMA = 0x202, ERR_WAIT_EPI = 0x203, ERR_DRAIN = 0x205;
+constexpr unsigned long long ERR_WAIT_TMA = 0x201, ERR_WAIT_MMA = 0x202, ERR_WAIT_EPI = 0x203, ERR_DRAIN = 0x205,
+                             ERR_INJECTED = 0x2FE;
 
 struct Bars {
     unsigned long long full[STAGES];      // 1 arrival + TMA transaction bytes
@@ -284,18 +285,15 @@ __device__ __forceinline__ void pair_join(f32x2 h, f32x2 l, float &hs, float &ls
 }
 
 // Barriers of the four warps that share a half of the tile's columns: 0, before a tile's column
-// sums are written (the last tile's are read); 1, when they are.  A warp that gives up arrives at both.
+// sums are written (the last tile's are read); 1, when they are.  They have no limit of their own: each warp
+// takes both for every item that needs sums, also after it has given up, and between two of them
+// only bounded waits, so the longest wait at one is the other warps' bounded wait on the accumulator.
 __device__ __forceinline__ void half_sync(int half, int which) {
     if (half == 0 && which == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
     else if (half == 0) asm volatile("bar.sync 2, 128;" ::: "memory");
     else if (which == 0) asm volatile("bar.sync 3, 128;" ::: "memory");
     else asm volatile("bar.sync 4, 128;" ::: "memory");
 }
-__device__ __forceinline__ void half_leave(int half) {
-    if (half == 0) asm volatile("bar.arrive 1, 128;\n\tbar.arrive 2, 128;" ::: "memory");
-    else asm volatile("bar.arrive 3, 128;\n\tbar.arrive 4, 128;" ::: "memory");
-}
-
 // exp_cw of two arguments x in [-87, 0] (its operations in its order; outside the
 // range the caller patches the entry)
 __device__ __forceinline__ void exp_cw2(f32x2 x, float &y0, float &y1) {
@@ -587,6 +585,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         float2 *colsum = reinterpret_cast<float2 *>(smem + SUM_OFF);   // [warp][column of the half]
         int acc = 0;
         uint32_t acc_phase = 0;
+        // A warp that gives up (ok false) does no more work but stays for the barriers of the items left:
+        // the other three may still get an accumulator or two and wait for it there.
+        bool ok = true;
+        // failure-path test hook: one warp waits (bounded) on a flag that nothing sets, the others go on
+        if (bt.inject_stall == STALL_BUILD && warp == 2)
+            ok = __all_sync(0xFFFFFFFFu, flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns));
         for (int t = blockIdx.x; t < nitems; t += gridDim.x) {
             const Tile tile = bt.tiles[t >> split];
             // The item's groups of 32 columns start at gi of the tile's; the warp takes `ng` from gi + gw:
@@ -626,11 +630,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 cp[2] = (j < n) ? inv_scale[j] : 0.f;
             }
             __syncwarp();
-            // the warp's lanes leave together (the group loop below synchronises them)
-            if (!__all_sync(0xFFFFFFFFu, mbar_wait(su32(&bars->acc_full[acc]), acc_phase, abort_flag, ctr, ERR_WAIT_EPI,
-                                                   wait_ns))) {
-                half_leave(half);
-                break;
+            // the warp's lanes give up together (the group loop below synchronises them)
+            ok = ok && __all_sync(0xFFFFFFFFu, mbar_wait(su32(&bars->acc_full[acc]), acc_phase, abort_flag, ctr,
+                                                         ERR_WAIT_EPI, wait_ns));
+            if (!ok) {
+                if (sums) half_sync(half, 1);
+                continue;
             }
             fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         bool ok = true;
         // failure-path test hook: wait (bounded) on a flag that nothing sets; the
         // expiry takes the same abort path as any other expired wait
-        if (bt.inject_stall) ok = __all_sync(0xFFFFFFFFu, flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns));
+        if (bt.inject_stall == STALL_CONTRACTION) ok = __all_sync(0xFFFFFFFFu, flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns));
         UnitRec nx = record(k_first);
         for (int64_t k = k_first; k < k_end && ok; k += k_step) {
             const UnitRec x = nx;

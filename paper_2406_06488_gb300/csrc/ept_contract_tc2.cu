@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
-            if (bt.inject_stall && !flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns)) ok = false;
+            if (bt.inject_stall == STALL_CONTRACTION && !flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns)) ok = false;
             UnitRec nr = pair_record(bt, pair, npu);
             for (int64_t pu = pair; pu < npu && ok; pu += npairs) {
                 const Unit x = unit_of(nr);

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             bool ok = true;
             // failure-path test hook: wait (bounded) on a flag that nothing sets; the
             // expiry takes the same abort path as any other expired wait
-            if (bt.inject_stall && !flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns)) ok = false;
+            if (bt.inject_stall == STALL_CONTRACTION && !flag_wait(&ctr->never_set, abort_flag, ctr, ERR_INJECTED, wait_ns)) ok = false;
             for (int64_t k = k_first; k < k_end && ok; k += k_step) {
                 const Unit x = decode_unit(bt, unit_at(k));
                 for (int s = 0; s < 2 && ok; ++s) {

@@ -59,6 +59,7 @@ __host__ __device__ inline int64_t blk_index(int64_t I, int64_t kb, int64_t NKB)
     return blk_off(I, NKB) + (kb - KB_PER_PANEL * I);
 }
 
+enum { STALL_CONTRACTION = 1, STALL_BUILD = 2 };   // Batch::inject_stall: the MMA issuer, an epilogue warp
 struct Counters {
     unsigned long long n_ge;
     unsigned long long n_near;
@@ -224,7 +225,7 @@ struct Batch {
     uint32_t *sel_hist;                  // median heuristic: 2048 bins per test (null if no test needs it)
     double *sacc;                        // streaming mode: FP64 sums of the windows' partials (Bp)
     int build_sums;                      // the tensor-core build also sums its blocks' rows and columns
-    int inject_stall;                    // failure-path test hook: the contraction's MMA issuer waits on a
+    int inject_stall;                    // failure-path test hook (STALL_*): a warp of that kernel waits on a
                                          //   flag that nothing sets until its bounded wait expires
     unsigned long long wait_ns;          // limit of the tensor-core kernels' bounded waits (0: 2 s)
 };

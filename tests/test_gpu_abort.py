@@ -1,0 +1,73 @@
+"""A block build whose wait expires gives up as a whole.  The hook makes one of its epilogue
+warps wait out the limit on a flag that nothing sets while the tiles' accumulators still
+complete, so that the warps that share its half of a tile's columns go on for a tile or two
+without it: with one tile or part of a tile per thread block, with several, with tests that
+take their sums elsewhere (a median bandwidth) in between, and in windows.  The call returns
+EPT_ETIMEOUT within a few limits, and the next run of the context is right."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_2406_06488_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2406_06488_gb300 import ept
+    c = ept.Context(0)
+    c.set_option("autotune", 0)
+    c.set_option("wait_limit_ms", 50)
+    yield c
+    c.close()
+
+
+def _pair(nx, ny, p, seed):
+    return workloads.gaussian_pair(workloads.TwoSampleSpec(nx=nx, ny=ny, p=p, y_mean=0.2, data_seed=seed))
+
+
+def _expires(ctx, call):
+    from paper_2406_06488_gb300 import ept
+    ctx.set_option("fault_inject_stall", 2)
+    t0 = time.perf_counter()
+    with pytest.raises(ept.EptError) as e:
+        call()
+    assert e.value.status == 5
+    assert time.perf_counter() - t0 < 2.0
+
+
+@pytest.mark.parametrize("nx,ny,p", [(70, 60, 3), (300, 400, 33), (900, 1100, 8), (2600, 2400, 20), (6000, 6100, 40)])
+def test_build_gives_up_as_a_whole(ctx, nx, ny, p):
+    X, Y = _pair(nx, ny, p, seed=nx)
+    want = ctx.test(X, Y, B=60, seed=2)
+    _expires(ctx, lambda: ctx.test(X, Y, B=60, seed=2))
+    got = ctx.test(X, Y, B=60, seed=2)
+    assert got.observed == want.observed and np.array_equal(got.stats, want.stats)
+
+
+def test_build_gives_up_in_a_batch(ctx):
+    tests = []
+    for k in range(60):
+        X, Y = _pair(200 + 11 * k, 300, 6, seed=k)
+        tests.append(dict(X=X, Y=Y, B=20, seed=k, stat="mmd", sigma="median" if k % 3 == 1 else 2.0))
+    want = ctx.test_batch(tests)
+    _expires(ctx, lambda: ctx.test_batch(tests))
+    for a, b in zip(want, ctx.test_batch(tests)):
+        assert a.observed == b.observed and a.n_ge == b.n_ge
+
+
+def test_build_gives_up_in_windows(ctx):
+    X, Y = _pair(2000, 2100, 9, seed=5)
+    try:
+        ctx.set_option("stream_blocks", 300)
+        want = ctx.test(X, Y, B=40, seed=3)
+        assert want.n_windows > 2
+        _expires(ctx, lambda: ctx.test(X, Y, B=40, seed=3))
+        got = ctx.test(X, Y, B=40, seed=3)
+        assert got.observed == want.observed and np.array_equal(got.stats, want.stats)
+    finally:
+        ctx.set_option("stream_blocks", 0)
