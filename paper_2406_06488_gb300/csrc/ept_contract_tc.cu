@@ -94,6 +94,7 @@ struct Bars {
     unsigned long long drain;            // 1 arrival (final tcgen05.commit)
     uint32_t tmem_base;
     int abort_flag;
+    int copies_issued;                   // the copies' thread arms no further stage
 };
 static_assert(sizeof(Bars) <= 1024, "barrier region");
 
@@ -131,6 +132,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         mbar_init(su32(&bars->red), EPI_THREADS);
         mbar_init(su32(&bars->drain), 1);
         bars->abort_flag = 0;
+        bars->copies_issued = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -175,18 +177,20 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     }
                 }
             }
-            if (!ok) {
-                // drain: the copies armed last on each stage complete that phase of its
-                // barrier (the producers arrive on every stage when they give up); wait
-                // for it (bounded) before the CTA may exit
-                for (int s2 = 0; s2 < STAGES; ++s2) {
-                    if (armed[s2] < 0) continue;
-                    const unsigned long long t0 = gtimer();
-                    while (!mbar_try(su32(&bars->full[s2]), (uint32_t)armed[s2])) {
-                        if (gtimer() - t0 > wait_ns) {
-                            atomicCAS(&ctr->err_code, 0ull, ERR_DRAIN);
-                            break;
-                        }
+            __threadfence_block();
+            *(volatile int *)&bars->copies_issued = 1;
+            // drain: the copies armed last on each stage complete that phase of its
+            // barrier (the producers arrive on every stage when they give up, and only after
+            // the line above, so that no phase completes without its copies); wait for it
+            // (bounded) before the CTA may exit, also where all were armed: another role may
+            // give up while the last ones are under way
+            for (int s2 = 0; s2 < STAGES; ++s2) {
+                if (armed[s2] < 0) continue;
+                const unsigned long long t0 = gtimer();
+                while (!mbar_try(su32(&bars->full[s2]), (uint32_t)armed[s2])) {
+                    if (gtimer() - t0 > wait_ns) {
+                        atomicCAS(&ctr->err_code, 0ull, ERR_DRAIN);
+                        break;
                     }
                 }
             }
@@ -358,7 +362,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             expand_bits(cur.x, e);
             expand_bits(cur.y, e + 16);
             if (!mbar_wait(su32(&bars->empty[stage]), phase ^ 1u, abort_flag, ctr, ERR_WAIT_MASK, wait_ns)) {
-                // giving up: the copies already under way can then complete their stages' phases
+                // giving up: once the copies' thread has left its loop (it needs no producer for
+                // that), those already under way can complete their stages' phases
+                const unsigned long long t0 = gtimer();
+                while (!*(volatile int *)&bars->copies_issued && gtimer() - t0 <= wait_ns) __nanosleep(100);
+                __threadfence_block();
                 for (int s2 = 0; s2 < STAGES; ++s2) mbar_arrive(su32(&bars->full[s2]));
                 break;
             }

@@ -226,17 +226,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     }
                 }
             }
-            if (!ok) {
-                // drain: the copies armed last on each stage complete that phase of
-                // c_full; wait for it (bounded) before the CTA may exit
-                for (int s2 = 0; s2 < STAGES; ++s2) {
-                    if (armed[s2] < 0) continue;
-                    const unsigned long long t0 = gtimer();
-                    while (!mbar_try(su32(&bars->c_full[s2]), (uint32_t)armed[s2])) {
-                        if (gtimer() - t0 > wait_ns) {
-                            atomicCAS(&ctr->err_code, 0ull, ERR_DRAIN);
-                            break;
-                        }
+            // drain: the copies armed last on each stage complete that phase of
+            // c_full; wait for it (bounded) before the CTA may exit,
+            // also where all were armed: another role may give up before they have arrived
+            for (int s2 = 0; s2 < STAGES; ++s2) {
+                if (armed[s2] < 0) continue;
+                const unsigned long long t0 = gtimer();
+                while (!mbar_try(su32(&bars->c_full[s2]), (uint32_t)armed[s2])) {
+                    if (gtimer() - t0 > wait_ns) {
+                        atomicCAS(&ctr->err_code, 0ull, ERR_DRAIN);
+                        break;
                     }
                 }
             }

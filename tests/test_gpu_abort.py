@@ -3,7 +3,9 @@ warps wait out the limit on a flag that nothing sets while the tiles' accumulato
 complete, so that the warps that share its half of a tile's columns go on for a tile or two
 without it: with one tile or part of a tile per thread block, with several, with tests that
 take their sums elsewhere (a median bandwidth) in between, and in windows.  The call returns
-EPT_ETIMEOUT within a few limits, and the next run of the context is right."""
+EPT_ETIMEOUT within a few limits, and the next run of the context is right.  The same for the
+contraction kernels, whose stalled issuer leaves every stage's copies and relabeling tiles done or
+under way."""
 import time
 
 import numpy as np
@@ -30,9 +32,9 @@ def _pair(nx, ny, p, seed):
     return workloads.gaussian_pair(workloads.TwoSampleSpec(nx=nx, ny=ny, p=p, y_mean=0.2, data_seed=seed))
 
 
-def _expires(ctx, call):
+def _expires(ctx, call, hook=2):
     from paper_2406_06488_gb300 import ept
-    ctx.set_option("fault_inject_stall", 2)
+    ctx.set_option("fault_inject_stall", hook)
     t0 = time.perf_counter()
     with pytest.raises(ept.EptError) as e:
         call()
@@ -71,3 +73,18 @@ def test_build_gives_up_in_windows(ctx):
         assert got.observed == want.observed and np.array_equal(got.stats, want.stats)
     finally:
         ctx.set_option("stream_blocks", 0)
+
+
+@pytest.mark.parametrize("kernel", [1, 2, 3])
+@pytest.mark.parametrize("nx,ny,B", [(60, 70, 30), (2600, 2400, 1500)])   # one unit of few K-blocks, and many units
+def test_contraction_gives_up(ctx, kernel, nx, ny, B):
+    X, Y = _pair(nx, ny, 12, seed=nx)
+    try:
+        ctx.set_option("contraction", kernel)
+        want = ctx.test(X, Y, B=B, seed=4)
+        for _ in range(3):
+            _expires(ctx, lambda: ctx.test(X, Y, B=B, seed=4), hook=1)
+            got = ctx.test(X, Y, B=B, seed=4)
+            assert got.observed == want.observed and np.array_equal(got.stats, want.stats)
+    finally:
+        ctx.set_option("contraction", 0)
