@@ -12,7 +12,7 @@
 // the entries are about as accurate as an FP32 Gram), and the epilogue multiplies
 // by 1/c_i and 1/c_j (exact).
 // The epilogue forms d^2, recomputes cancellation-prone near-duplicate pairs
-// (d^2 < tau (||z_i||^2 + ||z_j||^2)) from direct differences summed as FP32 pairs, applies sqrt (distances),
+// (d^2 < tau (||z_i||^2 + ||z_j||^2)) from direct differences (entry_direct), applies sqrt (distances),
 // exp(-d^2 / (2 sigma^2)) (Gaussian) or exp(-d / sigma) (Laplacian), forces the
 // diagonal to 0 / 1, zeroes padding, and
 // writes the FP32 entries into the packed upper blocks.
@@ -381,27 +381,26 @@ __device__ __forceinline__ uint32_t group_patch(const uint32_t (&v)[32], const f
     return fix;
 }
 
-// (h, l) += (x - y)^2: the difference as an exact pair (TwoSum), its square to about 2^-47
-// relative (the head's square exactly, by an FMA, and twice the head times the tail),
-// the sum as a pair.
-__device__ __forceinline__ void add_square(float x, float y, float &h, float &l) {
-    float dh, dl, s, e;
-    two_sum(x, -y, dh, dl);
-    const float p = dh * dh, pe = fmaf(dh, dh, -p);
-    two_sum(h, p, s, e);
-    h = s;
-    l += e + fmaf(2.f * dh, dl, pe);
+// The squared distance of two rows in FP64, feature by feature.
+__device__ __forceinline__ double square_sum_fp64(const float *zi, const float *zj, int64_t p) {
+    double sq = 0.0;
+#pragma unroll 1
+    for (int64_t k = 0; k < p; ++k) {
+        const double df = (double)zi[k] - (double)zj[k];
+        sq = fma(df, df, sq);
+    }
+    return sq;
 }
 
-// The entry of two rows by direct differences.  The squared distance is summed as an
-// unevaluated FP32 pair: GB300's FP64 rate is so low that eight warps' FP64 sums of 10
-// features took 8,000 cycles.  Eight loads of each row are in flight.  Sums outside
-// the range where the pair keeps its 47 bits are taken again in FP64; equal rows are
-// 0 in either.  Then the square root, by one Newton correction of the rounded root of
-// the pair (within 2^-40 of the exact root before its rounding), or the kernel value in FP64.
+// The entry of two rows by direct differences: the FP32 number that the squared distance summed in FP64
+// gives.  It is summed as an FP32 pair instead, wherever the pair's error bound leaves one result: GB300's FP64
+// rate is so low that eight warps' FP64 sums of 10 features took 8,000 cycles.  Eight loads of each row are in
+// flight.  Left to FP64: sums near the ends of FP32's range, and the entries that the bound does not decide (one
+// in 2^14 of 10 features, one in 2^8 of 1,000); equal rows are 0 in either.
 __device__ __forceinline__ float entry_direct(const float *zi, const float *zj, int64_t p, int kern,
                                               float neg_inv_2s2, float inv_sigma) {
-    float h = 0.f, l = 0.f, far = 0.f;
+    SquareSum sum;
+    float far = 0.f;
 #pragma unroll 1
     for (int64_t k = 0; k < p; k += 8) {
         float a[8], b[8];
@@ -413,23 +412,43 @@ __device__ __forceinline__ float entry_direct(const float *zi, const float *zj, 
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             far = fmaxf(far, fabsf(a[e] - b[e]));
-            add_square(a[e], b[e], h, l);
+            sum.add(a[e], b[e]);
+        }
+        sum.renormalise();
+    }
+    const float t = sum.h + sum.l;
+    if (far == 0.f) return (float)entry_from_d2(0.0, kern, neg_inv_2s2, inv_sigma);
+    if (t > 1e-20f && t < 1e30f) {
+        float out;
+        if (kern == 0) {
+            if (sum.root(p, out)) return out;
+        } else {
+            // a kernel value's relative error: its exponent's error, and 2^-50 of the exponent and of itself
+            // for the FP64 operations on either way
+            const double v = entry_from_d2((double)sum.h + (double)sum.l, kern, neg_inv_2s2, inv_sigma);
+            const float x = kern == 1 ? -t * neg_inv_2s2 : sqrtf(t) * inv_sigma;
+            const float rel = x * (float)(41 * p + 64) * 3.5527137e-15f + (x + 1.f) * 8.8817842e-16f;
+            const double err = v * (double)(rel * 1.001f);
+            out = (float)(v - err);
+            if (out == (float)(v + err)) return out;
         }
     }
-    const float t = h + l;
-    if (far != 0.f && !(t > 1e-20f && t < 1e30f)) {
-        double sq = 0.0;
-#pragma unroll 1
-        for (int64_t k = 0; k < p; ++k) {
-            const double df = (double)zi[k] - (double)zj[k];
-            sq = fma(df, df, sq);
-        }
-        return (float)entry_from_d2(sq, kern, neg_inv_2s2, inv_sigma);
+    return (float)entry_from_d2(square_sum_fp64(zi, zj, p), kern, neg_inv_2s2, inv_sigma);
+}
+
+// The entries of row i (this lane's) in columns j0 + e, e in `fix`, directly into the staged group.  Not inlined: with
+// it in the group loop the loop's registers spill (n = 20,000, p = 100: 745 us for the build phase, 870 with it).
+__device__ __noinline__ void fix_entries(uint32_t fix, uint8_t *buf, const TestDesc &d, int64_t i, int64_t j0) {
+    const int lane = threadIdx.x & 31;
+    const int64_t p = d.p;
+    while (fix) {
+        const int e = __ffs(fix) - 1;
+        fix &= fix - 1u;
+        const int64_t j = j0 + e;
+        const float *zi = row_ptr(d, i), *zj = row_ptr(d, j);
+        *reinterpret_cast<float *>(buf + lane * 128 + (((e >> 2) ^ (lane & 7)) << 4) + (e & 3) * 4) =
+            entry_direct(zi, zj, p, d.kern, d.neg_inv_2s2, d.inv_sigma);
     }
-    if (kern != 0) return (float)entry_from_d2((double)h + (double)l, kern, neg_inv_2s2, inv_sigma);
-    if (far == 0.f) return 0.f;
-    const float s = sqrtf(t);
-    return s + (fmaf(-s, s, h) + l) * (0.5f / s);   // the residual h + l - s s is exact up to l's last bits
 }
 
 template <bool SHARED>   // tiles shared by several CTAs (build_split); whole ones keep their constants
@@ -599,8 +618,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const int gw = split < 2 ? half * (BN / 64 >> split) : 0;
             const int ng = split < 2 ? BN / 64 >> split : (part & 1) == half ? 2 : 0;
             const TestDesc &d = bt.desc[tile.t];
-            const int64_t n = d.n, p = d.p, NKB = d.NKB, nx = d.nx;
-            const float *X = d.X, *Y = d.Y;
+            const int64_t n = d.n, NKB = d.NKB;
             const int kern = d.kern;
             const float neg_inv_2s2 = d.neg_inv_2s2, inv_sigma = d.inv_sigma, tau = d.tau;
             const float diag_val = (kern == 0) ? 0.f : 1.f;
@@ -678,28 +696,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     *reinterpret_cast<float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4)) =
                         make_float4(out[4 * c], out[4 * c + 1], out[4 * c + 2], out[4 * c + 3]);
                 // cancellation-prone pairs: d^2 by direct differences
-                const bool fixed = fix != 0u;
-                while (fix) {
-                    const int e = __ffs(fix) - 1;
-                    fix &= fix - 1u;
-                    const int64_t j = j0 + e;
-                    const float *zi = (i < nx) ? X + i * p : Y + (i - nx) * p;
-                    const float *zj = (j < nx) ? X + j * p : Y + (j - nx) * p;
-                    ++fixups;
-                    *reinterpret_cast<float *>(buf + lane * 128 + (((e >> 2) ^ (lane & 7)) << 4) + (e & 3) * 4) =
-                        entry_direct(zi, zj, p, kern, neg_inv_2s2, inv_sigma);
+                if (__any_sync(0xFFFFFFFFu, fix != 0u)) {
+                    fixups += __popc(fix);
+                    fix_entries(fix, buf, d, i, j0);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {   // every lane's, so that no entry is held in registers meanwhile
+                        const float4 x = *reinterpret_cast<const float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4));
+                        out[4 * c] = x.x;
+                        out[4 * c + 1] = x.y;
+                        out[4 * c + 2] = x.z;
+                        out[4 * c + 3] = x.w;
+                    }
                 }
                 if (sums) {
-                    if (fixed) {   // this lane's row changed in the buffer
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const float4 x = *reinterpret_cast<const float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4));
-                            out[4 * c] = x.x;
-                            out[4 * c + 1] = x.y;
-                            out[4 * c + 2] = x.z;
-                            out[4 * c + 3] = x.w;
-                        }
-                    }
 #pragma unroll
                     for (int e = 0; e < 32; e += 2) {
                         pair_add2(rh, rl, pack2(out[e], out[e + 1]));

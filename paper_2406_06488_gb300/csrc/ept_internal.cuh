@@ -339,11 +339,50 @@ __host__ __device__ __forceinline__ float exp_cw(float x) {
 }
 
 // Knuth's TwoSum: s = fl(a + b) and the exact rounding error e, a + b = s + e.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+__host__ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = a + b;
     const float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
 }
+
+// a b rounded by itself, never contracted into an addition that follows
+__host__ __device__ __forceinline__ float mul_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
+// A sum of squared differences as an unevaluated FP32 pair, where FP64 would be the limit.
+// Error, u = 2^-24 and S the exact sum: an element's difference is exact (dh + dl), its square p + pe +
+// 2 dh dl but for dl^2 <= u^2 dh^2 and a rounding of 3 u^2 dh^2; the sum's rounding error e <= u S is kept in l,
+// which the additions there move by 4 u^2 S and u |l|; with l below 33 u S between two calls of
+// renormalise() (at most eight elements apart) that is 41 u^2 S an element.
+struct SquareSum {
+    float h = 0.f, l = 0.f;
+    __host__ __device__ __forceinline__ void add(float x, float y) {
+        float dh, dl, s, e;
+        two_sum(x, -y, dh, dl);
+        const float p = mul_rn(dh, dh), pe = fmaf(dh, dh, -p);
+        two_sum(h, p, s, e);
+        h = s;
+        l += e + fmaf(2.f * dh, dl, pe);
+    }
+    __host__ __device__ __forceinline__ void renormalise() {
+        const float s = h + l;
+        l -= s - h;
+        h = s;
+    }
+    // The square root of the sum of n elements, rounded once: the rounded root s of h + l and its Newton
+    // correction c, within 13 u^2 s of the pair's root.  False when the error bound leaves two results possible.
+    __host__ __device__ __forceinline__ bool root(int64_t n, float &out) const {
+        const float s = sqrtf(h + l), c = (fmaf(-s, s, h) + l) * (0.5f / s);
+        const float err = s * ((float)(21 * n + 32) * 3.5527137e-15f);   // (21 n + 32) u^2
+        out = s + (c - err);
+        return out == s + (c + err);
+    }
+};
 
 __device__ __forceinline__ int find_test(const int64_t *pre, int nt, int64_t g) {
     int lo = 0, hi = nt - 1;
