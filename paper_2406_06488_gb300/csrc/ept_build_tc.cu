@@ -90,32 +90,28 @@ __device__ __forceinline__ const float *row_ptr(const TestDesc &d, int64_t i) {
     return (i < d.nx) ? d.X + i * d.p : d.Y + (i - d.nx) * d.p;
 }
 
-// Squared norm of a row by one warp, lane l taking elements 2l, 2l + 1 of each 64: the order that
-// decides whether a row near FP32's limit overflows within a lane (NaN) or only in the rounding (inf).
+// Squared norm of a row by one warp, lane l taking elements 2l, 2l + 1 of each 64 and the lanes' sums added in
+// FP64: for the rows that the pairs of k_split_rows leave open, and in the order that decides whether a row near
+// FP32's limit overflows within a lane (NaN) or only in the rounding (inf).
 __device__ __noinline__ double row_norm_by_warp(const float *z, int64_t p, int lane) {
-    float sh = 0.f, sl = 0.f;
+    NormSum sum;
     for (int64_t k = 2 * lane; k < p; k += 64) {
         #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            float v = (k + j < p) ? z[k + j] : 0.f;
-            if (!isfinite(v)) v = 0.f;
-            const float q = v * v, e = fmaf(v, v, -q);
-            float s2, f;
-            two_sum(sh, q, s2, f);
-            sh = s2;
-            sl += f + e;
+            const float v = (k + j < p) ? z[k + j] : 0.f;
+            sum.add(isfinite(v) ? v : 0.f);
         }
     }
-    double acc = (double)sh + (double)sl;
+    double acc = (double)sum.h + (double)sum.l;
     for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
     return acc;
 }
 
 // Pooled row i of a test -> FP16 hi / lo parts of c_i z_i (zero padding up to the
 // test's p_pad), the inverse scale 1/c_i, and the squared norm of the unscaled row
-// (each product split exactly into p + e by an FMA, the p summed with TwoSum and
-// every rounding error carried in a second FP32 sum: about FP64 accuracy without
-// FP64 arithmetic; the lanes' pairs are added the same way and rounded once).
+// (each lane's as an FP32 pair, NormSum; the lanes' pairs are added the same way wherever
+// their error bound leaves one FP32 result, else in FP64: the norm is the one that the FP64
+// sum gives).
 // c_i = 2^k with
 // max |c_i z_i| < 2^14, k clamped to [-60, 60] so that 1/c_i 1/c_j stays a normal
 // FP32 number (rows above 2^74 would overflow the FP32 norms in any case).
@@ -183,7 +179,7 @@ __global__ void __launch_bounds__(256) k_split_rows(const Batch bt) {
     k2 = k2 < -60 ? -60 : (k2 > 60 ? 60 : k2);
     const float c = __uint_as_float((uint32_t)(127 + k2) << 23);
     __half *zh = (__half *)bt.Zh + gr * bt.p_stride, *zl = (__half *)bt.Zl + gr * bt.p_stride;
-    float sh = 0.f, sl = 0.f;
+    NormSum sum;
     auto split = [&](int k, float4 v4) {
         __half2 h[2], l[2];
         #pragma unroll
@@ -191,15 +187,8 @@ __global__ void __launch_bounds__(256) k_split_rows(const Batch bt) {
             float v0 = (&v4.x)[2 * j], v1 = (&v4.x)[2 * j + 1];
             if (!isfinite(v0)) v0 = 0.f;
             if (!isfinite(v1)) v1 = 0.f;
-            const float p0 = v0 * v0, e0 = fmaf(v0, v0, -p0);
-            const float p1 = v1 * v1, e1 = fmaf(v1, v1, -p1);
-            float s2, f;
-            two_sum(sh, p0, s2, f);
-            sh = s2;
-            sl += f + e0;
-            two_sum(sh, p1, s2, f);
-            sh = s2;
-            sl += f + e1;
+            sum.add(v0);
+            sum.add(v1);
             const float w0 = v0 * c, w1 = v1 * c;
             h[j] = __floats2half2_rn(w0, w1);
             const float2 hf = __half22float2(h[j]);
@@ -214,19 +203,17 @@ __global__ void __launch_bounds__(256) k_split_rows(const Batch bt) {
     for (int k = 4 * sub + KEEP * STEP; k < p_pad; k += STEP) split(k, load(k));
     #pragma unroll
     for (int off = L / 2; off; off >>= 1) {
-        const float oh = __shfl_xor_sync(0xFFFFFFFFu, sh, off), ol = __shfl_xor_sync(0xFFFFFFFFu, sl, off);
-        float s2, f;
-        two_sum(sh, oh, s2, f);
-        sh = s2;
-        sl += ol;
-        sl += f;
+        const float oh = __shfl_xor_sync(0xFFFFFFFFu, sum.h, off), ol = __shfl_xor_sync(0xFFFFFFFFu, sum.l, off);
+        sum.merge(oh, ol);
     }
-    float norm = sh + sl;
-    // near FP32's limit (or past it within a lane): once more, by the whole warp
-    uint32_t over = __ballot_sync(0xFFFFFFFFu, sub == 0 && !(norm <= 1e38f));
-    while (over) {
-        const int src = __ffs(over) - 1;
-        over &= over - 1;
+    // not decided by the bound (one row in 2^12 of 100 features, one in 2^10 of 1,000), or near FP32's limit
+    // (past it within a lane): once more, by the whole warp.  A lane has at most p / L + 4 elements.
+    float norm;
+    const bool sure = sum.rounded((float)(p / L + 10), norm);
+    uint32_t open = __ballot_sync(0xFFFFFFFFu, sub == 0 && !(sure && norm <= 1e38f));
+    while (open) {
+        const int src = __ffs(open) - 1;
+        open &= open - 1;
         const float *zr = (const float *)__shfl_sync(0xFFFFFFFFu, (unsigned long long)z, src);
         const double a = row_norm_by_warp(zr, __shfl_sync(0xFFFFFFFFu, p, src), lane);
         if (lane - sub == src) norm = (float)a;

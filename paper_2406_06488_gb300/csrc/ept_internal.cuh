@@ -384,6 +384,34 @@ struct SquareSum {
     }
 };
 
+// A sum of squares as an unevaluated FP32 pair: each product is split exactly by an FMA, the heads are summed with
+// TwoSum and every rounding error is carried in l.  Error of m elements added and up to five merges, u = 2^-24: an
+// element's two additions to l round at most 2 u^2 and 2 m u^2 of the sum so far, a merge 10 u^2 (2 m + 5) in all:
+// below 2 u^2 (m + 6)^2.
+struct NormSum {
+    float h = 0.f, l = 0.f;
+    __host__ __device__ __forceinline__ void add(float v) {
+        const float p = mul_rn(v, v), e = fmaf(v, v, -p);
+        float s, f;
+        two_sum(h, p, s, f);
+        h = s;
+        l += f + e;
+    }
+    __host__ __device__ __forceinline__ void merge(float oh, float ol) {
+        float s, f;
+        two_sum(h, oh, s, f);
+        h = s;
+        l += ol;
+        l += f;
+    }
+    // The sum rounded once; false when twice the error bound (m6 >= m + 6) leaves two results possible.
+    __host__ __device__ __forceinline__ bool rounded(float m6, float &out) const {
+        const float err = h * (m6 * m6 * 1.4210855e-14f);   // 4 u^2
+        out = h + (l - err);
+        return out == h + (l + err);
+    }
+};
+
 __device__ __forceinline__ int find_test(const int64_t *pre, int nt, int64_t g) {
     int lo = 0, hi = nt - 1;
     while (lo < hi) {

@@ -63,3 +63,41 @@ def test_certain_roots_are_rounded_right(tmp_path, n, pairs):
     # twice the bound over the spacing of the results (2^-23 to 2^-24 of them), and chance
     share = 2 * (21 * n + 32) * 2.0 ** -48 / 2.0 ** -24
     assert int(left) <= pairs * share + 5 * (pairs * share) ** 0.5 + 3
+
+
+# Squared norms of rows of p features by L lanes, 4 elements a lane and step: a sum that NormSum calls certain is
+# the correctly rounded one, and few are left open.  Last number: rows whose pair alone rounds the other way.
+NORMS = r"""
+int main(int argc, char **argv) {
+    const int p = atoi(argv[1]), L = atoi(argv[2]), rows = atoi(argv[3]);
+    std::mt19937_64 g(p + L);
+    std::normal_distribution<float> nd;
+    long open = 0, wrong = 0, plain = 0;
+    double worst = 0.0;
+    std::vector<float> z(p);
+    for (int q = 0; q < rows; ++q) {
+        long double S = 0;
+        for (float &v : z) { v = nd(g); S += (long double)v * v; }
+        std::vector<ept::NormSum> lane(L);
+        for (int k = 0; k < p; ++k) lane[(k / 4) % L].add(z[k]);
+        for (int off = L / 2; off; off /= 2)
+            for (int k = 0; k < off; ++k) lane[k].merge(lane[k + off].h, lane[k + off].l);
+        const float m6 = (float)(p / L + 10), want = (float)S;
+        worst = std::fmax(worst, (double)(fabsl((long double)lane[0].h + lane[0].l - S) / S) / std::ldexp(2.0 * m6 * m6, -48));
+        float y;
+        plain += lane[0].h + lane[0].l != want;
+        if (!lane[0].rounded(m6, y)) ++open;
+        else wrong += y != want;
+    }
+    printf("%ld %ld %.17g %ld\n", open, wrong, worst, plain);
+}
+"""
+
+
+@pytest.mark.parametrize("p,L,rows", [(1, 32, 40000), (5, 8, 40000), (100, 8, 40000), (512, 8, 20000), (1000, 32, 10000),
+                                      (9001, 32, 1000), (200000, 32, 40)])
+def test_certain_norms_are_rounded_right(tmp_path, p, L, rows):
+    left, wrong, worst, _ = _program(tmp_path, "norms", NORMS)(p, L, rows).split()
+    assert int(wrong) == 0 and float(worst) <= 1.0
+    share = min(1.0, 8 * (p // L + 10) ** 2 * 2.0 ** -48 / 2.0 ** -24)
+    assert int(left) <= rows * share + 5 * (rows * share) ** 0.5 + 3
