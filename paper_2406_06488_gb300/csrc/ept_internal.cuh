@@ -412,6 +412,23 @@ struct NormSum {
     }
 };
 
+// A sum as three FP32 numbers: the roundings of h's additions are summed in l, theirs in r.  Of m terms of
+// magnitudes A in all, value() is within m^3 2^-72 A + 2^-52 |sum| of the exact sum (|l| <= m u A, |r| <= m^2 u^2 A,
+// u = 2^-24); m = 64 at a time, that is less than FP64 additions one by one lose (m 2^-53 A), which take
+// sixteen cycles of the SM each.
+struct TripleSum {
+    float h = 0.f, l = 0.f, r = 0.f;
+    __host__ __device__ __forceinline__ void add(float v) {
+        float s, e, f;
+        two_sum(h, v, s, e);
+        h = s;
+        two_sum(l, e, s, f);
+        l = s;
+        r += f;
+    }
+    __host__ __device__ __forceinline__ double value() const { return (double)h + ((double)l + (double)r); }
+};
+
 __device__ __forceinline__ int find_test(const int64_t *pre, int nt, int64_t g) {
     int lo = 0, hi = nt - 1;
     while (lo < hi) {

@@ -49,10 +49,10 @@ __global__ void __launch_bounds__(256) k_stream_rowsums(const Batch bt, int64_t 
 }
 
 // sacc[b] += the window's partials of relabeling b (fixed order).  CTA = 32 columns, warp w
-// takes every 32nd partial row: eight at a time (their loads in flight together) as an
-// unevaluated FP32 pair (TwoSum), the pairs in FP64.  Bound by the loads; with an FP64 addition per
-// partial on eight warps this GPU's FP64 rate was the limit (n = 100,000, B = 4000, 1.3 GB of
-// partials in three windows: 2.87 ms, now 1.00).
+// takes every 32nd partial row: eight at a time (their loads in flight together), 64 to a
+// TripleSum, those in FP64.  With an FP64 addition per partial on eight
+// warps this GPU's FP64 rate was the limit (n = 100,000, B = 4000, 1.3 GB of partials in three windows:
+// 2.87 ms; eight to an FP32 pair 1.00; now 0.56).
 __global__ void __launch_bounds__(1024) k_stream_accum(const Batch bt) {
     constexpr int NW = 32;
     __shared__ double ws[NW][32];
@@ -61,19 +61,17 @@ __global__ void __launch_bounds__(1024) k_stream_accum(const Batch bt) {
     const int64_t c = (int64_t)blockIdx.x * 32 + lane, Bp = d.Bp;
     const float *part = bt.partial + d.part0 + c;
     double acc = 0.0;
-    for (int64_t k0 = warp; k0 < d.nparts; k0 += 8 * NW) {
-        float v[8];
+    for (int64_t k1 = warp; k1 < d.nparts; k1 += 64 * NW) {
+        const int64_t end = k1 + 64 * NW < d.nparts ? k1 + 64 * NW : d.nparts;
+        TripleSum sum;
+        for (int64_t k0 = k1; k0 < end; k0 += 8 * NW) {
+            float v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = k0 + k * NW < d.nparts ? part[(k0 + k * NW) * Bp] : 0.f;
-        float h = 0.f, l = 0.f;
+            for (int k = 0; k < 8; ++k) v[k] = k0 + k * NW < d.nparts ? part[(k0 + k * NW) * Bp] : 0.f;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            float s2, e;
-            two_sum(h, v[k], s2, e);
-            h = s2;
-            l += e;
+            for (int k = 0; k < 8; ++k) sum.add(v[k]);
         }
-        acc += (double)h + (double)l;
+        acc += sum.value();
     }
     ws[warp][lane] = acc;
     __syncthreads();

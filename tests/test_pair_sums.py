@@ -101,3 +101,40 @@ def test_certain_norms_are_rounded_right(tmp_path, p, L, rows):
     assert int(wrong) == 0 and float(worst) <= 1.0
     share = min(1.0, 8 * (p // L + 10) ** 2 * 2.0 ** -48 / 2.0 ** -24)
     assert int(left) <= rows * share + 5 * (rows * share) ** 0.5 + 3
+
+
+# Sums of m partials over 2^20 in magnitude, both signs, exact in integers: the error within the bound and, in
+# all, no larger than that of FP64 additions one by one.
+TRIPLES = r"""
+int main(int argc, char **argv) {
+    const int m = atoi(argv[1]), sums = atoi(argv[2]);
+    std::mt19937_64 g(m);
+    double worst = 0.0;
+    long double err3 = 0, err64 = 0;
+    for (int q = 0; q < sums; ++q) {
+        ept::TripleSum s;
+        double d = 0.0;
+        long long S = 0, A = 0;
+        for (int k = 0; k < m; ++k) {
+            const long long v = (long long)(g() % (1 << 24)) << (g() % 21);
+            const bool neg = g() & 1;
+            S += neg ? -v : v;
+            A += v;
+            s.add((float)(neg ? -v : v) * 0x1p-44f);
+            d += (double)(neg ? -v : v) * 0x1p-44;
+        }
+        const long double want = (long double)S * 0x1p-44L, e = fabsl((long double)s.value() - want);
+        err3 += e;
+        err64 += fabsl((long double)d - want);
+        const double bound = (double)m * m * m * 0x1p-72 * ((double)A * 0x1p-44) + 0x1p-52 * std::fabs((double)want);
+        worst = std::fmax(worst, bound > 0 ? (double)e / bound : (double)e);
+    }
+    printf("%.17g %.17g %.17g\n", worst, (double)err3, (double)err64);
+}
+"""
+
+
+@pytest.mark.parametrize("m", [1, 2, 7, 8, 9, 63, 64])
+def test_triple_sums_lose_no_more_than_fp64(tmp_path, m):
+    worst, err3, err64 = (float(x) for x in _program(tmp_path, "triples", TRIPLES)(m, 200000).split())
+    assert worst <= 1.0 and err3 <= err64
