@@ -1389,8 +1389,8 @@ void launch_contract_simt(const Batch &b, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // Final combination (Algorithm 1, statistic and p-value lines): per relabeling
 // column b, Q_b = sum of its partials, stat_b = sign * (cT Q_b + S~/o^2).  The partials are summed
-// as unevaluated FP32 pairs (TwoSum: each addition's rounding error is kept exactly) of a
-// few each, which then meet in FP64 in a fixed order: this GPU's FP64 pipe takes 16 cycles for a
+// in FP32 numbers that keep the roundings (pairs of a few partials, or a TripleSum of 64),
+// which then meet in FP64 in a fixed order: this GPU's FP64 pipe takes 16 cycles for a
 // warp's operation, so that with FP64 per partial, or per few of them, it is the limit.
 // Then k_combine_count compares against stat_0 (the identity, evaluated by the same
 // kernels): stat_b >= stat_0 and near-ties |stat_b - stat_0| <= 1e-5 |stat_0|.
@@ -1404,10 +1404,11 @@ __device__ __forceinline__ void finish_stat(const Batch &bt, int t, const TestDe
     if (bt.errest) bt.errest[d.col0 + c] = d.ka * REFINE_U * d.cT * (a * inv_c);
 }
 
-// Many columns (a batch): a thread per column (256 per CTA), eight partials at a time in one
-// pair (their loads in flight together), the pairs in FP64: three FP64 operations per eight
-// partials.  The kernel below makes 16 FP64 merges per column whatever its partials, 1.08 ms for 512
-// uneven tests (2.6 million columns, 50 partials on average, 0.5 GB); this one takes 0.29 ms.  It
+// Many columns (a batch): a thread per column (256 per CTA), eight partials at a time (their
+// loads in flight together), 64 to a TripleSum and as many magnitudes to another, those in FP64.
+// The kernel below makes 16 FP64 merges per column whatever its partials, 1.08 ms for 512
+// uneven tests (2.6 million columns, 50 partials on average, 0.5 GB); this one takes 0.31 ms (0.29 with
+// FP32 pairs of eight and the magnitudes in one FP32 sum, which is less than the other kernel keeps).  It
 // needs two CTAs per SM to pay (COMBINE_COLUMNS_PER_SM): with few columns a thread's chain of loads
 // is longer than the sixteen warps' (5000 columns of 50 partials: 8 us against 6).  Tests of more
 // partials than COMBINE_THREAD_PARTS keep the other.
@@ -1429,24 +1430,24 @@ __global__ void __launch_bounds__(256) k_combine_columns(const Batch bt) {
     if (c >= d.ncols) return;
     const int64_t Bp = d.Bp;
     const float *part = bt.partial + d.part0 + c;
-    double q = 0.0;
-    float aabs = 0.f;
-    for (int64_t k0 = 0; k0 < nparts; k0 += 8) {
-        float v[8];
+    double q = 0.0, a = 0.0;
+    for (int64_t k1 = 0; k1 < nparts; k1 += 64) {
+        const int64_t end = k1 + 64 < nparts ? k1 + 64 : nparts;
+        TripleSum sum, mag;
+        for (int64_t k0 = k1; k0 < end; k0 += 8) {
+            float v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = k0 + k < nparts ? part[(k0 + k) * Bp] : 0.f;
-        float h = 0.f, l = 0.f;
+            for (int k = 0; k < 8; ++k) v[k] = k0 + k < nparts ? part[(k0 + k) * Bp] : 0.f;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            float s2, e;
-            two_sum(h, v[k], s2, e);
-            h = s2;
-            l += e;
-            aabs += fabsf(v[k]);
+            for (int k = 0; k < 8; ++k) {
+                sum.add(v[k]);
+                mag.add(fabsf(v[k]));
+            }
         }
-        q += (double)h + (double)l;
+        q += sum.value();
+        a += mag.value();
     }
-    finish_stat(bt, t, d, c, q, (double)aabs, bSt);
+    finish_stat(bt, t, d, c, q, a, bSt);
 }
 
 // Tests of more partials: a CTA covers 32 columns of one test (the column padding is a multiple of

@@ -103,11 +103,12 @@ def test_certain_norms_are_rounded_right(tmp_path, p, L, rows):
     assert int(left) <= rows * share + 5 * (rows * share) ** 0.5 + 3
 
 
-# Sums of m partials over 2^20 in magnitude, both signs, exact in integers: the error within the bound and, in
+# Sums of m partials over 2^20 in magnitude, of both signs or their magnitudes, exact in integers: the error within the bound and, in
 # all, no larger than that of FP64 additions one by one.
 TRIPLES = r"""
 int main(int argc, char **argv) {
     const int m = atoi(argv[1]), sums = atoi(argv[2]);
+    const bool magnitudes = atoi(argv[3]);
     std::mt19937_64 g(m);
     double worst = 0.0;
     long double err3 = 0, err64 = 0;
@@ -117,7 +118,7 @@ int main(int argc, char **argv) {
         long long S = 0, A = 0;
         for (int k = 0; k < m; ++k) {
             const long long v = (long long)(g() % (1 << 24)) << (g() % 21);
-            const bool neg = g() & 1;
+            const bool neg = (g() & 1) && !magnitudes;
             S += neg ? -v : v;
             A += v;
             s.add((float)(neg ? -v : v) * 0x1p-44f);
@@ -136,5 +137,7 @@ int main(int argc, char **argv) {
 
 @pytest.mark.parametrize("m", [1, 2, 7, 8, 9, 63, 64])
 def test_triple_sums_lose_no_more_than_fp64(tmp_path, m):
-    worst, err3, err64 = (float(x) for x in _program(tmp_path, "triples", TRIPLES)(m, 200000).split())
-    assert worst <= 1.0 and err3 <= err64
+    run = _program(tmp_path, "triples", TRIPLES)
+    for magnitudes in (0, 1):
+        worst, err3, err64 = (float(x) for x in run(m, 200000, magnitudes).split())
+        assert worst <= 1.0 and err3 <= err64
