@@ -388,7 +388,7 @@ void plan_batch(Plan &P, const std::vector<TestSpec> &specs, int prec, bool host
     P.off_partial = take((size_t)P.npart * 4);
     P.off_errest = take((size_t)P.nstats * 8);
     P.off_flags = take((size_t)P.nstats);
-    P.off_sel_hist = P.any_median ? take((size_t)P.n_tests * 2048 * 4) : 0;
+    P.off_sel_hist = P.any_median ? take((size_t)P.n_tests * 2048 * 8) : 0;
     P.total = o;
 }
 
@@ -953,7 +953,7 @@ Batch device_view(ept_ctx *c, const Plan &P) {
     b.observed = (double *)(A + P.off_observed);
     b.maskT = (uint32_t *)(A + P.off_maskT);
     b.ctr = (Counters *)(A + P.off_ctr);
-    b.sel_hist = P.any_median ? (uint32_t *)(A + P.off_sel_hist) : nullptr;
+    b.sel_hist = P.any_median ? (unsigned long long *)(A + P.off_sel_hist) : nullptr;
     b.sacc = nullptr;
     b.inject_stall = c->inject_stall;
     b.wait_ns = c->wait_ns;
@@ -1039,7 +1039,7 @@ ept_status enqueue_device(ept_ctx *c, const Plan &P, cudaStream_t s, bool timed,
     b.build_sums = tc ? 1 : 0;
     if (timed) CK(cudaEventRecord(c->ev[0], s));
     if (with_inputs && (st = enqueue_uploads(c, P, s)) != EPT_OK) return st;
-    if (P.any_median) CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)P.n_tests * 2048 * 4, s));
+    if (P.any_median) CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)P.n_tests * 2048 * 8, s));
     if (P.debug) launch_guards(c->arena, P.guards, false, b.ctr, s);
     CK(cudaEventRecord(c->ev[1], s));
 
@@ -2886,7 +2886,7 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     }
     if (P.any_median) {
         // median bandwidth: select it, then the block-sum pass turns distances into kernel values
-        CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)2048 * 4, s));
+        CK(cudaMemsetAsync(b.sel_hist, 0, (size_t)2048 * 8, s));
         launch_median_select(b, c->num_sms, s);
         launch_blocksums(b, true, s);
     }

@@ -222,7 +222,7 @@ struct Batch {
     uint8_t *flags;                      // per relabeling column: 1 = recompute in FP64
     uint32_t *maskT;
     Counters *ctr;
-    uint32_t *sel_hist;                  // median heuristic: 2048 bins per test (null if no test needs it)
+    unsigned long long *sel_hist;        // median heuristic: 2048 bins per test (null if no test needs it)
     double *sacc;                        // streaming mode: FP64 sums of the windows' partials (Bp)
     int build_sums;                      // the tensor-core build also sums its blocks' rows and columns
     int inject_stall;                    // failure-path test hook (STALL_*): a warp of that kernel waits on a

@@ -790,8 +790,8 @@ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
 
 // The bin of h[0 .. MED_BINS) that holds rank k, and the number of entries in the bins before it
 // (bin -1: k is past the end); every thread of the CTA (T threads, a multiple of 32) gets both.
-template <int T>
-__device__ __forceinline__ int find_bin(const uint32_t *h, unsigned long long k, unsigned long long &before) {
+template <int T, typename Bin>
+__device__ __forceinline__ int find_bin(const Bin *h, unsigned long long k, unsigned long long &before) {
     constexpr int PER = MED_BINS / T;
     __shared__ unsigned long long wsum[T / 32];
     __shared__ int bin_s;
@@ -901,7 +901,10 @@ __global__ void __launch_bounds__(1024) k_median_sample(const Batch bt) {
 // One pass over the stored entries: a CTA takes a run of consecutive blocks, and hands its
 // histogram over where the test changes and at the end.
 __global__ void __launch_bounds__(256) k_median_pass(const Batch bt) {
-    __shared__ uint32_t hist[MED_BINS];
+    // a CTA's counts in 32 bits (it reads fewer entries than that), a test's in 64: above n = 92,682 there are more
+    // than 2^32 pairs, and equal distances share a bin
+    __shared__ unsigned long long bins_s[MED_BINS];
+    uint32_t *hist = reinterpret_cast<uint32_t *>(bins_s);
     __shared__ bool last_s;
     const int64_t b0 = bt.nblk_total * (int64_t)blockIdx.x / gridDim.x;
     const int64_t b1 = bt.nblk_total * (int64_t)(blockIdx.x + 1) / gridDim.x;
@@ -948,9 +951,9 @@ __global__ void __launch_bounds__(256) k_median_pass(const Batch bt) {
             }
         }
         __syncthreads();
-        uint32_t *gh = bt.sel_hist + (int64_t)t * MED_BINS;
+        unsigned long long *gh = bt.sel_hist + (int64_t)t * MED_BINS;
         for (int k = threadIdx.x; k < MED_BINS; k += 256)
-            if (hist[k]) atomicAdd(&gh[k], hist[k]);
+            if (hist[k]) atomicAdd(&gh[k], (unsigned long long)hist[k]);
         for (int off = 16; off; off >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, off);
         if ((threadIdx.x & 31) == 0 && below) atomicAdd(&c->sel_below, (unsigned long long)below);
         __threadfence();
@@ -961,14 +964,14 @@ __global__ void __launch_bounds__(256) k_median_pass(const Batch bt) {
         // the test's last CTA: the bin of rank k
         __threadfence();
         for (int k = threadIdx.x; k < MED_BINS; k += 256) {
-            hist[k] = __ldcg(&gh[k]);
-            gh[k] = 0u;   // ready for the next pass
+            bins_s[k] = __ldcg(&gh[k]);
+            gh[k] = 0ull;   // ready for the next pass
         }
         __syncthreads();
         const bool first = c->sel_state == MED_SAMPLED;
         const unsigned long long under = first ? __ldcg(&c->sel_below) : 0ull, k = c->sel_k;
         unsigned long long before = 0;
-        const int bin = k >= under ? find_bin<256>(hist, k - under, before) : -1;   // uniform
+        const int bin = k >= under ? find_bin<256>(bins_s, k - under, before) : -1;   // uniform
         __syncthreads();
         if (threadIdx.x == 0) {
             c->sel_blocks = 0u;
