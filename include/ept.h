@@ -408,7 +408,10 @@ ept_status ept_set_option(ept_ctx *ctx, int option, int64_t value);
    started beside them (continuous batching).  Errors: EPT_ENOMEM if the request
    can never fit the budget, EPT_EBUSY if the queue is full.  Results equal
    ept_test's on the same inputs within rounding.  A request whose data is
-   rejected on the device (NaN/Inf) fails alone; the rest of its batch is kept. */
+   rejected on the device (NaN/Inf) fails alone; the rest of its batch is kept.
+   The host memory that held a finished request's samples is kept for later ones, as it
+   was left: at most 256 MB, the oldest first to go, all of it freed two seconds after
+   the last ept_submit or ept_wait, or with the context. */
 ept_status ept_submit(ept_ctx *ctx, const ept_test_desc *request, int prec, uint64_t *ticket);
 
 /* *done = 1 when the request has finished (or was cancelled), else 0. */

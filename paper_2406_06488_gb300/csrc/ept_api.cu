@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "../../include/ept.h"
+#include "ept_host.h"
 #include "ept_internal.cuh"
 
 using namespace ept;
@@ -521,99 +522,6 @@ struct GraphCache {
 
 namespace {
 struct Server;
-
-// Host memory copies spread over a small pool of worker threads (the caller works
-// too), used to gather pageable inputs into the pinned staging area at several times
-// the bandwidth of one core.  run() returns when every byte is copied.
-class HostCopier {
-public:
-    struct Job {
-        void *dst;
-        const void *src;
-        size_t bytes;
-    };
-    // a copier of up to 8 workers, half the machine's cores; null where no thread can be started
-    static std::unique_ptr<HostCopier> create() {
-        const unsigned hw = std::thread::hardware_concurrency();
-        std::unique_ptr<HostCopier> c(new (std::nothrow) HostCopier());
-        if (!c) return c;
-        try {
-            for (unsigned k = std::max(1u, std::min(8u, hw / 2)); k > 0; --k)
-                c->th_.emplace_back([p = c.get()] { p->worker(); });
-        } catch (const std::exception &) {   // fewer workers, or none
-            if (c->th_.empty()) c.reset();
-        }
-        return c;
-    }
-    ~HostCopier() {
-        {
-            std::lock_guard<std::mutex> lk(mu_);
-            stop_ = true;
-        }
-        cv_.notify_all();
-        for (std::thread &t : th_) t.join();
-    }
-    void run(const std::vector<Job> &jobs) {
-        size_t total = 0;
-        for (const Job &j : jobs) total += j.bytes;
-        const size_t PIECE = total >= ((size_t)32 << 20) ? (size_t)1 << 20 : (size_t)1 << 18;
-        {
-            std::unique_lock<std::mutex> lk(mu_);
-            cv_done_.wait(lk, [this] { return active_ == 0; });   // a late worker of the last run has left
-            pieces_.clear();
-            for (const Job &j : jobs)
-                for (size_t o = 0; o < j.bytes; o += PIECE)
-                    pieces_.push_back({(uint8_t *)j.dst + o, (const uint8_t *)j.src + o, std::min(PIECE, j.bytes - o)});
-            next_.store(0);
-            remaining_.store(pieces_.size());
-            ++gen_;
-        }
-        cv_.notify_all();
-        work();
-        std::unique_lock<std::mutex> lk(mu_);
-        cv_done_.wait(lk, [this] { return remaining_.load() == 0 && active_ == 0; });
-    }
-
-private:
-    void work() {
-        const size_t n = pieces_.size();
-        for (;;) {
-            const size_t k = next_.fetch_add(1);
-            if (k >= n) break;
-            memcpy(pieces_[k].dst, pieces_[k].src, pieces_[k].bytes);
-            if (remaining_.fetch_sub(1) == 1) {
-                std::lock_guard<std::mutex> lk(mu_);
-                cv_done_.notify_all();
-            }
-        }
-    }
-    void worker() {
-        uint64_t seen = 0;
-        for (;;) {
-            {
-                std::unique_lock<std::mutex> lk(mu_);
-                cv_.wait(lk, [&] { return stop_ || gen_ != seen; });
-                if (stop_) return;
-                seen = gen_;
-                ++active_;
-            }
-            work();
-            {
-                std::lock_guard<std::mutex> lk(mu_);
-                --active_;
-            }
-            cv_done_.notify_all();
-        }
-    }
-    std::vector<std::thread> th_;
-    std::mutex mu_;
-    std::condition_variable cv_, cv_done_;
-    std::vector<Job> pieces_;
-    std::atomic<size_t> next_{0}, remaining_{0};
-    int active_ = 0;
-    uint64_t gen_ = 0;
-    bool stop_ = false;
-};
 }  // namespace
 
 struct ept_ctx {
@@ -874,7 +782,7 @@ void stage_host(ept_ctx *c, Plan &P, const std::vector<TestSpec> &specs, bool on
         if (!c->copier) c->copier = HostCopier::create();
     }
     if (gather_bytes >= ((size_t)4 << 20) && c->copier) {
-        c->copier->run(gather);
+        c->copier->run(gather.data(), gather.size());
     } else {
         for (const HostCopier::Job &j : gather) memcpy(j.dst, j.src, j.bytes);
     }
@@ -2168,11 +2076,6 @@ enum ReqState { REQ_PENDING = 0, REQ_RUNNING = 1, REQ_DONE = 2, REQ_CANCELLED = 
 
 using Clock = std::chrono::steady_clock;
 
-struct HostBuffer {
-    std::unique_ptr<float[]> data;
-    size_t cap = 0;   // floats
-};
-
 struct Request {
     uint64_t ticket = 0;
     TestSpec spec;
@@ -2217,66 +2120,9 @@ struct Server {
     size_t max_pending = 1 << 16;
     int64_t peak_busy = 0;         // the most lanes that held a running batch at the same time
     int64_t submits_busy = 0;      // requests submitted while some lane held a running batch
-    // Sample memory of finished requests, for the next ones (guarded by mu; at most SPARE_BYTES, freed with the
-    // server).  Copying the samples is most of a burst's time, and into fresh memory half of the copy is
-    // page faults: 88 MB take one core 9 ms, into used memory 5, and with the workers below 1.3.
-    std::vector<HostBuffer> spare;
-    size_t spare_bytes = 0;
-    // Worker threads for the samples' copies; a submitter that finds them taken copies by itself.
-    std::mutex copy_mu;
-    std::unique_ptr<HostCopier> copier;
+    HostPool samples;              // sample memory of finished requests, for the next ones
+    SharedCopier<std::mutex> copier;
 };
-
-constexpr size_t SPARE_BYTES = (size_t)256 << 20;
-constexpr size_t SPARE_MIN = (size_t)128 << 10;     // smaller buffers are the heap's own business
-constexpr size_t PARALLEL_COPY = (size_t)1 << 20;   // below, waking the workers costs what they would save
-
-// Memory for `floats` values: a spare buffer of up to twice that, else a new one (data == nullptr: none to be had).
-HostBuffer take_buffer(Server *S, size_t floats) {
-    {
-        std::lock_guard<std::mutex> lk(S->mu);
-        size_t best = S->spare.size();
-        for (size_t k = 0; k < S->spare.size(); ++k) {
-            const size_t cap = S->spare[k].cap;
-            if (cap >= floats && cap / 2 <= floats && (best == S->spare.size() || cap < S->spare[best].cap)) best = k;
-        }
-        if (best < S->spare.size()) {
-            HostBuffer b = std::move(S->spare[best]);
-            S->spare[best] = std::move(S->spare.back());
-            S->spare.pop_back();
-            S->spare_bytes -= b.cap * sizeof(float);
-            return b;
-        }
-    }
-    HostBuffer b;
-    b.data.reset(new (std::nothrow) float[floats]);
-    b.cap = b.data ? floats : 0;
-    return b;
-}
-
-// Keeps a finished request's memory (lock held); what does not fit is freed by the caller, without the lock.
-void give_buffer(Server *S, HostBuffer &b) {
-    const size_t bytes = b.cap * sizeof(float);
-    if (bytes < SPARE_MIN || S->spare_bytes + bytes > SPARE_BYTES) return;
-    S->spare_bytes += bytes;
-    S->spare.push_back(std::move(b));
-    b.cap = 0;
-}
-
-void copy_samples(Server *S, const std::vector<HostCopier::Job> &jobs) {
-    size_t bytes = 0;
-    for (const HostCopier::Job &j : jobs) bytes += j.bytes;
-    std::unique_lock<std::mutex> lk(S->copy_mu, std::try_to_lock);
-    if (bytes >= PARALLEL_COPY && lk.owns_lock()) {
-        if (!S->copier) S->copier = HostCopier::create();
-        if (S->copier) {
-            S->copier->run(jobs);
-            return;
-        }
-    }
-    if (lk.owns_lock()) lk.unlock();
-    for (const HostCopier::Job &j : jobs) memcpy(j.dst, j.src, j.bytes);
-}
 
 void CUDART_CB lane_finished(void *arg) {
     Server *S = (Server *)arg;
@@ -2464,6 +2310,11 @@ void serve_loop(Server *S, int device) {
                 if (st != EPT_OK) finish_requests(S, L, st, msg, nullptr, nullptr);
                 progressed = true;
             }
+        }
+        if (!progressed && S->samples.idle(HostPool::Clock::now())) {
+            lk.unlock();
+            S->samples.release();
+            lk.lock();
         }
         if (!progressed)
             S->cv_work.wait_for(lk, std::chrono::milliseconds(any_busy ? 1 : 50),
@@ -2993,13 +2844,14 @@ ept_status ept_submit(ept_ctx *c, const ept_test_desc *q, int prec, uint64_t *ti
     Request *r = new (std::nothrow) Request();
     if (!r) return fail(EPT_ENOMEM, "host allocation failed");
     const size_t fx = (size_t)q->nx * q->p, fy = (size_t)q->ny * q->p;
-    r->samples = take_buffer(S, fx + fy);
+    r->samples = S->samples.take(fx + fy);
     if (!r->samples.data) {
         delete r;
         return fail(EPT_ENOMEM, "host allocation failed");
     }
     float *const X = r->samples.data.get(), *const Y = X + fx;
-    copy_samples(S, {{X, q->X, fx * sizeof(float)}, {Y, q->Y, fy * sizeof(float)}});
+    const HostCopier::Job jobs[2] = {{X, q->X, fx * sizeof(float)}, {Y, q->Y, fy * sizeof(float)}};
+    S->copier.copy(jobs, 2);
     r->stats.assign((size_t)q->B, 0.0);
     r->spec = one_test(X, q->nx, Y, q->ny, q->p, q->stat, q->sigma, q->B, q->seed, nullptr,
                        q->B > 0 ? r->stats.data() : nullptr)[0];
@@ -3064,8 +2916,8 @@ ept_status ept_wait(ept_ctx *c, uint64_t ticket, double *perm_stats, ept_result 
         if (out) *out = r->res;
         if (perm_stats && !r->stats.empty()) memcpy(perm_stats, r->stats.data(), r->stats.size() * 8);
     }
-    give_buffer(S, r->samples);
     lk.unlock();
+    S->samples.give(std::move(r->samples));
     delete r;
     if (state == REQ_CANCELLED) return fail(EPT_ECANCELLED, "request %llu was cancelled", (unsigned long long)ticket);
     if (st != EPT_OK) return fail(st, "%s", msg.c_str());
