@@ -111,7 +111,8 @@ private:
 };
 
 // A HostCopier that several threads share: one at a time has the workers, and a thread that finds them taken
-// copies by itself.
+// copies by itself.  A copy too small for the workers does not ask for them, not even for a moment: a large copy
+// that came just then would go to one core.
 template <class Mutex>
 class SharedCopier {
 public:
@@ -119,14 +120,14 @@ public:
     void copy(const HostCopier::Job *jobs, size_t njobs) {
         size_t bytes = 0;
         for (size_t k = 0; k < njobs; ++k) bytes += jobs[k].bytes;
-        if (copy_by_workers(jobs, njobs, bytes)) return;
+        if (bytes >= PARALLEL && copy_by_workers(jobs, njobs)) return;
         for (size_t k = 0; k < njobs; ++k) memcpy(jobs[k].dst, jobs[k].src, jobs[k].bytes);
     }
 
 private:
-    bool copy_by_workers(const HostCopier::Job *jobs, size_t njobs, size_t bytes) {
+    bool copy_by_workers(const HostCopier::Job *jobs, size_t njobs) {
         std::unique_lock<Mutex> lk(mu_, std::try_to_lock);
-        if (bytes < PARALLEL || !lk.owns_lock()) return false;
+        if (!lk.owns_lock()) return false;
         if (!copier_) copier_ = HostCopier::create();
         if (!copier_) return false;
         try {

@@ -75,3 +75,34 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_small_copies_leave_the_workers_alone(tmp_path):
+    _run(tmp_path, r"""
+struct CountedMutex {   // how often it is asked for; refused while `taken`
+    static int asked;
+    static bool taken;
+    void lock() {}
+    void unlock() {}
+    bool try_lock() { ++asked; return !taken; }
+};
+int CountedMutex::asked = 0;
+bool CountedMutex::taken = false;
+int main() {
+    using Copier = SharedCopier<CountedMutex>;
+    Copier copier;
+    for (size_t bytes : {(size_t)0, (size_t)1, (size_t)4097, Copier::PARALLEL - 2, Copier::PARALLEL, (size_t)50000001})
+        for (bool taken : {false, true}) {
+            std::vector<uint8_t> x(bytes), y(bytes + 1);
+            for (size_t k = 0; k < bytes; ++k) x[k] = (uint8_t)(k * 131 + (k >> 9) + 1);
+            const size_t h = bytes / 3;   // two jobs
+            const HostCopier::Job jobs[2] = {{y.data(), x.data(), h}, {y.data() + h, x.data() + h, bytes - h}};
+            CountedMutex::taken = taken;
+            CountedMutex::asked = 0;
+            copier.copy(jobs, 2);
+            CHECK(CountedMutex::asked == (bytes >= Copier::PARALLEL ? 1 : 0));
+            CHECK(std::equal(x.begin(), x.end(), y.begin()) && y[bytes] == 0);
+        }
+    return 0;
+}
+""")
