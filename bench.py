@@ -34,10 +34,7 @@ if ROOT not in sys.path:
 
 METRIC = "permuted stats/s & p99 test latency, tuned vs plain FP32 GPU at rel err ≤1e-5"
 UNIT = "permuted stats/s"
-KERNELS_PER_STEP = 10  # libept kernels launched by one ept_test run (split path, a given bandwidth; two
-                       # fewer up to 1,024 rows), before any recomputation
-BATCH_KERNELS_PER_STEP = 11  # ept_test_batch: the same and the batch's error status
-# (the recomputation of flagged statistics adds Result.refine_launches launches to a step)
+COUNTERS_BYTES = 128   # a test's counters in the result copy (struct Counters)
 # dram read + write bytes of one k_contract_tc launch on the highdim and mmd workloads, from the
 # ncu captures summarised in profiles/k_contract_tc_highdim_ed.md and k_contract_tc_mmd.md (to be
 # reset to {} whenever the kernel changes, until it is captured again)
@@ -45,6 +42,26 @@ CONTRACT_TRAFFIC = {"highdim": 60.79e6, "mmd": 1088.0e6}
 # streaming mode: DRAM bytes per stored block of the contraction, from the n = 60,000 capture summarised in
 # profiles/k_contract_tc_stream_60k.md (scaled to a launch by its window's blocks)
 STREAM_TRAFFIC_PER_BLOCK = 9168.4e6 / 110920
+
+
+def _kernels(specs, windows=0):
+    """libept kernels that one run of these tests launches (split precision), before any recomputation of flagged
+    statistics (Result.refine_launches)."""
+    if windows:   # streaming mode: build and row sums of each window, then its build, packing, contraction, sums
+        return 7 + 6 * windows
+    k = 10                                                # draws, split, build, row sums, centring (2), packing,
+    if max(s.nx + s.ny for s in specs) <= 1024:           #   contraction, combination, counting
+        k -= 2                                            # row sums and centring in one
+    if any(s.stat != "ed" and s.sigma < 0 for s in specs):
+        k += 6                                            # median bandwidth: sample, four passes, block sums
+    return k + (1 if len(specs) > 1 else 0)               # a batch's error status
+
+
+def _result_bytes(specs):
+    """Bytes of the copy that brings a run's counters, observed statistics and statistics to the host: each of the
+    first two rounded up to 256."""
+    up = lambda b: (b + 255) // 256 * 256   # noqa: E731
+    return up(COUNTERS_BYTES * len(specs)) + up(8 * len(specs)) + 8 * sum(s.B + 1 for s in specs)
 
 
 def _args():
@@ -455,8 +472,8 @@ def run_ours(args):
                      "mma_flops_per_launch": mma_flops,
                      "mma_frac": mma_flops / t_contract / 1e12 / peak},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int((spec.nx + spec.ny) * spec.p * 4),
-                "d2h_bytes_per_step": int((spec.B + 1) * 8 + 48), "steps": args.e2e_steps},
-        "gpu_launches": (KERNELS_PER_STEP - (2 if spec.nx + spec.ny <= 1024 else 0) + last.refine_launches) * args.steps,
+                "d2h_bytes_per_step": _result_bytes([spec]), "steps": args.e2e_steps},
+        "gpu_launches": (_kernels([spec]) + last.refine_launches) * args.steps,
         "clocks": clocks,
         "result": {"observed": last.observed, "p_value": last.p_value, "n_near_tie": last.n_near_tie,
                    "sigma": last.sigma, "n_refined": last.n_refined},
@@ -719,8 +736,8 @@ def run_batched(args):
                      "frac": achieved / peak, "traffic": None, "kernel": "k_contract_tc",
                      "peak_kind": "%s bf16 dense burst" % peak_kind, "algorithmic_flops_per_launch": alg_flops},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(in_bytes),
-                "d2h_bytes_per_step": int(sum((sp.B + 1) * 8 + 48 for sp in specs)), "steps": args.e2e_steps},
-        "gpu_launches": (BATCH_KERNELS_PER_STEP + last[0].refine_launches) * args.steps,
+                "d2h_bytes_per_step": _result_bytes(specs), "steps": args.e2e_steps},
+        "gpu_launches": (_kernels(specs) + last[0].refine_launches) * args.steps,
         "clocks": clocks,
     }
     if cpu is not None:
@@ -987,8 +1004,8 @@ def run_stream(args):
                      "peak_kind": "%s bf16 dense sustained (seconds-long step)" % peak_kind,
                      "algorithmic_flops_per_test": alg_flops, "launches_per_test": nwin},
         "e2e": {"value": spec.B * ws / e2e_s, "unit": UNIT, "h2d_bytes_per_step": int(n * spec.p * 4),
-                "d2h_bytes_per_step": int((spec.B + 1) * 8 + 48), "steps": 1},
-        "gpu_launches": (7 + 7 * nwin) * steps,
+                "d2h_bytes_per_step": _result_bytes([spec]), "steps": 1},
+        "gpu_launches": _kernels([spec], windows=nwin) * steps,
         "clocks": clocks,
         "result": {"observed": last.observed, "p_value": last.p_value, "n_near_tie": last.n_near_tie,
                    "n_windows": nwin},
