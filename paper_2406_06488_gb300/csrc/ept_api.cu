@@ -2717,8 +2717,8 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     c->urec_serial = c->tab_serial = 0;   // and the arena its data, over a cached plan's tables and records
     stage_host(c, P, specs, on_device != 0);
     uint8_t *A = c->arena;
-    Batch b = device_view(c, P);
-    b.inject_stall = 0;   // the hook is for runs
+    const Batch b = device_view(c, P);
+    if (prec == EPT_PREC_SPLIT_BF16 && c->inject_stall == STALL_BUILD) c->inject_stall = 0;   // the hook is one-shot
     if ((st = upload_tables(c, P, s)) != EPT_OK) return st;
     if ((st = enqueue_inputs(c, s)) != EPT_OK) return st;
     CK(cudaStreamWaitEvent(s, c->ev_in, 0));
@@ -2748,6 +2748,8 @@ ept_status ept_build_blocks(ept_ctx *c, const float *X, int64_t nx, const float 
     CK(cudaMemcpyAsync(h, b.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
     if (!on_device) CK(cudaMemcpyAsync(D_out, dout, out_bytes, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    if (h->err_code)
+        return fail(EPT_ETIMEOUT, "device-side bounded wait gave up (code 0x%llx)", (unsigned long long)h->err_code);
     if (h->nonfinite) return fail(EPT_EINVAL, "X or Y holds NaN or Inf");
     return EPT_OK;
 }

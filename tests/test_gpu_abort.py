@@ -88,3 +88,10 @@ def test_contraction_gives_up(ctx, kernel, nx, ny, B):
             assert got.observed == want.observed and np.array_equal(got.stats, want.stats)
     finally:
         ctx.set_option("contraction", 0)
+
+
+def test_build_blocks_reports_an_expired_wait(ctx):
+    X, Y = _pair(700, 900, 5, seed=9)
+    want = ctx.build_blocks(X, Y)
+    _expires(ctx, lambda: ctx.build_blocks(X, Y))
+    assert np.array_equal(ctx.build_blocks(X, Y), want)
