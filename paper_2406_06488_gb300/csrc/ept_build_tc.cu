@@ -616,7 +616,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             // the blocks' row and column sums and largest entry (a median test's come from its
             // kernel values, in k_blocksums)
             const bool sums = bt.build_sums && !d.median;
-            f32x2 rh = 0, rl = 0;   // the row's even and odd columns of a K-block
+            float rowh = 0.f, rowl = 0.f;   // the row's sum over a K-block's first group
             float mx = 0.f;
             if (sums) half_sync(half, 0);
             unsigned fixups = 0;
@@ -696,16 +696,21 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     }
                 }
                 if (sums) {
+                    f32x2 rh = 0, rl = 0;   // even and odd columns, sixteen each, as k_blocksums' chains
 #pragma unroll
                     for (int e = 0; e < 32; e += 2) {
                         pair_add2(rh, rl, pack2(out[e], out[e + 1]));
                         mx = fmaxf(mx, fmaxf(out[e], out[e + 1]));
                     }
+                    float h, l;
+                    pair_join(rh, rl, h, l);
                     if (gl & 1) {   // a K-block is complete
-                        float h, l;
-                        pair_join(rh, rl, h, l);
-                        bt.rowpart[drow + lane + (int64_t)(g >> 1) * PANEL] = (double)h + (double)l;
-                        rh = rl = 0;
+                        float s, e;
+                        two_sum(rowh, h, s, e);
+                        bt.rowpart[drow + lane + (int64_t)(g >> 1) * PANEL] = (double)s + (double)((rowl + l) + e);
+                    } else {
+                        rowh = h;
+                        rowl = l;
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
