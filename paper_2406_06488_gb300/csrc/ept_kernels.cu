@@ -772,7 +772,7 @@ void launch_blocksums(const Batch &b, bool median_only, cudaStream_t s) {
 // passes are launched, those left return at once.
 // A pass reads every stored entry once (n = 10,500: 224 MB) and adds to shared memory for one
 // entry in twenty; histograms of the leading digits of every entry took 167 us a pass,
-// three times, since distances share a few leading digits; now 28 us for the sample, 84 and 73 us for the
+// three times, since distances share a few leading digits; now 27 us for the sample, 83 and 75 us for the
 // passes that do the work and 7 us for the two that return.
 constexpr int MED_SAMPLES = 16384, MED_BINS = 2048, MED_PASSES = 4;
 
@@ -780,6 +780,7 @@ constexpr int MED_SAMPLES = 16384, MED_BINS = 2048, MED_PASSES = 4;
 // the entries from `lo` on (first pass: from 0 on)
 enum { MED_SAMPLED = 1, MED_INSIDE = 2, MED_DONE = 3 };
 
+// the 32-bit finaliser of MurmurHash3 (Appleby, public domain)
 __device__ __forceinline__ uint32_t mix32(uint32_t x) {
     x ^= x >> 16;
     x *= 0x85EBCA6Bu;
@@ -902,7 +903,8 @@ __global__ void __launch_bounds__(1024) k_median_sample(const Batch bt) {
 // histogram over where the test changes and at the end.
 __global__ void __launch_bounds__(256) k_median_pass(const Batch bt) {
     // a CTA's counts in 32 bits (it reads fewer entries than that), a test's in 64: above n = 92,682 there are more
-    // than 2^32 pairs, and equal distances share a bin
+    // than 2^32 pairs, and equal distances share a bin (smaller tests look their bin up in 32 bits: 0.5 us a
+    // pass of a few rows)
     __shared__ unsigned long long bins_s[MED_BINS];
     uint32_t *hist = reinterpret_cast<uint32_t *>(bins_s);
     __shared__ bool last_s;
@@ -963,15 +965,20 @@ __global__ void __launch_bounds__(256) k_median_pass(const Batch bt) {
         if (!last_s) continue;
         // the test's last CTA: the bin of rank k
         __threadfence();
+        const bool wide = (unsigned long long)n * (unsigned long long)(n - 1) / 2ull >> 32 != 0ull;
         for (int k = threadIdx.x; k < MED_BINS; k += 256) {
-            bins_s[k] = __ldcg(&gh[k]);
+            const unsigned long long v = __ldcg(&gh[k]);
+            if (wide) bins_s[k] = v;
+            else hist[k] = (uint32_t)v;
             gh[k] = 0ull;   // ready for the next pass
         }
         __syncthreads();
         const bool first = c->sel_state == MED_SAMPLED;
         const unsigned long long under = first ? __ldcg(&c->sel_below) : 0ull, k = c->sel_k;
         unsigned long long before = 0;
-        const int bin = k >= under ? find_bin<256>(bins_s, k - under, before) : -1;   // uniform
+        const int bin = k < under ? -1   // uniform
+                        : wide    ? find_bin<256>(bins_s, k - under, before)
+                                  : find_bin<256>(hist, k - under, before);
         __syncthreads();
         if (threadIdx.x == 0) {
             c->sel_blocks = 0u;
