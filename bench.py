@@ -38,10 +38,10 @@ COUNTERS_BYTES = 128   # a test's counters in the result copy (struct Counters)
 # dram read + write bytes of one k_contract_tc launch on the highdim and mmd workloads, from the
 # ncu captures summarised in profiles/k_contract_tc_highdim_ed.md and k_contract_tc_mmd.md (to be
 # reset to {} whenever the kernel changes, until it is captured again)
-CONTRACT_TRAFFIC = {"highdim": 60.79e6, "mmd": 1088.0e6}
+CONTRACT_TRAFFIC = {"highdim": 60.74e6, "mmd": 1087.6e6}
 # streaming mode: DRAM bytes per stored block of the contraction, from the n = 60,000 capture summarised in
 # profiles/k_contract_tc_stream_60k.md (scaled to a launch by its window's blocks)
-STREAM_TRAFFIC_PER_BLOCK = 9168.4e6 / 110920
+STREAM_TRAFFIC_PER_BLOCK = 9172.6e6 / 110920
 
 
 def _kernels(specs, windows=0):

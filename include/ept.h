@@ -96,7 +96,7 @@ typedef struct {
     double p_value;       /* (1 + n_ge) / (1 + B); 1 when B = 0 */
     int64_t n_ge;         /* #{b : stat*_b >= observed}, compared in FP64 */
     int64_t n_near_tie;   /* #{b : |stat*_b - observed| <= 1e-5 * |observed|} */
-    int64_t n_fixup;      /* near-duplicate pairs whose distance was recomputed in FP64 */
+    int64_t n_fixup;      /* near-duplicate pairs recomputed from direct differences, rounded as in FP64 */
     double ms_build;      /* device time of the block phase (norms .. packing) */
     double ms_perm;       /* device time of relabeling draws + contraction + combine */
     double ms_total;      /* device time of the whole call, copies included */
@@ -369,9 +369,9 @@ ept_status ept_test_batch(ept_ctx *ctx, const ept_test_desc *tests, int64_t n_te
    tensor-memory operand (M = 128 relabelings stored from registers with tcgen05.st,
    N = 128 rows of C from shared memory; each epilogue thread sums its own
    relabeling's row values, no transposes).  0: the library's choice (1).  Measured
-   on a GB300 (n = 5000, B = 10^4 contraction): 1 256 us, 2 311 us, 3 451 us (the
-   MMA pipe alone, with N = 128, needs 366 us for the work that N = 256 does in 254
-   us).  The statistics agree to the accumulation order.
+   on a GB300 (n = 5000, B = 10^4 contraction): 1 256 us, 2 311 us, 3 451 us (its
+   MMAs alone, with N = 128, need 366 us; 1 without its epilogue and producers takes
+   246).  The statistics agree to the accumulation order.
    EPT_OPT_SERVE_LANES (default 3, 1..16): serving batches in flight at once;
    EPT_OPT_SERVE_SLOTS (default 256): serving requests in flight at once; both
    before the first ept_submit.  EPT_EINVAL for an unknown option or value.

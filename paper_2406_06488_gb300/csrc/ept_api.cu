@@ -53,7 +53,7 @@ ept_status fail(ept_status st, const char *fmt, ...) {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// pairs with d^2 < tau (||x||^2 + ||y||^2) are recomputed directly in FP64: the norm
+// pairs with d^2 < tau (||x||^2 + ||y||^2) are recomputed from direct differences: the norm
 // expansion amplifies rounding by at most 1/tau on the pairs it keeps
 const double NEAR_DUP_TAU = 1.0 / 4.0;
 // relabeling masks above this size (a quarter of the L2) change the contraction's unit order

@@ -28,9 +28,9 @@
 // accumulators of 128 columns let the epilogue of one sub-unit overlap the main
 // loop of the next; the relabeling stages take another 32 columns each).
 //
-// Measured on a GB300 (n = 5000, B = 10^4): 452 us against 258 us for
+// Measured on a GB300 (n = 5000, B = 10^4): 452 us against 256 us for
 // ept_contract_tc.cu.  The MMAs alone (no copies, producers or epilogue) take 366 us
-// here against 254 us there for the same multiply-adds: an MMA with N = 128 does
+// here; that kernel without its epilogue and producers takes 246: an MMA with N = 128 does
 // less work per cycle than one with N = 256 (with the C half-block as the
 // shared-memory A operand and N = 128 relabelings, 410 us), and N = 256 rows of C
 // would need 2 x 256 accumulator columns beside the relabeling stages, more than the
